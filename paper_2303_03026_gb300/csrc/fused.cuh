@@ -44,6 +44,19 @@ constexpr int FB = 16;          // block edge handled by the fused kernel
 // (the 32 faces on the +x/+y block boundary).  The 2D kernel uses the same
 // roles with threads 0 .. 64G-1 copying and converting the halo.
 constexpr int FT = FB * FB + FB;
+// Double with a two-ghost-cell limiter: every cell's limited slopes are
+// evaluated once (its two face states handed to the neighbouring face through
+// the face-flux array) instead of once per face, since the FP64 pipe bounds
+// these kernels; the helpers are then a whole warp: lane r < 16 the x faces of
+// row r, lane 16 + r the y faces of column r, one flux evaluation for both.
+// With the refined approximations of fp64.cuh for division and square root: a
+// step of the 3D AMR blast in double (6.0 M cells) 85.6 -> 42.0 ms, of the 1024^2
+// vortex with koren 10.3 -> 5.3 ms.  float keeps one slope per face: there the
+// exchange costs more issue slots than the slopes it saves.
+template <class T, int LIM> constexpr bool share_slopes() { return sizeof(T) == 8 && LIM != -2; }
+template <class T, int LIM> constexpr int fused_threads() {
+  return share_slopes<T, LIM>() ? FB * FB + 2 * FB : FT;
+}
 constexpr int FXW = 20;           // row stride of the face-flux arrays
 
 // ghost layers of a tile for a limiter template value (-2: the five-point
@@ -167,15 +180,16 @@ __device__ __forceinline__ void cfl_terms(const T* u, double gammad, T g, bool f
                                           const T* idx, T& smx, T& cmx) {
   T w[NV];
   cons2prim(gammad, u, w, ff, gm1f);
-  const T ir = T(1) / w[0];
+  const T ir = rcp_T(w[0]);
   const T a2 = g * w[4] * ir;
   const T bb = (w[5] * w[5] + w[6] * w[6] + w[7] * w[7]) * ir;
   const T dd = a2 - bb, sab = a2 + bb;
   T s = T(0);
 #pragma unroll
   for (int d = 0; d < DIM; d++) {
-    const T bt2 = fmax(bb - w[5 + d] * w[5 + d] * ir, T(0));  // no negative rounding
-    const T cf = sqrt(T(0.5) * (sab + sqrt(dd * dd + T(4) * a2 * bt2)));
+    const T bt = bb - w[5 + d] * w[5 + d] * ir;
+    const T bt2 = gt0(bt) ? bt : T(0);  // no negative rounding
+    const T cf = sqrt_T(T(0.5) * (sab + sqrt_T(dd * dd + T(4) * a2 * bt2)));
     const T spd = fabs(w[1 + d]) + cf;
     s += spd * idx[d];
     cmx = fmax(cmx, spd);
@@ -200,43 +214,28 @@ template <class T, int LIM, int FLUX, bool FULL> constexpr bool xy_pair_ok() {
   return sizeof(T) == 4 && LIM == AMRVAC_LIM_VANLEER && FLUX == AMRVAC_FLUX_HLLD && !FULL;
 }
 
-template <class T> __device__ __forceinline__ T over_dx(T a, T dx, T idx);
-template <> __device__ __forceinline__ double over_dx(double a, double dx, double) { return a / dx; }
-template <> __device__ __forceinline__ float over_dx(float a, float, float idx) { return a * idx; }
-
-// face flux from a 4-cell stencil accessor S(v, t), t = 0..3 for cells
-// f-2, f-1, f, f+1 around the face f-1/2; LIM < 0: runtime limiter lim
-template <class T, int D, int LIM, int FLUX, class Acc>
-__device__ __forceinline__ void stencil_flux(Acc S, int glm, T g, T ch, T* f, int lim) {
-  if constexpr (sizeof(T) == 4) {
-    // FP32 bulk: left/right states packed in float2 lanes (physics_f2.cuh)
-    stencil_flux_f2<D, LIM, FLUX>(S, glm, g, ch, f, lim);
-    return;
-  }
-  const int L = LIM >= 0 ? LIM : lim;
-  T wl[NV], wr[NV];
-#pragma unroll
-  for (int v = 0; v < NV; v++) {
-    T a = S(v, 0), b = S(v, 1), c = S(v, 2), e = S(v, 3);
-    wl[v] = recon_plus<T>(L, a, b, c);
-    wr[v] = recon_minus<T>(L, b, c, e);
-  }
-  if (!(wl[0] > T(0)) || !(wl[4] > T(0)) || !(wr[0] > T(0)) || !(wr[4] > T(0))) {
+// Riemann flux of a face (local frame of direction D) from its two limited
+// states, first order (the cell values cl(v), cr(v)) where one is not positive
+template <class T, int D, int FLUX, class CL, class CR>
+__device__ __forceinline__ void limited_flux(T* wl, T* wr, CL cl, CR cr, int glm,
+                                             const FaceConst<T>& fc, T* f) {
+  if (!gt0(wl[0]) || !gt0(wl[4]) || !gt0(wr[0]) || !gt0(wr[4])) {
 #pragma unroll
     for (int v = 0; v < NV; v++) {
-      wl[v] = S(v, 1);
-      wr[v] = S(v, 2);
+      wl[v] = cl(v);
+      wr[v] = cr(v);
     }
   }
-  face_flux_d<T, D>(FLUX, glm, g, ch, wl, wr, f);
+  face_flux_d<T, D>(FLUX, glm, fc, wl, wr, f);
 }
 
 // face flux from the six-cell stencil S(v, t), t = 0..5 for cells f-3 .. f+2
 // around the face f-1/2, with a five-point limiter lim (lam: wenozp5's lambda)
 template <class T, int D, int FLUX, class Acc>
-__device__ __forceinline__ void stencil_flux5(Acc S, int lim, T lam, int glm, T g, T ch, T* f) {
+__device__ __forceinline__ void stencil_flux5(Acc S, int lim, T lam, int glm,
+                                              const FaceConst<T>& fc, T* f) {
   if constexpr (sizeof(T) == 4) {
-    stencil_flux5_f2<D, FLUX>(S, lim, lam, glm, g, ch, f);
+    stencil_flux5_f2<D, FLUX>(S, lim, lam, glm, fc.g, fc.ch, f);
   } else {
     T wl[NV], wr[NV];
 #pragma unroll
@@ -245,14 +244,106 @@ __device__ __forceinline__ void stencil_flux5(Acc S, int lim, T lam, int glm, T 
       wl[v] = recon5_plus<T>(lim, c, lam);
       wr[v] = recon5_minus<T>(lim, c + 1, lam);
     }
-    if (!(wl[0] > T(0)) || !(wl[4] > T(0)) || !(wr[0] > T(0)) || !(wr[4] > T(0))) {
+    limited_flux<T, D, FLUX>(
+        wl, wr, [&](int v) { return S(v, 2); }, [&](int v) { return S(v, 3); }, glm, fc, f);
+  }
+}
+
+// The helper warp's share of the x and y faces of a plane in the shared-slope
+// layout.  Lane r < 16 works along row r in x, lane 16 + r along column r in y,
+// both in the face's local frame (component c is variable v(c)): `row` points
+// to the ghost end of its line of cells (stride st between cells, cv between
+// variables), `fr` to its face 0 in the flux array (strides fs and fv).
+template <class T, int G> struct HelperLine {
+  const T* row;
+  T* fr;
+  int st, cv, fs, fv;
+  bool ydir;
+  __device__ __forceinline__ int var(int c) const { return ydir ? yface_var(c) : c; }
+  // the state of cell -1 at face 0 into the flux array, that of cell 16 at
+  // face 16 into lo
+  __device__ __forceinline__ void slopes(int lim, T* lo) const {
 #pragma unroll
-      for (int v = 0; v < NV; v++) {
-        wl[v] = S(v, 2);
-        wr[v] = S(v, 3);
-      }
+    for (int c = 0; c < NV; c++) {
+      const T* r = row + var(c) * cv;
+      T other, hi;
+      cell_faces(lim, r[(G - 2) * st], r[(G - 1) * st], r[G * st], other, hi);
+      fr[var(c) * fv] = hi;
+      cell_faces(lim, r[(FB + G - 1) * st], r[(FB + G) * st], r[(FB + G + 1) * st], lo[c], hi);
     }
-    face_flux_d<T, D>(FLUX, glm, g, ch, wl, wr, f);
+  }
+  // flux of face 16, into the flux array and (variable order) out
+  template <int FLUX>
+  __device__ __forceinline__ void flux(T* lo, int glm, const FaceConst<T>& fc, T* out) const {
+    T wl[NV], f[NV];
+#pragma unroll
+    for (int c = 0; c < NV; c++) wl[c] = fr[var(c) * fv + FB * fs];
+    limited_flux<T, 0, FLUX>(
+        wl, lo, [&](int c) { return row[var(c) * cv + (FB + G - 1) * st]; },
+        [&](int c) { return row[var(c) * cv + (FB + G) * st]; }, glm, fc, f);
+#pragma unroll
+    for (int c = 0; c < NV; c++) fr[var(c) * fv + FB * fs] = f[c];
+#pragma unroll
+    for (int c = 0; c < NV; c++) out[yface_var(c)] = f[c];
+#pragma unroll
+    for (int c = 0; c < NV; c++) out[c] = ydir ? out[c] : f[c];
+  }
+};
+
+// The shared-slope x and y fluxes of a plane: prim[v][y][x] its primitives with
+// G ghost layers, fx and fy the face arrays (which first carry the states
+// handed over).  keep(face, idx, f) sees every block-boundary flux.  Contains
+// one barrier; the caller's next barrier makes the fluxes visible.
+template <class T, int LIM, int FLUX, int G, int PW, class Keep>
+__device__ __forceinline__ void shared_slope_xy(const T (*prim)[PW][PW], T (*fx)[FB][FXW],
+                                                T (*fy)[FB + 1][FXW], int x, int y, bool owner,
+                                                int runtime_lim, int glm, const FaceConst<T>& fc,
+                                                Keep keep) {
+  const int lim = LIM >= 0 ? LIM : runtime_lim;
+  if (owner) {
+    T lox[NV], loy[NV];
+#pragma unroll
+    for (int v = 0; v < NV; v++) {
+      const T c = prim[v][y + G][x + G];
+      T hi;
+      cell_faces(lim, prim[v][y + G][x + G - 1], c, prim[v][y + G][x + G + 1], lox[v], hi);
+      fx[v][y][x + 1] = hi;
+      cell_faces(lim, prim[v][y + G - 1][x + G], c, prim[v][y + G + 1][x + G], loy[v], hi);
+      fy[v][y + 1][x] = hi;
+    }
+    __syncthreads();
+    T wl[NV], f[NV];
+#pragma unroll
+    for (int v = 0; v < NV; v++) wl[v] = fx[v][y][x];
+    limited_flux<T, 0, FLUX>(
+        wl, lox, [&](int v) { return prim[v][y + G][x + G - 1]; },
+        [&](int v) { return prim[v][y + G][x + G]; }, glm, fc, f);
+#pragma unroll
+    for (int v = 0; v < NV; v++) fx[v][y][x] = f[v];
+    if (x == 0) keep(0, y, f);
+#pragma unroll
+    for (int v = 0; v < NV; v++) wl[v] = fy[v][y][x];
+    limited_flux<T, 1, FLUX>(
+        wl, loy, [&](int v) { return prim[v][y + G - 1][x + G]; },
+        [&](int v) { return prim[v][y + G][x + G]; }, glm, fc, f);
+#pragma unroll
+    for (int v = 0; v < NV; v++) fy[v][y][x] = f[v];
+    if (y == 0) keep(2, x, f);
+  } else {
+    const int r = threadIdx.x & 15;
+    HelperLine<T, G> h;
+    h.ydir = (threadIdx.x & 16) != 0;
+    h.row = h.ydir ? &prim[0][0][r + G] : &prim[0][r + G][0];
+    h.fr = h.ydir ? &fy[0][0][r] : &fx[0][r][0];
+    h.st = h.ydir ? PW : 1;
+    h.cv = PW * PW;
+    h.fs = h.ydir ? FXW : 1;
+    h.fv = h.ydir ? (FB + 1) * FXW : FB * FXW;
+    T lo[NV], out[NV];
+    h.slopes(lim, lo);
+    __syncthreads();
+    h.template flux<FLUX>(lo, glm, fc, out);
+    keep(h.ydir ? 3 : 1, r, out);
   }
 }
 
@@ -370,7 +461,7 @@ __global__ void __launch_bounds__(256)
 // LIM -2: the five-point limiters (runtime limiter, three ghost layers: a
 // 6-plane ring of 22 x 22 planes and 192 halo cells a plane, one CTA per SM)
 template <class T, int DIM, int LIM, int FLUX, bool FULL, bool PAIR>
-__global__ void __launch_bounds__(FT, sizeof(T) == 4 && !PAIR && LIM != -2 ? 2 : 1)
+__global__ void __launch_bounds__(fused_threads<T, LIM>(), sizeof(T) == 4 && !PAIR && LIM != -2 ? 2 : 1)
     k_fused(DevMesh M, const T* U0, const T* __restrict__ Uk, const T* U2, T* out, T* out2,
             const int* __restrict__ work, int nwork, const T* __restrict__ gslab,
             int* __restrict__ counter, StageParams sp) {
@@ -393,6 +484,7 @@ __global__ void __launch_bounds__(FT, sizeof(T) == 4 && !PAIR && LIM != -2 ? 2 :
   constexpr int SLAB_FACE = NV * G * FB * NT2;    // one face: [v][layer][t2][t1]
   static_assert(!PAIR || xy_pair_ok<T, LIM, FLUX, FULL>(), "face pairs: FP32 vanleer + HLLD");
   constexpr bool XYPAIR = PAIR;
+  constexpr bool SHARE = share_slopes<T, LIM>();
 
   const bool owner = tid < FB * FB;
   const int hr = tid - FB * FB;  // helper index 0..15
@@ -452,7 +544,7 @@ __global__ void __launch_bounds__(FT, sizeof(T) == 4 && !PAIR && LIM != -2 ? 2 :
 
     const T ch = lc[LC_CH], dt = lc[LC_DT];
     const T ca = sp_val<T>(sp.a, sp.af), cb = sp_val<T>(sp.b, sp.bf);
-    const T dx0 = lc[LC_DX], dx1 = lc[LC_DX + 1], dx2 = lc[LC_DX + 2];
+    const FaceConst<T> fc = face_const(g, ch);
     const T idx0 = idd[0], idx1 = idd[1], idx2 = idd[2];
     const T damp = lc[LC_DAMP];
 
@@ -565,23 +657,37 @@ __global__ void __launch_bounds__(FT, sizeof(T) == 4 && !PAIR && LIM != -2 ? 2 :
     const T lam[3] = {G == NG ? T(0) : (T)M.wzlam[(q * MAXLEV + L) * 3],
                       G == NG ? T(0) : (T)M.wzlam[(q * MAXLEV + L) * 3 + 1],
                       G == NG ? T(0) : (T)M.wzlam[(q * MAXLEV + L) * 3 + 2]};
+    // SHARE: the state of the own column's last cell at its next z face
+    T zhi[SHARE ? NV : 1];
+    auto zslot = [&](int zc, int o) { return (zc + o + 2 * NSLOT) % NSLOT; };
+    auto zcell = [&](int s, int v) -> T { return S.plane[s][v][y + G][x + G]; };
     auto zflux = [&](int zc, T* f) {
       // z face between planes zc-1 and zc of the thread's own column
-      if constexpr (G == NG) {
-        int s0 = (zc - 2 + 2 * NSLOT) % NSLOT, s1 = (zc - 1 + 2 * NSLOT) % NSLOT;
-        int s2 = (zc + 2 * NSLOT) % NSLOT, s3 = (zc + 1 + 2 * NSLOT) % NSLOT;
+      if constexpr (SHARE) {
+        const int lim = LIM >= 0 ? LIM : sp.limiter;
+        const int s1 = zslot(zc, -1), s2 = zslot(zc, 0), s3 = zslot(zc, 1);
+        T wr[NV], hi[NV];
+#pragma unroll
+        for (int v = 0; v < NV; v++)
+          cell_faces(lim, zcell(s1, v), zcell(s2, v), zcell(s3, v), wr[v], hi[v]);
+        limited_flux<T, 2, FLUX>(
+            zhi, wr, [&](int v) { return zcell(s1, v); }, [&](int v) { return zcell(s2, v); },
+            sp.glm, fc, f);
+#pragma unroll
+        for (int v = 0; v < NV; v++) zhi[v] = hi[v];
+      } else if constexpr (G == NG) {
+        int s0 = zslot(zc, -2), s1 = zslot(zc, -1), s2 = zslot(zc, 0), s3 = zslot(zc, 1);
         auto acc = [&](int v, int t) -> T {
-          int s = t == 0 ? s0 : (t == 1 ? s1 : (t == 2 ? s2 : s3));
-          return S.plane[s][v][y + NG][x + NG];
+          return zcell(t == 0 ? s0 : (t == 1 ? s1 : (t == 2 ? s2 : s3)), v);
         };
-        stencil_flux<T, 2, LIM, FLUX>(acc, sp.glm, g, ch, f, sp.limiter);
+        stencil_flux_f2<2, LIM, FLUX>(acc, sp.glm, g, ch, f, sp.limiter);
       } else {
         // planes zc-3 .. zc+2 (the ring holds exactly these six)
         int sl6[6];
 #pragma unroll
         for (int t = 0; t < 6; t++) sl6[t] = (zc - 3 + t + 2 * NSLOT) % NSLOT;
-        auto acc = [&](int v, int t) -> T { return S.plane[sl6[t]][v][y + G][x + G]; };
-        stencil_flux5<T, 2, FLUX>(acc, sp.limiter, lam[2], sp.glm, g, ch, f);
+        auto acc = [&](int v, int t) -> T { return zcell(sl6[t], v); };
+        stencil_flux5<T, 2, FLUX>(acc, sp.limiter, lam[2], sp.glm, fc, f);
       }
     };
 
@@ -601,7 +707,18 @@ __global__ void __launch_bounds__(FT, sizeof(T) == 4 && !PAIR && LIM != -2 ? 2 :
     for (int pz = -G; pz < G; pz++) issue_plane(pz);
     cp_async_wait_all();
     for (int pz = -G; pz < G; pz++) convert_plane(pz);
-    if (owner) zflux(0, fzp);  // own column only
+    if (owner) {  // own column only
+      if constexpr (SHARE) {
+        const int lim = LIM >= 0 ? LIM : sp.limiter;
+        const int s1 = zslot(-1, -1), s2 = zslot(-1, 0), s3 = zslot(-1, 1);
+#pragma unroll
+        for (int v = 0; v < NV; v++) {
+          T lo;
+          cell_faces(lim, zcell(s1, v), zcell(s2, v), zcell(s3, v), lo, zhi[v]);
+        }
+      }
+      zflux(0, fzp);
+    }
     if (FULL && sp.reflux && owner && nb[4] <= -3) keep_face_flux(M, nb[4], y * FB + x, fzp);
     __syncthreads();  // the halo copies of planes 0 and 1 are visible
     convert_halo(0);
@@ -636,7 +753,13 @@ __global__ void __launch_bounds__(FT, sizeof(T) == 4 && !PAIR && LIM != -2 ? 2 :
         issue_plane(z + G);  // commits this thread's copies as one group
       }
       const int sl = z % NSLOT, fb = z & 1;
-      {
+      if constexpr (SHARE) {
+        shared_slope_xy<T, LIM, FLUX, G, PW>(
+            S.plane[sl], S.fx[fb], S.fy[fb], x, y, owner, sp.limiter, sp.glm, fc,
+            [&](int face, int t, const T* f) {
+              if (FULL && sp.reflux && nb[face] <= -3) keep_face_flux(M, nb[face], z * FB + t, f);
+            });
+      } else {
         // owners: the x and y faces on the low side of their cell; helpers: the
         // x face at the +x block boundary of row hr and the y face at the +y
         // boundary of column hr
@@ -647,14 +770,14 @@ __global__ void __launch_bounds__(FT, sizeof(T) == 4 && !PAIR && LIM != -2 ? 2 :
         auto ay = [&](int v, int t) -> T { return S.plane[sl][v][fyr + t][fyc + G]; };
         if constexpr (G == NG5) {
           // five-point limiters: six-cell stencils
-          stencil_flux5<T, 0, FLUX>(ax, sp.limiter, lam[0], sp.glm, g, ch, f);
+          stencil_flux5<T, 0, FLUX>(ax, sp.limiter, lam[0], sp.glm, fc, f);
 #pragma unroll
           for (int v = 0; v < NV; v++) S.fx[fb][v][fxr][fxc] = f[v];
           if (FULL && sp.reflux) {
             const int face = owner ? (x == 0 ? 0 : -1) : 1;
             if (face >= 0 && nb[face] <= -3) keep_face_flux(M, nb[face], z * FB + fxr, f);
           }
-          stencil_flux5<T, 1, FLUX>(ay, sp.limiter, lam[1], sp.glm, g, ch, f);
+          stencil_flux5<T, 1, FLUX>(ay, sp.limiter, lam[1], sp.glm, fc, f);
 #pragma unroll
           for (int v = 0; v < NV; v++) S.fy[fb][v][fyr][fyc] = f[v];
           if (FULL && sp.reflux) {
@@ -677,14 +800,14 @@ __global__ void __launch_bounds__(FT, sizeof(T) == 4 && !PAIR && LIM != -2 ? 2 :
             if (facey >= 0 && nb[facey] <= -3) keep_face_flux(M, nb[facey], z * FB + fyc, f2);
           }
         } else {
-          stencil_flux<T, 0, LIM, FLUX>(ax, sp.glm, g, ch, f, sp.limiter);
+          stencil_flux_f2<0, LIM, FLUX>(ax, sp.glm, g, ch, f, sp.limiter);
 #pragma unroll
           for (int v = 0; v < NV; v++) S.fx[fb][v][fxr][fxc] = f[v];
           if (FULL && sp.reflux) {  // x faces on the block boundary: face 0 (owners x = 0), 1 (helpers)
             const int face = owner ? (x == 0 ? 0 : -1) : 1;
             if (face >= 0 && nb[face] <= -3) keep_face_flux(M, nb[face], z * FB + fxr, f);
           }
-          stencil_flux<T, 1, LIM, FLUX>(ay, sp.glm, g, ch, f, sp.limiter);
+          stencil_flux_f2<1, LIM, FLUX>(ay, sp.glm, g, ch, f, sp.limiter);
 #pragma unroll
           for (int v = 0; v < NV; v++) S.fy[fb][v][fyr][fyc] = f[v];
           if (FULL && sp.reflux) {  // y faces on the block boundary: face 2 (owners y = 0), 3 (helpers)
@@ -720,9 +843,9 @@ __global__ void __launch_bounds__(FT, sizeof(T) == 4 && !PAIR && LIM != -2 ? 2 :
       T un[NV];
 #pragma unroll
       for (int v = 0; v < NV; v++) {
-        T acc = over_dx<T>(S.fx[fb][v][y][x + 1] - S.fx[fb][v][y][x], dx0, idx0);
-        acc += over_dx<T>(S.fy[fb][v][y + 1][x] - S.fy[fb][v][y][x], dx1, idx1);
-        if (DIM == 3) acc += over_dx<T>(fz[v] - fzp[v], dx2, idx2);
+        T acc = (S.fx[fb][v][y][x + 1] - S.fx[fb][v][y][x]) * idx0;
+        acc += (S.fy[fb][v][y + 1][x] - S.fy[fb][v][y][x]) * idx1;
+        if (DIM == 3) acc += (fz[v] - fzp[v]) * idx2;
         const size_t at = (size_t)v * vs + (size_t)b * ncell + c;
         const T uk = PRE0 ? ukr[PRE0 ? v : 0] : Uk[at];
         T ut = uk - dt * acc;
@@ -757,14 +880,21 @@ namespace amrvac {
 
 // ---------------------------------------------------------------- launcher
 
+// the kernel of a dimension (the other one is not instantiated)
+template <class T, int DIM, int LIM, int FLUX, bool FULL, bool PAIR> constexpr auto fused_kernel() {
+  if constexpr (DIM == 3) return &k_fused<T, 3, LIM, FLUX, FULL, PAIR>;
+  else return &k_fused2d<T, LIM, FLUX, FULL, PAIR>;
+}
+
 template <class T, int DIM, int LIM, int FLUX, bool FULL, bool PAIR = false>
 static int launch_one(amrvac_state* s, const T* U0, const T* Uk, const T* U2, T* out, T* out2,
                       const int* work, int nwork, int* counter, StageParams sp) {
   static_assert(DIM == 2 || LIM != -2 || sizeof(T) == 4,
                 "five-point limiters in 3D: FP32 bulk only (a double 6-plane ring does not fit)");
-  auto kern = DIM == 3 ? k_fused<T, 3, LIM, FLUX, FULL, PAIR> : k_fused2d<T, LIM, FLUX, FULL, PAIR>;
+  const auto kern = fused_kernel<T, DIM, LIM, FLUX, FULL, PAIR>();
   const int smem = DIM == 3 ? (int)sizeof(FusedSmem<T, 3, PAIR, tile_ghosts(LIM)>)
                             : (int)sizeof(Fused2dSmem<T, tile_ghosts(LIM)>);
+  constexpr int NT = fused_threads<T, LIM>();
   static int nsm = 0, per_sm = 0;  // per instantiation, this device
   if (nsm == 0) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
@@ -773,7 +903,7 @@ static int launch_one(amrvac_state* s, const T* U0, const T* Uk, const T* U2, T*
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, FT, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem);
     if (per_sm < 1) per_sm = 1;
   }
   if (nwork <= 0) return 0;
@@ -783,7 +913,7 @@ static int launch_one(amrvac_state* s, const T* U0, const T* Uk, const T* U2, T*
   if (s->tune.dynamic) {
     if (cudaMemsetAsync(counter, 0, sizeof(int), s->stream) != cudaSuccess) return -1;
   }
-  kern<<<grid, FT, smem, s->stream>>>(s->mesh, U0, Uk, U2, out, out2, work, nwork,
+  kern<<<grid, NT, smem, s->stream>>>(s->mesh, U0, Uk, U2, out, out2, work, nwork,
                                        (const T*)s->gslab, s->tune.dynamic ? counter : nullptr,
                                        sp);
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;

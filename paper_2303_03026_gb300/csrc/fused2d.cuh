@@ -51,7 +51,7 @@ template <class T, int G = NG> struct Fused2dSmem {
 
 
 template <class T, int LIM, int FLUX, bool FULL, bool PAIR>
-__global__ void __launch_bounds__(FT, sizeof(T) == 4 && !PAIR ? 2 : 1)
+__global__ void __launch_bounds__(fused_threads<T, LIM>(), sizeof(T) == 4 && !PAIR ? 2 : 1)
     k_fused2d(DevMesh M, const T* U0, const T* __restrict__ Uk, const T* U2, T* out, T* out2,
               const int* __restrict__ work, int nwork, const T* __restrict__ gslab,
               int* __restrict__ counter, StageParams sp) {
@@ -211,7 +211,15 @@ __global__ void __launch_bounds__(FT, sizeof(T) == 4 && !PAIR ? 2 : 1)
 
       const T ch = lc[LC_CH], dt = lc[LC_DT];
       const T ca = sp_val<T>(sp.a, sp.af), cb = sp_val<T>(sp.b, sp.bf);
-      {
+      const FaceConst<T> fc = face_const(g, ch);
+      if constexpr (share_slopes<T, LIM>()) {
+        shared_slope_xy<T, LIM, FLUX, G, Fused2dSmem<T, G>::PW>(
+            S.prim, S.fx, S.fy, x, y, owner, sp.limiter, sp.glm, fc,
+            [&](int face, int t, const T* f) {
+              if (FULL && sp.reflux && M.nbr[b * 6 + face] == NBR_GENERAL)
+                keep_face_flux(M, -3 - M.gface[b * 6 + face], t, f);
+            });
+      } else {
         // owners: the x and y faces on the low side of their cell; helpers:
         // the x face at the +x block boundary of row hr and the y face at the
         // +y boundary of column hr
@@ -224,7 +232,7 @@ __global__ void __launch_bounds__(FT, sizeof(T) == 4 && !PAIR ? 2 : 1)
           // five-point limiters: six-cell stencils (three ghost layers)
           const int lv = M.blk[b * 5 + 1];
           const T lamx = (T)M.wzlam[(q * MAXLEV + lv) * 3], lamy = (T)M.wzlam[(q * MAXLEV + lv) * 3 + 1];
-          stencil_flux5<T, 0, FLUX>(ax, sp.limiter, lamx, sp.glm, g, ch, f);
+          stencil_flux5<T, 0, FLUX>(ax, sp.limiter, lamx, sp.glm, fc, f);
 #pragma unroll
           for (int v = 0; v < NV; v++) S.fx[v][fxr][fxc] = f[v];
           if (FULL && sp.reflux) {
@@ -232,7 +240,7 @@ __global__ void __launch_bounds__(FT, sizeof(T) == 4 && !PAIR ? 2 : 1)
             const int code = face >= 0 ? M.nbr[b * 6 + face] : 0;
             if (code == NBR_GENERAL) keep_face_flux(M, -3 - M.gface[b * 6 + face], fxr, f);
           }
-          stencil_flux5<T, 1, FLUX>(ay, sp.limiter, lamy, sp.glm, g, ch, f);
+          stencil_flux5<T, 1, FLUX>(ay, sp.limiter, lamy, sp.glm, fc, f);
 #pragma unroll
           for (int v = 0; v < NV; v++) S.fy[v][fyr][fyc] = f[v];
           if (FULL && sp.reflux) {
@@ -258,7 +266,7 @@ __global__ void __launch_bounds__(FT, sizeof(T) == 4 && !PAIR ? 2 : 1)
             if (codey == NBR_GENERAL) keep_face_flux(M, -3 - M.gface[b * 6 + facey], fyc, f2);
           }
         } else {
-          stencil_flux<T, 0, LIM, FLUX>(ax, sp.glm, g, ch, f, sp.limiter);
+          stencil_flux_f2<0, LIM, FLUX>(ax, sp.glm, g, ch, f, sp.limiter);
 #pragma unroll
           for (int v = 0; v < NV; v++) S.fx[v][fxr][fxc] = f[v];
           if (FULL && sp.reflux) {  // block-boundary x faces: 0 (owners x = 0), 1 (helpers)
@@ -267,7 +275,7 @@ __global__ void __launch_bounds__(FT, sizeof(T) == 4 && !PAIR ? 2 : 1)
             if (code == NBR_GENERAL)
               keep_face_flux(M, -3 - M.gface[b * 6 + face], fxr, f);
           }
-          stencil_flux<T, 1, LIM, FLUX>(ay, sp.glm, g, ch, f, sp.limiter);
+          stencil_flux_f2<1, LIM, FLUX>(ay, sp.glm, g, ch, f, sp.limiter);
 #pragma unroll
           for (int v = 0; v < NV; v++) S.fy[v][fyr][fyc] = f[v];
           if (FULL && sp.reflux) {  // block-boundary y faces: 2 (owners y = 0), 3 (helpers)
@@ -281,15 +289,14 @@ __global__ void __launch_bounds__(FT, sizeof(T) == 4 && !PAIR ? 2 : 1)
       __syncthreads();
       wnn = counter ? S.next : wn + gridDim.x;
       if (owner) {
-        const T dx0 = lc[LC_DX], dx1 = lc[LC_DX + 1];
         const T idx0 = idd[0], idx1 = idd[1];
         const T damp = lc[LC_DAMP];
         const int c = y * FB + x;
         T un[NV];
 #pragma unroll
         for (int v = 0; v < NV; v++) {
-          T acc = over_dx<T>(S.fx[v][y][x + 1] - S.fx[v][y][x], dx0, idx0);
-          acc += over_dx<T>(S.fy[v][y + 1][x] - S.fy[v][y][x], dx1, idx1);
+          T acc = (S.fx[v][y][x + 1] - S.fx[v][y][x]) * idx0;
+          acc += (S.fy[v][y + 1][x] - S.fy[v][y][x]) * idx1;
           const T uk = S.cons[s][v][y + G][x + G];
           T ut = uk - dt * acc;
           if (v == 8) ut = ut * damp;

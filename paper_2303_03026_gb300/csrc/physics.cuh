@@ -19,6 +19,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "fp64.cuh"
 
 namespace amrvac {
 
@@ -32,7 +33,7 @@ template <> struct Num<float> {
 
 // sign with sgn(0) = 0, by selects (no integer-to-float conversion)
 template <class T> __device__ __forceinline__ T sgnT(T x) {
-  return x > T(0) ? T(1) : (x < T(0) ? T(-1) : T(0));
+  return gt0(x) ? T(1) : (gt0(-x) ? T(-1) : T(0));
 }
 
 // ---------------------------------------------------------------- primitives
@@ -95,7 +96,7 @@ template <class T>
 __device__ __forceinline__ void cons2prim(double gamma, const T* u, T* w, bool ff = false,
                                           float gm1f = 0.f) {
   T rho = u[0];
-  T ir = T(1) / rho;
+  T ir = rcp_T(rho);
   T vx = u[1] * ir, vy = u[2] * ir, vz = u[3] * ir;
   w[0] = rho;
   w[1] = vx;
@@ -117,21 +118,25 @@ __device__ __forceinline__ void cons2prim(double gamma, const T* u, T* w, bool f
 template <class T>
 __device__ __forceinline__ T fast_speed(T gamma, const T* w, int d) {
   int t1 = d == 2 ? 0 : d + 1, t2 = d == 0 ? 2 : d - 1;
-  T ir = T(1) / w[0];
+  T ir = rcp_T(w[0]);
   T a2 = gamma * w[4] * ir;
   T bn = w[5 + d], b1 = w[5 + t1], b2 = w[5 + t2];
   T bt = b1 * b1 + b2 * b2;
   T bt2 = bt * ir;
   T bb = (bn * bn + bt) * ir;
   T dd = a2 - bb;
-  return sqrt(T(0.5) * (a2 + bb + sqrt(dd * dd + T(4) * a2 * bt2)));
+  return sqrt_T(T(0.5) * (a2 + bb + sqrt_T(dd * dd + T(4) * a2 * bt2)));
 }
 
 // small values (Sect. 7.4): density or pressure below its floor, or not
 // positive at all (the floors default to 0)
 template <class T> __device__ __forceinline__ bool is_small_prim(T rho, T p, T rho_floor,
                                                                   T p_floor) {
-  return !(rho > T(0) && rho >= rho_floor) || !(p > T(0) && p >= p_floor);
+  // (gt0, ge0, le_pos: no FP64 comparison; a floor that is not positive always
+  // holds for a positive value, a NaN floor never)
+  const bool fr = ge0(-rho_floor) || le_pos(rho_floor, rho);
+  const bool fp = ge0(-p_floor) || le_pos(p_floor, p);
+  return !(gt0(rho) && fr) || !(gt0(p) && fp);
 }
 
 // ---------------------------------------------------------------- limiters
@@ -160,7 +165,7 @@ template <class T> __device__ __forceinline__ T sym_slope(int lim, T dm, T dp) {
 // with p3 = (2a + t)/3; 0 where dp = 0 (the limit of phi dp)
 template <class T> __device__ __forceinline__ T cada3_half(T dm, T dp) {
   const T s = sgnT(dp), a = fabs(dp), t = s * dm;
-  const T p3 = (T(2) * a + t) / T(3);
+  const T p3 = (T(2) * a + t) * T(1.0 / 3.0);
   const T inner = fmin(fmin(T(2) * t, p3), T(1.6) * a);
   const T pa = fmax(T(0), fmin(p3, fmax(T(-0.5) * t, inner)));
   return T(0.5) * s * pa;
@@ -188,32 +193,62 @@ template <class T> __device__ __forceinline__ T venk_increment(T a, T b, T c) {
   return fmin(pr, pl) * d;
 }
 
-// face value at i+1/2 from the cell with values (a, b, c) = (w_{i-1}, w_i, w_{i+1})
-template <class T> __device__ __forceinline__ T recon_plus(int lim, T a, T b, T c) {
-  T dm = b - a, dp = c - b;
-  if (lim == AMRVAC_LIM_VENK) return b + venk_increment(a, b, c);
-  if (lim == AMRVAC_LIM_CADA3) return b + cada3_half(dm, dp);  // keeps a slope at extrema
-  if (!(dm * dp > T(0))) return b;
-  if (lim >= AMRVAC_LIM_SUPERBEE) return b + T(0.5) * sym_slope(lim, dm, dp);
-  if (lim == AMRVAC_LIM_MINMOD) return b + T(0.5) * minmod2(dm, dp);
-  if (lim == AMRVAC_LIM_VANLEER) return b + T(0.5) * (T(2) * dm * dp / (dm + dp));
-  T am = fabs(dm), ap = fabs(dp);
-  T l3 = fmin(fmin(T(2) * am, (am + T(2) * ap) / T(3)), T(2) * ap);
-  return b + T(0.5) * sgnT(dp) * l3;
+// Face values of the cell with values (a, b, c) = (w_{i-1}, w_i, w_{i+1}): hi at
+// i+1/2 and lo at i-1/2, from one evaluation of the limited slope (the caller
+// that uses one of them leaves the other to dead-code elimination)
+template <class T>
+__device__ __forceinline__ void cell_faces(int lim, T a, T b, T c, T& lo, T& hi) {
+  const T dm = b - a, dp = c - b;
+  if (lim == AMRVAC_LIM_VENK) {
+    const T s = venk_increment(a, b, c);
+    lo = b - s;
+    hi = b + s;
+    return;
+  }
+  if (lim == AMRVAC_LIM_CADA3) {  // keeps a slope at extrema
+    hi = b + cada3_half(dm, dp);
+    lo = b + cada3_half(-dp, -dm);  // the mirrored stencil
+    return;
+  }
+  const T prod = dm * dp;
+  lo = b;
+  hi = b;
+  if (!gt0(prod)) return;
+  if (lim == AMRVAC_LIM_VANLEER) {
+    const T s = prod * rcp_T(dm + dp);
+    lo = b - s;
+    hi = b + s;
+    return;
+  }
+  if (lim >= AMRVAC_LIM_SUPERBEE) {
+    const T s = T(0.5) * sym_slope(lim, dm, dp);
+    lo = b - s;
+    hi = b + s;
+    return;
+  }
+  // minmod and koren as halves: min(|dm|, |dp|)/2, and min(|dm|, (|dm| +
+  // 2 |dp|)/6, |dp|) towards i+1/2 (mirrored towards i-1/2)
+  const T am = fabs(dm), ap = fabs(dp), m = min_pos(am, ap);
+  if (lim == AMRVAC_LIM_MINMOD) {
+    const T s = copysign(T(0.5) * m, dp);
+    lo = b - s;
+    hi = b + s;
+    return;
+  }
+  hi = b + copysign(min_pos(m, (am + T(2) * ap) * T(1.0 / 6.0)), dp);
+  lo = b - copysign(min_pos(m, (ap + T(2) * am) * T(1.0 / 6.0)), dp);
 }
 
-// face value at i-1/2 from the cell with values (a, b, c)
+template <class T> __device__ __forceinline__ T recon_plus(int lim, T a, T b, T c) {
+  T lo, hi;
+  cell_faces(lim, a, b, c, lo, hi);
+  return hi;
+}
+
 template <class T> __device__ __forceinline__ T recon_minus(int lim, T a, T b, T c) {
-  T dm = b - a, dp = c - b;
-  if (lim == AMRVAC_LIM_VENK) return b - venk_increment(a, b, c);
-  if (lim == AMRVAC_LIM_CADA3) return b + cada3_half(-dp, -dm);  // the mirrored stencil
-  if (!(dm * dp > T(0))) return b;
-  if (lim >= AMRVAC_LIM_SUPERBEE) return b - T(0.5) * sym_slope(lim, dm, dp);
-  if (lim == AMRVAC_LIM_MINMOD) return b - T(0.5) * minmod2(dm, dp);
-  if (lim == AMRVAC_LIM_VANLEER) return b - T(0.5) * (T(2) * dm * dp / (dm + dp));
-  T am = fabs(dm), ap = fabs(dp);
-  T l3 = fmin(fmin(T(2) * ap, (ap + T(2) * am) / T(3)), T(2) * am);
-  return b - T(0.5) * sgnT(dm) * l3;
+  T lo, hi;
+  cell_faces(lim, a, b, c, lo, hi);
+  return lo;
 }
 
 // Five-point limiters of the limiter table (3 ghost cells), face value at
@@ -238,7 +273,7 @@ template <class T> __device__ __forceinline__ T minmod4g(T w, T x, T y, T z) {
 
 template <class T> __device__ __forceinline__ T mp5_face(T vm2, T vm1, T v0, T vp1, T vp2) {
   const T a = T(4);
-  const T vor = (T(2) * vm2 - T(13) * vm1 + T(47) * v0 + T(27) * vp1 - T(3) * vp2) / T(60);
+  const T vor = (T(2) * vm2 - T(13) * vm1 + T(47) * v0 + T(27) * vp1 - T(3) * vp2) * T(1.0 / 60.0);
   const T vmp = v0 + minmod2(vp1 - v0, a * (v0 - vm1));
   if ((vor - v0) * (vor - vmp) <= T(0)) return vor;
   const T djm1 = vm2 - T(2) * vm1 + v0, dj = vm1 - T(2) * v0 + vp1, djp1 = v0 - T(2) * vp1 + vp2;
@@ -291,9 +326,9 @@ __device__ __forceinline__ T weno5_face(int kind, T vm2, T vm1, T v0, T vp1, T v
     b1 = beta_rn(tt1, uu1);
     b2 = beta_rn(tt2, uu2);
   }
-  const T q0 = (T(2) * vm2 - T(7) * vm1 + T(11) * v0) / T(6);
-  const T q1 = (-vm1 + T(5) * v0 + T(2) * vp1) / T(6);
-  const T q2 = (T(2) * v0 + T(5) * vp1 - vp2) / T(6);
+  const T q0 = (T(2) * vm2 - T(7) * vm1 + T(11) * v0) * T(1.0 / 6.0);
+  const T q1 = (-vm1 + T(5) * v0 + T(2) * vp1) * T(1.0 / 6.0);
+  const T q2 = (T(2) * v0 + T(5) * vp1 - vp2) * T(1.0 / 6.0);
   T a0, a1, a2;
   if (kind == 2) {
     const T eps = sizeof(T) == 8 ? T(1e-40) : T(1e-36), tau = fabs(b0 - b2);
@@ -397,14 +432,19 @@ __device__ __forceinline__ void local_cons_flux(T ig1, const T* q, T bx, T* U, T
   F[7] = bz * u - bx * w;
 }
 
-template <class T> __device__ __forceinline__ T local_fast(T g, const T* q, T bx) {
-  T ir = T(1) / q[0];
+// square of the fast speed
+template <class T> __device__ __forceinline__ T local_fast2(T g, const T* q, T bx) {
+  T ir = rcp_T(q[0]);
   T bt = q[6] * q[6] + q[7] * q[7];
   T a2 = g * q[4] * ir;
   T bt2 = bt * ir;
   T bb = (bx * bx + bt) * ir;
   T dd = a2 - bb;
-  return sqrt(T(0.5) * (a2 + bb + sqrt(dd * dd + T(4) * a2 * bt2)));
+  return T(0.5) * (a2 + bb + sqrt_T(dd * dd + T(4) * (a2 * bt2)));
+}
+
+template <class T> __device__ __forceinline__ T local_fast(T g, const T* q, T bx) {
+  return sqrt_T(local_fast2(g, q, bx));
 }
 
 template <class T>
@@ -415,12 +455,13 @@ __device__ __forceinline__ void hll_local(T g, T ig1, const T* ql, const T* qr, 
   T cfl = local_fast(g, ql, bx), cfr = local_fast(g, qr, bx);
   T sl = fmin(ql[1] - cfl, qr[1] - cfr);
   T sr = fmax(ql[1] + cfl, qr[1] + cfr);
-  T inv = T(1) / (sr - sl);
+  T inv = rcp_T(sr - sl);
+  const bool left = ge0(sl), right = ge0(-sr);
+  const T wl = sr * inv, wr = -(sl * inv), wu = sl * wl;
 #pragma unroll
   for (int c = 0; c < 8; c++) {
-    if (sl >= T(0)) f[c] = FL[c];
-    else if (sr <= T(0)) f[c] = FR[c];
-    else f[c] = (sr * FL[c] - sl * FR[c] + sl * sr * (UR[c] - UL[c])) * inv;
+    const T m = wl * FL[c] + wr * FR[c] + wu * (UR[c] - UL[c]);
+    f[c] = left ? FL[c] : (right ? FR[c] : m);
   }
 }
 
@@ -460,11 +501,13 @@ __device__ __forceinline__ void hllc_local(T g, T ig1, const T* ql, const T* qr,
     for (int c = 0; c < 8; c++) f[c] = FR[c];
     return;
   }
+  const T inv = rcp_T(sr - sl);
   T uh[8];
 #pragma unroll
-  for (int c = 0; c < 8; c++) uh[c] = (sr * UR[c] - sl * UL[c] - FR[c] + FL[c]) / (sr - sl);
-  const T sm = uh[1] / uh[0];
-  const T vy = uh[2] / uh[0], vz = uh[3] / uh[0];
+  for (int c = 0; c < 8; c++) uh[c] = (sr * UR[c] - sl * UL[c] - FR[c] + FL[c]) * inv;
+  const T ih = rcp_T(uh[0]);
+  const T sm = uh[1] * ih;
+  const T vy = uh[2] * ih, vz = uh[3] * ih;
   const T by = uh[6], bz = uh[7];
   const T pts = ql[0] * (sl - ql[1]) * (sm - ql[1]) + ptl;
   const T vbs = sm * bx + vy * by + vz * bz;
@@ -473,14 +516,14 @@ __device__ __forceinline__ void hllc_local(T g, T ig1, const T* ql, const T* qr,
   const T* U = left ? UL : UR;
   const T* F = left ? FL : FR;
   const T S = left ? sl : sr, pt = left ? ptl : ptr;
-  const T su = S - q[1], ssm = S - sm;
+  const T su = S - q[1], isd = rcp_T(S - sm);
   const T vb = q[1] * bx + q[2] * q[6] + q[3] * q[7];
   T Us[8];
-  Us[0] = q[0] * su / ssm;
+  Us[0] = q[0] * su * isd;
   Us[1] = Us[0] * sm;
-  Us[2] = (q[0] * q[2] * su - (bx * by - bx * q[6])) / ssm;
-  Us[3] = (q[0] * q[3] * su - (bx * bz - bx * q[7])) / ssm;
-  Us[4] = (U[4] * su + pts * sm - pt * q[1] - bx * (vbs - vb)) / ssm;
+  Us[2] = (q[0] * q[2] * su - (bx * by - bx * q[6])) * isd;
+  Us[3] = (q[0] * q[3] * su - (bx * bz - bx * q[7])) * isd;
+  Us[4] = (U[4] * su + pts * sm - pt * q[1] - bx * (vbs - vb)) * isd;
   Us[5] = bx;
   Us[6] = by;
   Us[7] = bz;
@@ -489,37 +532,33 @@ __device__ __forceinline__ void hllc_local(T g, T ig1, const T* ql, const T* qr,
 }
 
 template <class T> struct StarState {
-  T rs, vs, ws, bys, bzs, es;
+  T rs, vs, ws, bys, bzs, es, vbs;
 };
 
+// single-star state of one side: su = S - u, A = rho su, psm = p_T* S_M, sbx =
+// S_M B_x, bx2 = B_x^2
 template <class T>
-__device__ __forceinline__ StarState<T> hlld_star(const T* q, T e, T pt, T s, T sm, T pts,
-                                                  T bx) {
+__device__ __forceinline__ StarState<T> hlld_star(const T* q, T e, T pt, T s, T su, T A, T sm,
+                                                  T psm, T sbx, T bx, T bx2) {
   StarState<T> r;
-  T rho = q[0], u = q[1], v = q[2], w = q[3], by = q[6], bz = q[7];
-  T su = s - u;
-  T isd = T(1) / (s - sm);
-  r.rs = rho * su * isd;
-  T big = rho * su * (s - sm);
-  T den = big - bx * bx;
-  T scale = fmax(fabs(big), bx * bx);
-  if (fabs(den) <= Num<T>::hlld_eps * scale) {
-    r.vs = v;
-    r.ws = w;
-    r.bys = by;
-    r.bzs = bz;
-  } else {
-    T iden = T(1) / den;
-    T tv = bx * (sm - u) * iden;
-    T tb = (rho * su * su - bx * bx) * iden;
-    r.vs = v - by * tv;
-    r.ws = w - bz * tv;
-    r.bys = by * tb;
-    r.bzs = bz * tb;
-  }
-  T vb = u * bx + v * by + w * bz;
-  T vbs = sm * bx + r.vs * r.bys + r.ws * r.bzs;
-  r.es = (su * e - pt * u + pts * sm + bx * (vb - vbs)) * isd;
+  const T u = q[1], v = q[2], w = q[3], by = q[6], bz = q[7];
+  const T ssm = s - sm;
+  const T isd = rcp_T(ssm);
+  r.rs = A * isd;
+  const T big = A * ssm;
+  const T den = big - bx2;
+  const T scale = max_pos(fabs(big), bx2);
+  const bool flat = le_pos(fabs(den), Num<T>::hlld_eps * scale);
+  const T iden = rcp_T(den);
+  const T tv = bx * (sm - u) * iden;
+  const T tb = (A * su - bx2) * iden;
+  r.vs = flat ? v : v - by * tv;
+  r.ws = flat ? w : w - bz * tv;
+  r.bys = flat ? by : by * tb;
+  r.bzs = flat ? bz : bz * tb;
+  const T vb = u * bx + v * by + w * bz;
+  r.vbs = sbx + r.vs * r.bys + r.ws * r.bzs;
+  r.es = (su * e - pt * u + psm + bx * (vb - r.vbs)) * isd;
   return r;
 }
 
@@ -566,33 +605,38 @@ __device__ __forceinline__ void hlld_local(T g, T ig1, const T* ql, const T* qr,
     er = qr[4] * ig1 + T(0.5) * qr[0] * (qr[1] * qr[1] + qr[2] * qr[2] + qr[3] * qr[3]) +
          T(0.5) * b2;
   }
-  T cfl = local_fast(g, ql, bx), cfr = local_fast(g, qr, bx);
-  T ul = ql[1], ur = qr[1];
-  T cmax = fmax(cfl, cfr);
-  T sl = fmin(ul, ur) - cmax;
-  T sr = fmax(ul, ur) + cmax;
-  T rl = ql[0], rr = qr[0];
-  T sul = sl - ul, sur = sr - ur;
-  T iden = T(1) / (sur * rr - sul * rl);
-  T sm = (sur * rr * ur - sul * rl * ul - ptr + ptl) * iden;
-  T pts = (sur * rr * ptl - sul * rl * ptr + rl * rr * sur * sul * (ur - ul)) * iden;
-  StarState<T> L = hlld_star(ql, el, ptl, sl, sm, pts, bx);
-  StarState<T> R = hlld_star(qr, er, ptr, sr, sm, pts, bx);
-  T sqrl = sqrt(L.rs), sqrr = sqrt(R.rs);
-  T ssl = sm - fabs(bx) / sqrl, ssr = sm + fabs(bx) / sqrr;
-  T sb = sgnT(bx);
-  T issum = T(1) / (sqrl + sqrr);
-  T vss = (sqrl * L.vs + sqrr * R.vs + (R.bys - L.bys) * sb) * issum;
-  T wss = (sqrl * L.ws + sqrr * R.ws + (R.bzs - L.bzs) * sb) * issum;
-  T byss = (sqrl * R.bys + sqrr * L.bys + sqrl * sqrr * (R.vs - L.vs) * sb) * issum;
-  T bzss = (sqrl * R.bzs + sqrr * L.bzs + sqrl * sqrr * (R.ws - L.ws) * sb) * issum;
-  T vbss = sm * bx + vss * byss + wss * bzss;
-  T essl = L.es - sqrl * (sm * bx + L.vs * L.bys + L.ws * L.bzs - vbss) * sb;
-  T essr = R.es + sqrr * (sm * bx + R.vs * R.bys + R.ws * R.bzs - vbss) * sb;
+  // one root for both sides: the larger of the squared fast speeds
+  const T cmax = sqrt_T(fmax(local_fast2(g, ql, bx), local_fast2(g, qr, bx)));
+  const T ul = ql[1], ur = qr[1], du = ur - ul;
+  const bool up = gt0(du);
+  const T sl = (up ? ul : ur) - cmax;
+  const T sr = (up ? ur : ul) + cmax;
+  const T bx2 = bx * bx;
+  const T sul = sl - ul, sur = sr - ur;
+  const T Al = ql[0] * sul, Ar = qr[0] * sur;
+  const T iden = rcp_T(Ar - Al);
+  const T sm = ((Ar * ur + ptl) - (Al * ul + ptr)) * iden;
+  const T pts = (Ar * ptl - Al * ptr + Al * Ar * du) * iden;
+  const T psm = pts * sm, sbx = sm * bx;
+  const StarState<T> L = hlld_star(ql, el, ptl, sl, sul, Al, sm, psm, sbx, bx, bx2);
+  const StarState<T> R = hlld_star(qr, er, ptr, sr, sur, Ar, sm, psm, sbx, bx, bx2);
+  T sqrl, sqrr, isql, isqr;
+  sqrt_pair(L.rs, sqrl, isql);
+  sqrt_pair(R.rs, sqrr, isqr);
+  const T abx = fabs(bx);
+  const T ssl = sm - abx * isql, ssr = sm + abx * isqr;
+  const T sb = sgnT(bx);
+  const T issum = rcp_T(sqrl + sqrr);
+  const T wl = sqrl * issum, wr = sqrr * issum, wsb = sb * issum, wq = sqrl * wr * sb;
+  const T vss = wl * L.vs + wr * R.vs + (R.bys - L.bys) * wsb;
+  const T wss = wl * L.ws + wr * R.ws + (R.bzs - L.bzs) * wsb;
+  const T byss = wl * R.bys + wr * L.bys + (R.vs - L.vs) * wq;
+  const T bzss = wl * R.bzs + wr * L.bzs + (R.ws - L.ws) * wq;
+  const T vbss = sbx + vss * byss + wss * bzss;
   // region of the fan that contains x/t = 0 (same tie rules as the oracle)
-  const bool left = sm >= T(0);
-  const bool outer = left ? (sl > T(0)) : (sr < T(0));
-  const bool single = left ? (ssl >= T(0)) : !(ssr >= T(0));
+  const bool left = ge0(sm);
+  const bool outer = left ? gt0(sl) : gt0(-sr);
+  const bool single = left ? ge0(ssl) : !ge0(ssr);
   T q[8];
 #pragma unroll
   for (int c = 0; c < 8; c++) q[c] = left ? ql[c] : qr[c];
@@ -600,26 +644,39 @@ __device__ __forceinline__ void hlld_local(T g, T ig1, const T* ql, const T* qr,
   phys_flux_state(q, bx, left ? ptl : ptr, left ? el : er, U, F);
   const T rs = left ? L.rs : R.rs, vs = left ? L.vs : R.vs, ws = left ? L.ws : R.ws;
   const T bys = left ? L.bys : R.bys, bzs = left ? L.bzs : R.bzs, es = left ? L.es : R.es;
+  // e** = e* -/+ sqrt(rho*) (v*.B* - v**.B**) sgn(Bx)
+  const T ess = es + (left ? -sqrl : sqrr) * sb * ((left ? L.vbs : R.vbs) - vbss);
   const T c1 = left ? sl : sr, c2 = left ? ssl : ssr;
   const T US[8] = {rs, rs * sm, rs * vs, rs * ws, es, bx, bys, bzs};
-  const T USS[8] = {rs, rs * sm, rs * vss, rs * wss, left ? essl : essr, bx, byss, bzss};
+  const T c2r = c2 * rs;  // the double-star state keeps rho* and S_M
+  const T D[8] = {T(0),          T(0), c2r * (vss - vs),  c2r * (wss - ws),
+                  c2 * (ess - es), T(0), c2 * (byss - bys), c2 * (bzss - bzs)};
 #pragma unroll
   for (int c = 0; c < 8; c++) {
-    T fs = F[c] + c1 * (US[c] - U[c]);
-    T v = single ? fs : fs + c2 * (USS[c] - US[c]);
+    const T fs = F[c] + c1 * (US[c] - U[c]);
+    const T v = single || c == 0 || c == 1 || c == 5 ? fs : fs + D[c];
     f[c] = outer ? F[c] : v;
   }
 }
 
+// constants of a face flux: gamma, 1/(gamma - 1), c_h and 1/(2 c_h)
+template <class T> struct FaceConst {
+  T g, ig1, ch, hich;
+};
+template <class T> __device__ __forceinline__ FaceConst<T> face_const(T g, T ch) {
+  return {g, rcp_T(g - T(1)), ch, T(0.5) * rcp_T(ch)};
+}
+
 // Face flux along D from primitive face states wl, wr (global frame).
 template <class T, int D>
-__device__ __forceinline__ void face_flux_d(int flux, int glm, T g, T ch, const T* wl,
-                                            const T* wr, T* f) {
+__device__ __forceinline__ void face_flux_d(int flux, int glm, const FaceConst<T>& fc,
+                                            const T* wl, const T* wr, T* f) {
+  const T g = fc.g, ch = fc.ch, ig1 = fc.ig1;
   constexpr int t1 = D == 2 ? 0 : D + 1, t2 = D == 0 ? 2 : D - 1;
   T bnl = wl[5 + D], bnr = wr[5 + D];
   T bns, psis;
   if (glm) {
-    bns = T(0.5) * (bnl + bnr) - (wr[8] - wl[8]) / (T(2) * ch);
+    bns = T(0.5) * (bnl + bnr) - (wr[8] - wl[8]) * fc.hich;
     psis = T(0.5) * (wl[8] + wr[8]) - T(0.5) * ch * (bnr - bnl);
   } else {
     bns = T(0.5) * (bnl + bnr);
@@ -628,7 +685,6 @@ __device__ __forceinline__ void face_flux_d(int flux, int glm, T g, T ch, const 
   T ql[8] = {wl[0], wl[1 + D], wl[1 + t1], wl[1 + t2], wl[4], bns, wl[5 + t1], wl[5 + t2]};
   T qr[8] = {wr[0], wr[1 + D], wr[1 + t1], wr[1 + t2], wr[4], bns, wr[5 + t1], wr[5 + t2]};
   T fl[8];
-  const T ig1 = T(1) / (g - T(1));
   if (flux == AMRVAC_FLUX_HLL) hll_local(g, ig1, ql, qr, bns, fl);
   else if (flux == AMRVAC_FLUX_HLLD) hlld_local(g, ig1, ql, qr, bns, fl);
   else if (flux == AMRVAC_FLUX_TVDLF) tvdlf_local(g, ig1, ql, qr, bns, fl);
@@ -647,9 +703,10 @@ __device__ __forceinline__ void face_flux_d(int flux, int glm, T g, T ch, const 
 template <class T>
 __device__ __forceinline__ void face_flux(int flux, int glm, T g, T ch, int d, const T* wl,
                                           const T* wr, T* f) {
-  if (d == 0) face_flux_d<T, 0>(flux, glm, g, ch, wl, wr, f);
-  else if (d == 1) face_flux_d<T, 1>(flux, glm, g, ch, wl, wr, f);
-  else face_flux_d<T, 2>(flux, glm, g, ch, wl, wr, f);
+  const FaceConst<T> fc = face_const(g, ch);
+  if (d == 0) face_flux_d<T, 0>(flux, glm, fc, wl, wr, f);
+  else if (d == 1) face_flux_d<T, 1>(flux, glm, fc, wl, wr, f);
+  else face_flux_d<T, 2>(flux, glm, fc, wl, wr, f);
 }
 
 }  // namespace amrvac

@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(256) k_update(DevMesh M, const T* U0,
     const T damp2 = sp.glm ? (T)exp(-sp.glm_alpha * rt.ch * dt2 / dxmin) : T(1);
     const T dt = (T)dt1, dtb = (T)dt2, a = (T)sp.a, bb = (T)sp.b;
     const T a2 = (T)sp.a2, b2 = (T)sp.b2;
-    const T idx0 = (T)dx[0], idx1 = (T)dx[1], idx2 = (T)dx[2];
+    const T idx0 = (T)(1.0 / dx[0]), idx1 = (T)(1.0 / dx[1]), idx2 = (T)(1.0 / dx[2]);
     for (int c = threadIdx.x; c < M.ncell; c += blockDim.x) {
       int i = c % nx0, j = (c / nx0) % nx1, k = c / (nx0 * nx1);
       T un[NV], u2n[NV];
@@ -164,14 +164,14 @@ __global__ void __launch_bounds__(256) k_update(DevMesh M, const T* U0,
 #pragma unroll
         for (int v = 0; v < NV; v++) {
           const T* g0 = F0 + ((size_t)b * NV + v) * nf0;
-          T acc = (g0[f0 + 1] - g0[f0]) / idx0;
+          T acc = (g0[f0 + 1] - g0[f0]) * idx0;
           if (M.ndim > 1) {
             const T* g1 = F1 + ((size_t)b * NV + v) * nf1;
-            acc += (g1[f1 + nx0] - g1[f1]) / idx1;
+            acc += (g1[f1 + nx0] - g1[f1]) * idx1;
           }
           if (M.ndim > 2) {
             const T* g2 = F2 + ((size_t)b * NV + v) * nf2;
-            acc += (g2[f2 + (size_t)nx0 * nx1] - g2[f2]) / idx2;
+            acc += (g2[f2 + (size_t)nx0 * nx1] - g2[f2]) * idx2;
           }
           size_t at = (size_t)v * vs + (size_t)b * M.ncell + c;
           T ut = Uk[at] - dt * acc;
