@@ -377,16 +377,11 @@ amrvac_status amrvac_state_load(amrvac_state* s, const char* path);
 /*
  * Launch shape of the fused stage kernel (its tile is the 16^d block):
  * resident CTAs per SM (0 = as many as fit), work-list order (0 = Morton curve
- * per instance, 1 = storage order), block scheduling (0 = static, 1 = dynamic
- * via a device counter), and the faces a thread packs into the two lanes of
- * its FP32x2 instructions (0 = the two sides of one face: a 96-register kernel,
- * two CTAs per SM; 1 = the x and y faces of its cell together: fewer
- * instructions, a ~160-register kernel with one CTA per SM; FP32 bulk with
- * vanleer + HLLD only, ignored otherwise).  ctas_per_sm, order and dynamic do
- * not change the arithmetic (results are bit-identical across them); faces = 1
- * evaluates the same formulas with another FP32 grouping (results agree to
- * float rounding).  Setting a tuning drops the captured step graph.  Not part
- * of the paper (a GB300 launch-shape choice).
+ * per instance, 1 = storage order) and block scheduling (0 = static, 1 = dynamic
+ * via a device counter).  faces (0 or 1) is kept for callers and caches that set
+ * it: one FP32 kernel serves both values.  None of them changes the arithmetic
+ * (results are bit-identical).  Setting a tuning drops the captured step graph.
+ * Not part of the paper (a GB300 launch-shape choice).
  */
 typedef struct {
   int32_t ctas_per_sm;
@@ -400,8 +395,8 @@ amrvac_status amrvac_set_tuning(amrvac_state* s, const amrvac_tuning* t);
 amrvac_status amrvac_get_tuning(amrvac_state* s, amrvac_tuning* t);
 
 /*
- * Times every launch shape (ctas_per_sm x order x dynamic, and faces where it
- * applies: 8 or 12 shapes) over trial_steps full steps on the state itself
+ * Times every launch shape (ctas_per_sm x order x dynamic: 8 shapes, faces 0)
+ * over trial_steps full steps on the state itself
  * (U^n and the clocks are restored after each trial and at the end), keeps the
  * fastest and returns it in *best.  With cache_path, a tuning stored there for
  * the same (ndim, block size, precision, flux, limiter, pressure, block-count

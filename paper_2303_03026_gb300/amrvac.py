@@ -343,9 +343,8 @@ class State:
                 "error": (err.code, err.block, err.cell, err.var)}
 
     def set_tuning(self, ctas_per_sm=0, order="morton", dynamic=False, faces="sides"):
-        """Launch shape of the fused kernels (amrvac_tuning): faces "sides" packs
-        the two sides of one face per float2 lane pair, "xy" a cell's x and y
-        faces (FP32 vanleer + HLLD)."""
+        """Launch shape of the fused kernels (amrvac_tuning); faces ("sides" or
+        "xy") is accepted and kept, one kernel serves both."""
         t = Tuning(int(ctas_per_sm), {"morton": 0, "storage": 1}[order], int(bool(dynamic)),
                    {"sides": 0, "xy": 1}[faces], 0.0)
         _check(load().amrvac_set_tuning(self._h, C.byref(t)), "amrvac_set_tuning")

@@ -20,9 +20,10 @@ LIB = os.path.join(OUT_DIR, "libamrvac_gb300.so")
 SOURCES = ["api.cu", "plain.cu", "fused.cu", "noalloc.cu", "fix.cu", "reflux.cu", "regrid.cu"]
 # the fused kernel source is compiled once per (precision, dimension, limiter)
 # limiter groups: minmod, vanleer, koren as compile-time limiters, -1 = the
-# other two-ghost-cell limiters at run time, -2 = the five-point limiters at run
-# time (2D tiles only)
+# other two-ghost-cell limiters at run time (FP32: superbee, woodward, mcbeta; -3
+# the rest), -2 = the five-point limiters at run time
 FUSED_GROUPS = ([(t, d, l) for t in ("float", "double") for d in (2, 3) for l in (0, 1, 2, -1)] +
+                [("float", d, -3) for d in (2, 3)] +
                 [(t, 2, -2) for t in ("float", "double")] + [("float", 3, -2)])
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xptxas", "-v",
@@ -48,8 +49,8 @@ def _digest() -> str:
 
 
 # the translation unit of the fused stage kernels and everything it includes
-FUSED_KERNEL_FILES = ["fused_inst.cu", "fused.cuh", "fused2d.cuh", "ghost.cuh", "physics.cuh",
-                      "physics_f2.cuh", "reduce.cuh", "state.hpp", "common.cuh"]
+FUSED_KERNEL_FILES = ["fused_inst.cu", "fused.cuh", "fused2d.cuh", "fused_f2.cuh", "ghost.cuh",
+                      "physics.cuh", "physics_f2.cuh", "fp64.cuh", "reduce.cuh", "state.hpp", "common.cuh"]
 
 
 def kernel_digest() -> str:
@@ -81,7 +82,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         # FP32 bulk: approximate single-precision division and square root
         # (MUFU based, <= 2 ulp) and flush-to-zero; double arithmetic unaffected
         fast = ["-prec-div=false", "-prec-sqrt=false", "-ftz=true"] if t == "float" else []
-        units.append(("fused_inst.cu", "fused_%s_%dd_l%s.o" % (t, d, {-1: "rt", -2: "r5"}.get(l, l)),
+        units.append(("fused_inst.cu", "fused_%s_%dd_l%s.o" % (t, d, {-1: "rt", -2: "r5", -3: "rx"}.get(l, l)),
                       ["-DAMRVAC_FT=" + t, "-DAMRVAC_FD=%d" % d, "-DAMRVAC_FL=%d" % l] + fast))
 
     def compile_one(unit):

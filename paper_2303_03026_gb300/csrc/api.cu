@@ -1042,23 +1042,11 @@ amrvac_status amrvac_autotune(amrvac_state* s, int32_t trial_steps, const char* 
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
     return AMRVAC_E_CUDA;
-  // face pairs apply to the lean FP32 vanleer + HLLD scheme groups; their
-  // kernel holds one CTA per SM, so only the default CTA count is tried
-  bool pairs = s->cfg.precision == AMRVAC_FP32_BULK && !s->cfg.reflux &&
-               s->cfg.time != AMRVAC_SSPRK54;
-  bool eligible = false;
-  for (int d = 0; d < s->cfg.ndim; d++)
-    pairs = pairs && s->cfg.bc[d][0] != AMRVAC_BC_SYMMETRIC && s->cfg.bc[d][1] != AMRVAC_BC_SYMMETRIC;
-  for (int g = 0; g < s->ngroups; g++)
-    eligible = eligible || (s->grp_flux[g] == AMRVAC_FLUX_HLLD && s->grp_lim[g] == AMRVAC_LIM_VANLEER);
-  pairs = pairs && eligible;
-  amrvac_tuning cand[12];
+  amrvac_tuning cand[8];
   int nc = 0;
-  for (int faces = 0; faces <= (pairs ? 1 : 0); faces++)
-    for (int ctas : {0, 1})
-      for (int order : {0, 1})
-        for (int dyn : {0, 1})
-          if (faces == 0 || ctas == 0) cand[nc++] = amrvac_tuning{ctas, order, dyn, faces, 0.0};
+  for (int ctas : {0, 1})
+    for (int order : {0, 1})
+      for (int dyn : {0, 1}) cand[nc++] = amrvac_tuning{ctas, order, dyn, 0, 0.0};
   amrvac_tuning win{0, 0, 0, 0, 1e300};
   for (int c = 0; c < nc && !st; c++) {
     st = amrvac_set_tuning(s, &cand[c]);

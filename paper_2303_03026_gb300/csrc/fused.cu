@@ -37,7 +37,13 @@ template <class T, int DIM> static int by_limiter(amrvac_state* s, int k, int ep
     case AMRVAC_LIM_VANLEER: return launch_fused_l<T, DIM, AMRVAC_LIM_VANLEER>(s, k, epilogue, g);
     case AMRVAC_LIM_KOREN: return launch_fused_l<T, DIM, AMRVAC_LIM_KOREN>(s, k, epilogue, g);
   }
-  // the other limiters share one instantiation with a runtime limiter
+  // superbee, woodward and mcbeta share one instantiation, in FP32 albada, cada3
+  // and venk another (in double all six the first)
+  if constexpr (sizeof(T) == 4) {
+    const int l = s->grp_lim[g];
+    if (l == AMRVAC_LIM_ALBADA || l == AMRVAC_LIM_CADA3 || l == AMRVAC_LIM_VENK)
+      return launch_fused_l<T, DIM, -3>(s, k, epilogue, g);
+  }
   return launch_fused_l<T, DIM, -1>(s, k, epilogue, g);
 }
 

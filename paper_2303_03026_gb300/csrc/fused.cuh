@@ -1,5 +1,6 @@
 // Fused persistent stage kernels for 16x16x16 (3D, here) and 16x16 (2D,
-// fused2d.cuh) blocks.
+// fused2d.cuh) blocks: double, and FP32 with the five-point limiters (FP32 with
+// two ghost layers: fused_f2.cuh).
 //
 // One CTA of 272 threads owns one block at a time and loops over the work
 // list (grid = resident CTAs).  Thread (x, y) < 256 owns a column of the block;
@@ -51,8 +52,7 @@ constexpr int FT = FB * FB + FB;
 // row r, lane 16 + r the y faces of column r, one flux evaluation for both.
 // With the refined approximations of fp64.cuh for division and square root: a
 // step of the 3D AMR blast in double (6.0 M cells) 85.6 -> 42.0 ms, of the 1024^2
-// vortex with koren 10.3 -> 5.3 ms.  float keeps one slope per face: there the
-// exchange costs more issue slots than the slopes it saves.
+// vortex with koren 10.3 -> 5.3 ms. 
 template <class T, int LIM> constexpr bool share_slopes() { return sizeof(T) == 8 && LIM != -2; }
 template <class T, int LIM> constexpr int fused_threads() {
   return share_slopes<T, LIM>() ? FB * FB + 2 * FB : FT;
@@ -70,24 +70,20 @@ __device__ __forceinline__ int fused_row(int warp, int lane) {
   return (warp & 3) + (warp >> 2) * 8 + (lane >> 4) * 4;
 }
 
-// DEEP: the one-CTA-per-SM layout (face pairs), with room for a 6-plane ring
-// (planes land one iteration before they are converted) and three U0 slots.
 // G: ghost layers; a plane is (16 + 2G)^2 (row stride 20 or 22) and the ring
 // holds the 2G planes of a z stencil
-template <class T, int DIM, bool DEEP = false, int G = NG> struct FusedSmem {
-  static_assert(!DEEP || G == NG, "the deep ring takes two ghost layers");
+template <class T, int DIM, int G = NG> struct FusedSmem {
   static constexpr int PW = FB + 2 * G;
-  static constexpr int NSLOT = DIM == 3 ? (DEEP ? 6 : 2 * G) : 1;
-  static constexpr int NU0 = DEEP ? 3 : 1;
+  static constexpr int NSLOT = DIM == 3 ? 2 * G : 1;
   T plane[NSLOT][NV][PW][PW];
   // face fluxes of the current plane, double-buffered by plane parity so that
   // one barrier per plane separates writers and readers
   T fx[2][NV][FB][FXW];       // x faces: column i = face i - 1/2, i = 0..16
   T fy[2][NV][FB + 1][FXW];   // y faces: row j = face j - 1/2
-  // float path: U0 of the owners' cells of the current plane (and, DEEP, of
-  // the next two), copied in ahead of the update (the fp64 path reads U0
-  // directly: a double slot would not fit beside its planes)
-  T u0[NU0][sizeof(T) == 4 ? NV : 1][FB * FB];
+  // float path: U0 of the owners' cells of the current plane, copied in ahead
+  // of the update (the fp64 path reads U0 directly: a double slot would not fit
+  // beside its planes)
+  T u0[sizeof(T) == 4 ? NV : 1][FB * FB];
   double red[8][NPART];
   int next;
 };
@@ -206,14 +202,6 @@ __device__ __forceinline__ void keep_face_flux(const DevMesh& M, int code, int i
   for (int v = 0; v < NV; v++) reg[(size_t)v * M.farea] = f[v];
 }
 
-// the instantiations that can compute the x and y faces of a cell together in
-// the two float2 lanes (stencil_flux_xy): FP32 vanleer + HLLD, lean.  16% fewer
-// instructions, but ~160 registers, hence one CTA per SM; a tuning choice
-// (amrvac_tuning.faces)
-template <class T, int LIM, int FLUX, bool FULL> constexpr bool xy_pair_ok() {
-  return sizeof(T) == 4 && LIM == AMRVAC_LIM_VANLEER && FLUX == AMRVAC_FLUX_HLLD && !FULL;
-}
-
 // Riemann flux of a face (local frame of direction D) from its two limited
 // states, first order (the cell values cl(v), cr(v)) where one is not positive
 template <class T, int D, int FLUX, class CL, class CR>
@@ -235,7 +223,7 @@ template <class T, int D, int FLUX, class Acc>
 __device__ __forceinline__ void stencil_flux5(Acc S, int lim, T lam, int glm,
                                               const FaceConst<T>& fc, T* f) {
   if constexpr (sizeof(T) == 4) {
-    stencil_flux5_f2<D, FLUX>(S, lim, lam, glm, fc.g, fc.ch, f);
+    stencil_flux5_f2<D, FLUX>(S, lim, lam, FaceConst2{fc.g, fc.ig1, fc.ch, fc.hich, glm}, f);
   } else {
     T wl[NV], wr[NV];
 #pragma unroll
@@ -456,21 +444,18 @@ __global__ void __launch_bounds__(256)
 // mirrored reads of symmetric walls are compiled in (they are runtime-uniform
 // branches that still cost the hot loop registers and scheduling freedom, so
 // the lean instantiation runs otherwise)
-// PAIR: the x and y faces of a thread's cell share the float2 lanes (one CTA
-// per SM: no minimum-occupancy register cap)
 // LIM -2: the five-point limiters (runtime limiter, three ghost layers: a
 // 6-plane ring of 22 x 22 planes and 192 halo cells a plane, one CTA per SM)
-template <class T, int DIM, int LIM, int FLUX, bool FULL, bool PAIR>
-__global__ void __launch_bounds__(fused_threads<T, LIM>(), sizeof(T) == 4 && !PAIR && LIM != -2 ? 2 : 1)
+template <class T, int DIM, int LIM, int FLUX, bool FULL>
+__global__ void __launch_bounds__(fused_threads<T, LIM>(), 1)
     k_fused(DevMesh M, const T* U0, const T* __restrict__ Uk, const T* U2, T* out, T* out2,
             const int* __restrict__ work, int nwork, const T* __restrict__ gslab,
             int* __restrict__ counter, StageParams sp) {
   extern __shared__ __align__(16) unsigned char smraw[];
   static_assert(DIM == 3, "16x16 blocks in 2D use k_fused2d");
-  // the face-pair kernel (one CTA per SM) also takes the deep ring
-  constexpr bool DEEP = PAIR;
+  static_assert(sizeof(T) == 8 || LIM == -2, "FP32 with two ghost layers: k_fused_f2");
   constexpr int G = tile_ghosts(LIM);
-  using Smem = FusedSmem<T, DIM, DEEP, G>;
+  using Smem = FusedSmem<T, DIM, G>;
   Smem& S = *reinterpret_cast<Smem*>(smraw);
   constexpr int NZ = DIM == 3 ? FB : 1;
   constexpr int NSLOT = Smem::NSLOT;
@@ -482,8 +467,6 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), sizeof(T) == 4 && !PA
   const bool ff = sp.pressure_ff != 0;
   constexpr int NT2 = DIM == 3 ? FB : 1;          // second tangential extent of a face
   constexpr int SLAB_FACE = NV * G * FB * NT2;    // one face: [v][layer][t2][t1]
-  static_assert(!PAIR || xy_pair_ok<T, LIM, FLUX, FULL>(), "face pairs: FP32 vanleer + HLLD");
-  constexpr bool XYPAIR = PAIR;
   constexpr bool SHARE = share_slopes<T, LIM>();
 
   const bool owner = tid < FB * FB;
@@ -675,12 +658,6 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), sizeof(T) == 4 && !PA
             sp.glm, fc, f);
 #pragma unroll
         for (int v = 0; v < NV; v++) zhi[v] = hi[v];
-      } else if constexpr (G == NG) {
-        int s0 = zslot(zc, -2), s1 = zslot(zc, -1), s2 = zslot(zc, 0), s3 = zslot(zc, 1);
-        auto acc = [&](int v, int t) -> T {
-          return zcell(t == 0 ? s0 : (t == 1 ? s1 : (t == 2 ? s2 : s3)), v);
-        };
-        stencil_flux_f2<2, LIM, FLUX>(acc, sp.glm, g, ch, f, sp.limiter);
       } else {
         // planes zc-3 .. zc+2 (the ring holds exactly these six)
         int sl6[6];
@@ -697,13 +674,12 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), sizeof(T) == 4 && !PA
     // ahead of the update; read back by the same thread only)
     auto issue_u0 = [&](int pz) {
       const T* src = U0 + (size_t)b * ncell + (pz * FB + y) * FB + x;
-      T* dst = &S.u0[pz % Smem::NU0][0][tid];
+      T* dst = &S.u0[0][tid];
 #pragma unroll
       for (int v = 0; v < NV; v++) cp_async_elem_after_reads(dst + v * FB * FB, src + v * vs);
     };
 
     T fzp[NV];
-    if (DEEP && pre0) issue_u0(0);
     for (int pz = -G; pz < G; pz++) issue_plane(pz);
     cp_async_wait_all();
     for (int pz = -G; pz < G; pz++) convert_plane(pz);
@@ -723,12 +699,6 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), sizeof(T) == 4 && !PA
     __syncthreads();  // the halo copies of planes 0 and 1 are visible
     convert_halo(0);
     __syncthreads();  // plane 0 with its halo in primitives
-    if constexpr (DEEP) {
-      // one plane ahead of the loop: plane 2 and U0 of plane 1 in flight
-      if (pre0) issue_u0(1);
-      issue_plane(2);
-    }
-
 
     // One barrier per plane.  Iteration z: issue the copies of U0 of plane z
     // (stages k > 0) and of plane z+G into the slot of plane z-G (its last
@@ -739,19 +709,10 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), sizeof(T) == 4 && !PA
     // face z+1/2 (planes z+1-G .. z+G); barrier; update of plane z.  The buffer of parity z is rewritten at
     // iteration z+2, after the barrier of iteration z+1, which every thread
     // passes only after its update of plane z.
-    // DEEP: the same with the copies one iteration earlier: iteration z issues
-    // plane z+3 and U0 of plane z+2 into a 6-plane ring and three U0 slots and
-    // waits only for the group of the previous iteration (plane z+2, U0 z+1).
 #pragma unroll 1
     for (int z = 0; z < NZ; z++) {
-      if constexpr (DEEP) {
-        if (pre0 && z + 2 < NZ) issue_u0(z + 2);
-        if (z + 3 <= NZ + 1) issue_plane(z + 3);  // commits one group
-        else cp_async_commit();                   // an empty group keeps the count
-      } else {
-        if (pre0) issue_u0(z);
-        issue_plane(z + G);  // commits this thread's copies as one group
-      }
+      if (pre0) issue_u0(z);
+      issue_plane(z + G);  // commits this thread's copies as one group
       const int sl = z % NSLOT, fb = z & 1;
       if constexpr (SHARE) {
         shared_slope_xy<T, LIM, FLUX, G, PW>(
@@ -768,60 +729,26 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), sizeof(T) == 4 && !PA
         T f[NV];
         auto ax = [&](int v, int t) -> T { return S.plane[sl][v][fxr + G][fxc + t]; };
         auto ay = [&](int v, int t) -> T { return S.plane[sl][v][fyr + t][fyc + G]; };
-        if constexpr (G == NG5) {
-          // five-point limiters: six-cell stencils
-          stencil_flux5<T, 0, FLUX>(ax, sp.limiter, lam[0], sp.glm, fc, f);
+        stencil_flux5<T, 0, FLUX>(ax, sp.limiter, lam[0], sp.glm, fc, f);
 #pragma unroll
-          for (int v = 0; v < NV; v++) S.fx[fb][v][fxr][fxc] = f[v];
-          if (FULL && sp.reflux) {
-            const int face = owner ? (x == 0 ? 0 : -1) : 1;
-            if (face >= 0 && nb[face] <= -3) keep_face_flux(M, nb[face], z * FB + fxr, f);
-          }
-          stencil_flux5<T, 1, FLUX>(ay, sp.limiter, lam[1], sp.glm, fc, f);
+        for (int v = 0; v < NV; v++) S.fx[fb][v][fxr][fxc] = f[v];
+        if (FULL && sp.reflux) {
+          const int face = owner ? (x == 0 ? 0 : -1) : 1;
+          if (face >= 0 && nb[face] <= -3) keep_face_flux(M, nb[face], z * FB + fxr, f);
+        }
+        stencil_flux5<T, 1, FLUX>(ay, sp.limiter, lam[1], sp.glm, fc, f);
 #pragma unroll
-          for (int v = 0; v < NV; v++) S.fy[fb][v][fyr][fyc] = f[v];
-          if (FULL && sp.reflux) {
-            const int face = owner ? (y == 0 ? 2 : -1) : 3;
-            if (face >= 0 && nb[face] <= -3) keep_face_flux(M, nb[face], z * FB + fyc, f);
-          }
-        } else if constexpr (XYPAIR) {
-          // both faces at once, one per float2 lane
-          T f2[NV];
-          stencil_flux_xy(ax, ay, sp.glm, g, ch, f, f2);
-#pragma unroll
-          for (int v = 0; v < NV; v++) {
-            S.fx[fb][v][fxr][fxc] = f[v];
-            S.fy[fb][v][fyr][fyc] = f2[v];
-          }
-          if (FULL && sp.reflux) {
-            const int face = owner ? (x == 0 ? 0 : -1) : 1;
-            if (face >= 0 && nb[face] <= -3) keep_face_flux(M, nb[face], z * FB + fxr, f);
-            const int facey = owner ? (y == 0 ? 2 : -1) : 3;
-            if (facey >= 0 && nb[facey] <= -3) keep_face_flux(M, nb[facey], z * FB + fyc, f2);
-          }
-        } else {
-          stencil_flux_f2<0, LIM, FLUX>(ax, sp.glm, g, ch, f, sp.limiter);
-#pragma unroll
-          for (int v = 0; v < NV; v++) S.fx[fb][v][fxr][fxc] = f[v];
-          if (FULL && sp.reflux) {  // x faces on the block boundary: face 0 (owners x = 0), 1 (helpers)
-            const int face = owner ? (x == 0 ? 0 : -1) : 1;
-            if (face >= 0 && nb[face] <= -3) keep_face_flux(M, nb[face], z * FB + fxr, f);
-          }
-          stencil_flux_f2<1, LIM, FLUX>(ay, sp.glm, g, ch, f, sp.limiter);
-#pragma unroll
-          for (int v = 0; v < NV; v++) S.fy[fb][v][fyr][fyc] = f[v];
-          if (FULL && sp.reflux) {  // y faces on the block boundary: face 2 (owners y = 0), 3 (helpers)
-            const int face = owner ? (y == 0 ? 2 : -1) : 3;
-            if (face >= 0 && nb[face] <= -3) keep_face_flux(M, nb[face], z * FB + fyc, f);
-          }
+        for (int v = 0; v < NV; v++) S.fy[fb][v][fyr][fyc] = f[v];
+        if (FULL && sp.reflux) {
+          const int face = owner ? (y == 0 ? 2 : -1) : 3;
+          if (face >= 0 && nb[face] <= -3) keep_face_flux(M, nb[face], z * FB + fyc, f);
         }
       }
       // owners: own cell of plane z+G -> primitives (needed by the z face
       // below); owners 256-NH..255 also a halo cell of plane z+1, whose copies
       // owners 0..NH-1 waited for before the previous barrier (needed next
       // iteration)
-      if constexpr (DEEP) asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-      else cp_async_wait_all();
+      cp_async_wait_all();
       convert_plane(z + G);
       if (z + 1 < NZ) convert_halo(z + 1);
       // float path: the stage input of the own cell, loaded before the z face
@@ -851,7 +778,7 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), sizeof(T) == 4 && !PA
         T ut = uk - dt * acc;
         if (v == 8) ut = ut * damp;
         un[v] = sp.plain ? ut
-                         : ca * (PRE0 ? S.u0[z % Smem::NU0][v][tid] : U0[at]) +
+                         : ca * (PRE0 ? S.u0[v][tid] : U0[at]) +
                                cb * ut;
         if (FULL && sp.has2) {
           // SSPRK(5,4) stage 3: w = a2 U2 + b2 (Uk + c2 dt L); U2 is out's
@@ -875,26 +802,40 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), sizeof(T) == 4 && !PA
 }  // namespace amrvac
 
 #include "fused2d.cuh"
+#include "fused_f2.cuh"
 
 namespace amrvac {
 
 // ---------------------------------------------------------------- launcher
 
-// the kernel of a dimension (the other one is not instantiated)
-template <class T, int DIM, int LIM, int FLUX, bool FULL, bool PAIR> constexpr auto fused_kernel() {
-  if constexpr (DIM == 3) return &k_fused<T, 3, LIM, FLUX, FULL, PAIR>;
-  else return &k_fused2d<T, LIM, FLUX, FULL, PAIR>;
-}
+// the kernel of a dimension and precision (the others are not instantiated), its
+// threads and shared memory
+template <class T, int DIM, int LIM, int FLUX, bool FULL> struct FusedKernel {
+  static constexpr bool F2 = sizeof(T) == 4 && LIM != -2;
+  static constexpr int threads = F2 ? F2_T : fused_threads<T, LIM>();
+  static constexpr auto kernel() {
+    if constexpr (F2 && DIM == 3) return &k_fused_f2<LIM, FLUX, FULL>;
+    else if constexpr (F2) return &k_fused2d_f2<LIM, FLUX, FULL>;
+    else if constexpr (DIM == 3) return &k_fused<T, 3, LIM, FLUX, FULL>;
+    else return &k_fused2d<T, LIM, FLUX, FULL>;
+  }
+  static constexpr int smem() {
+    if constexpr (F2 && DIM == 3) return (int)sizeof(FusedF2Smem);
+    else if constexpr (F2) return (int)sizeof(Fused2dF2Smem);
+    else if constexpr (DIM == 3) return (int)sizeof(FusedSmem<T, 3, tile_ghosts(LIM)>);
+    else return (int)sizeof(Fused2dSmem<T, tile_ghosts(LIM)>);
+  }
+};
 
-template <class T, int DIM, int LIM, int FLUX, bool FULL, bool PAIR = false>
+template <class T, int DIM, int LIM, int FLUX, bool FULL>
 static int launch_one(amrvac_state* s, const T* U0, const T* Uk, const T* U2, T* out, T* out2,
                       const int* work, int nwork, int* counter, StageParams sp) {
   static_assert(DIM == 2 || LIM != -2 || sizeof(T) == 4,
                 "five-point limiters in 3D: FP32 bulk only (a double 6-plane ring does not fit)");
-  const auto kern = fused_kernel<T, DIM, LIM, FLUX, FULL, PAIR>();
-  const int smem = DIM == 3 ? (int)sizeof(FusedSmem<T, 3, PAIR, tile_ghosts(LIM)>)
-                            : (int)sizeof(Fused2dSmem<T, tile_ghosts(LIM)>);
-  constexpr int NT = fused_threads<T, LIM>();
+  using K = FusedKernel<T, DIM, LIM, FLUX, FULL>;
+  const auto kern = K::kernel();
+  constexpr int NT = K::threads;
+  const int smem = K::smem();
   static int nsm = 0, per_sm = 0;  // per instantiation, this device
   if (nsm == 0) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
@@ -959,13 +900,6 @@ int launch_fused_l(amrvac_state* s, int k, int epilogue, int g) {
   const bool full = sp.has2 || sp.reflux || wall;
   const int flux = s->grp_flux[g];
   int m;
-  if constexpr (xy_pair_ok<T, LIM, AMRVAC_FLUX_HLLD, false>()) {
-    if (flux == AMRVAC_FLUX_HLLD && !full && s->tune.faces == 1)
-      return (m = launch_one<T, DIM, LIM, AMRVAC_FLUX_HLLD, false, true>(
-                  s, U0, Uk, U2, out, out2, work, nwork, counter, sp)) < 0
-                 ? -1
-                 : n + m;
-  }
   if (flux == AMRVAC_FLUX_HLLD)
     m = full ? launch_one<T, DIM, LIM, AMRVAC_FLUX_HLLD, true>(s, U0, Uk, U2, out, out2, work,
                                                                nwork, counter, sp)

@@ -50,13 +50,13 @@ template <class T, int G = NG> struct Fused2dSmem {
 };
 
 
-template <class T, int LIM, int FLUX, bool FULL, bool PAIR>
-__global__ void __launch_bounds__(fused_threads<T, LIM>(), sizeof(T) == 4 && !PAIR ? 2 : 1)
+template <class T, int LIM, int FLUX, bool FULL>
+__global__ void __launch_bounds__(fused_threads<T, LIM>(), sizeof(T) == 4 ? 2 : 1)
     k_fused2d(DevMesh M, const T* U0, const T* __restrict__ Uk, const T* U2, T* out, T* out2,
               const int* __restrict__ work, int nwork, const T* __restrict__ gslab,
               int* __restrict__ counter, StageParams sp) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  static_assert(!PAIR || xy_pair_ok<T, LIM, FLUX, FULL>(), "face pairs: FP32 vanleer + HLLD");
+  static_assert(sizeof(T) == 8 || LIM == -2, "FP32 with two ghost layers: k_fused2d_f2");
   constexpr int G = tile_ghosts(LIM);
   Fused2dSmem<T, G>& S = *reinterpret_cast<Fused2dSmem<T, G>*>(smraw);
   constexpr int SLAB_FACE = NV * G * FB;  // one face: [v][layer][t1]
@@ -228,62 +228,24 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), sizeof(T) == 4 && !PA
         T f[NV];
         auto ax = [&](int v, int t) -> T { return S.prim[v][fxr + G][fxc + t]; };
         auto ay = [&](int v, int t) -> T { return S.prim[v][fyr + t][fyc + G]; };
-        if constexpr (LIM == -2) {
-          // five-point limiters: six-cell stencils (three ghost layers)
-          const int lv = M.blk[b * 5 + 1];
-          const T lamx = (T)M.wzlam[(q * MAXLEV + lv) * 3], lamy = (T)M.wzlam[(q * MAXLEV + lv) * 3 + 1];
-          stencil_flux5<T, 0, FLUX>(ax, sp.limiter, lamx, sp.glm, fc, f);
+        // five-point limiters: six-cell stencils (three ghost layers)
+        const int lv = M.blk[b * 5 + 1];
+        const T lamx = (T)M.wzlam[(q * MAXLEV + lv) * 3], lamy = (T)M.wzlam[(q * MAXLEV + lv) * 3 + 1];
+        stencil_flux5<T, 0, FLUX>(ax, sp.limiter, lamx, sp.glm, fc, f);
 #pragma unroll
-          for (int v = 0; v < NV; v++) S.fx[v][fxr][fxc] = f[v];
-          if (FULL && sp.reflux) {
-            const int face = owner ? (x == 0 ? 0 : -1) : 1;
-            const int code = face >= 0 ? M.nbr[b * 6 + face] : 0;
-            if (code == NBR_GENERAL) keep_face_flux(M, -3 - M.gface[b * 6 + face], fxr, f);
-          }
-          stencil_flux5<T, 1, FLUX>(ay, sp.limiter, lamy, sp.glm, fc, f);
+        for (int v = 0; v < NV; v++) S.fx[v][fxr][fxc] = f[v];
+        if (FULL && sp.reflux) {
+          const int face = owner ? (x == 0 ? 0 : -1) : 1;
+          const int code = face >= 0 ? M.nbr[b * 6 + face] : 0;
+          if (code == NBR_GENERAL) keep_face_flux(M, -3 - M.gface[b * 6 + face], fxr, f);
+        }
+        stencil_flux5<T, 1, FLUX>(ay, sp.limiter, lamy, sp.glm, fc, f);
 #pragma unroll
-          for (int v = 0; v < NV; v++) S.fy[v][fyr][fyc] = f[v];
-          if (FULL && sp.reflux) {
-            const int face = owner ? (y == 0 ? 2 : -1) : 3;
-            const int code = face >= 0 ? M.nbr[b * 6 + face] : 0;
-            if (code == NBR_GENERAL) keep_face_flux(M, -3 - M.gface[b * 6 + face], fyc, f);
-          }
-        } else if constexpr (PAIR) {
-          // both faces at once, one per float2 lane
-          T f2[NV];
-          stencil_flux_xy(ax, ay, sp.glm, g, ch, f, f2);
-#pragma unroll
-          for (int v = 0; v < NV; v++) {
-            S.fx[v][fxr][fxc] = f[v];
-            S.fy[v][fyr][fyc] = f2[v];
-          }
-          if (FULL && sp.reflux) {
-            const int face = owner ? (x == 0 ? 0 : -1) : 1;
-            const int code = face >= 0 ? M.nbr[b * 6 + face] : 0;
-            if (code == NBR_GENERAL) keep_face_flux(M, -3 - M.gface[b * 6 + face], fxr, f);
-            const int facey = owner ? (y == 0 ? 2 : -1) : 3;
-            const int codey = facey >= 0 ? M.nbr[b * 6 + facey] : 0;
-            if (codey == NBR_GENERAL) keep_face_flux(M, -3 - M.gface[b * 6 + facey], fyc, f2);
-          }
-        } else {
-          stencil_flux_f2<0, LIM, FLUX>(ax, sp.glm, g, ch, f, sp.limiter);
-#pragma unroll
-          for (int v = 0; v < NV; v++) S.fx[v][fxr][fxc] = f[v];
-          if (FULL && sp.reflux) {  // block-boundary x faces: 0 (owners x = 0), 1 (helpers)
-            const int face = owner ? (x == 0 ? 0 : -1) : 1;
-            const int code = face >= 0 ? M.nbr[b * 6 + face] : 0;
-            if (code == NBR_GENERAL)
-              keep_face_flux(M, -3 - M.gface[b * 6 + face], fxr, f);
-          }
-          stencil_flux_f2<1, LIM, FLUX>(ay, sp.glm, g, ch, f, sp.limiter);
-#pragma unroll
-          for (int v = 0; v < NV; v++) S.fy[v][fyr][fyc] = f[v];
-          if (FULL && sp.reflux) {  // block-boundary y faces: 2 (owners y = 0), 3 (helpers)
-            const int face = owner ? (y == 0 ? 2 : -1) : 3;
-            const int code = face >= 0 ? M.nbr[b * 6 + face] : 0;
-            if (code == NBR_GENERAL)
-              keep_face_flux(M, -3 - M.gface[b * 6 + face], fyc, f);
-          }
+        for (int v = 0; v < NV; v++) S.fy[v][fyr][fyc] = f[v];
+        if (FULL && sp.reflux) {
+          const int face = owner ? (y == 0 ? 2 : -1) : 3;
+          const int code = face >= 0 ? M.nbr[b * 6 + face] : 0;
+          if (code == NBR_GENERAL) keep_face_flux(M, -3 - M.gface[b * 6 + face], fyc, f);
         }
       }
       __syncthreads();

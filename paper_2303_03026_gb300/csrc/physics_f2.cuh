@@ -1,12 +1,10 @@
-// FP32 face flux with the left and right states packed in float2 lanes.
-//
-// HLL and HLLD (Miyoshi & Kusano 2005) treat the two sides of a face with the
-// same formulas: conserved state, total pressure, fast speed, single-star
-// state.  Packing (left, right) into the two halves of a float2 and using the
-// packed FP32x2 instructions of sm_100+ (__ffma2_rn, __fadd2_rn, __fmul2_rn)
-// evaluates both sides with one instruction.  Formulas, region rules and
-// degeneracy threshold are those of hll_local / hlld_local in physics.cuh;
-// only the grouping of operations differs (FP32 rounding level).
+// FP32 physics with two values per float2: the packed FP32x2 instructions of
+// sm_100+ (__ffma2_rn, __fadd2_rn, __fmul2_rn) work on two primitive variables of
+// a cell (limited face states) or on the two sides of a face (Riemann flux).
+// The fused FP32 kernels are bound by instruction issue, so whatever can be
+// packed is; selects, minima, roots and reciprocals are per lane.  Formulas,
+// region rules and thresholds are those of physics.cuh; only the grouping of
+// operations differs (FP32 rounding level).
 #pragma once
 
 #include "physics.cuh"
@@ -17,12 +15,95 @@ __device__ __forceinline__ float2 sp2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-// a - b as one packed FMA with -1
+// a - b as one packed FMA with -1 (exact: one rounding)
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, sp2(-1.f), a); }
+__device__ __forceinline__ float2 neg2(float2 a) { return mul2(a, sp2(-1.f)); }
 __device__ __forceinline__ float2 rcp2(float2 a) { return make_float2(1.f / a.x, 1.f / a.y); }
 __device__ __forceinline__ float2 sqrt2(float2 a) { return make_float2(sqrtf(a.x), sqrtf(a.y)); }
+__device__ __forceinline__ float2 min2(float2 a, float2 b) {
+  return make_float2(fminf(a.x, b.x), fminf(a.y, b.y));
+}
+__device__ __forceinline__ float2 max2(float2 a, float2 b) {
+  return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y));
+}
+__device__ __forceinline__ float2 abs2(float2 a) { return make_float2(fabsf(a.x), fabsf(a.y)); }
+__device__ __forceinline__ float2 sel2(bool px, bool py, float2 a, float2 b) {
+  return make_float2(px ? a.x : b.x, py ? a.y : b.y);
+}
 
-// fast speeds of both sides; bt = B_t^2, bx2 = B_n^2
+// ---------------------------------------------------------------- limiters
+
+// parameters of the runtime symmetric limiters, slope = sgn(dp) min(beta mn,
+// c1 mx + c2 mn) with mn, mx the smaller and larger of |dm|, |dp|: superbee
+// (2, 1, 0), woodward (2, 1/2, 1/2), mcbeta (1.4, 1/2, 1/2)
+struct SymLim {
+  float beta, c1, c2;
+};
+__device__ __forceinline__ SymLim sym_lim(int lim) {
+  if (lim == AMRVAC_LIM_SUPERBEE) return {2.f, 1.f, 0.f};
+  return {lim == AMRVAC_LIM_WOODWARD ? 2.f : 1.4f, 0.5f, 0.5f};
+}
+
+// Increments of two variables with cell values b and neighbours a (i-1) and c
+// (i+1): the face values are b - lo at i-1/2 and b + hi at i+1/2, from one slope
+// evaluation.
+// LIM: MINMOD, VANLEER, KOREN; -1 the symmetric family by sl; -3 albada, cada3
+// or venk by the runtime value lim.
+template <int LIM>
+__device__ __forceinline__ void cell_increments2(float2 a, float2 b, float2 c, int lim, SymLim sl,
+                                                 float2& lo, float2& hi) {
+  const float2 dm = sub2(b, a), dp = sub2(c, b);
+  if constexpr (LIM == -3) {
+    if (lim == AMRVAC_LIM_CADA3) {
+      hi = make_float2(cada3_half(dm.x, dp.x), cada3_half(dm.y, dp.y));
+      lo = make_float2(cada3_half(dp.x, dm.x), cada3_half(dp.y, dm.y));
+      return;
+    }
+    if (lim == AMRVAC_LIM_VENK) {
+      lo = hi = make_float2(venk_increment(a.x, b.x, c.x), venk_increment(a.y, b.y, c.y));
+      return;
+    }
+  }
+  const float2 prod = mul2(dm, dp);
+  const bool px = prod.x > 0.f, py = prod.y > 0.f;
+  if constexpr (LIM == AMRVAC_LIM_KOREN) {
+    // halves: min(|dm|, |dp|, (|dm| + 2 |dp|)/6) towards i+1/2, mirrored to i-1/2
+    const float2 am = abs2(dm), ap = abs2(dp), m = min2(am, ap);
+    const float2 k6 = sp2(1.f / 6.f);
+    const float2 h = min2(m, mul2(fma2(sp2(2.f), ap, am), k6));
+    const float2 l = min2(m, mul2(fma2(sp2(2.f), am, ap), k6));
+    hi = make_float2(px ? copysignf(h.x, dp.x) : 0.f, py ? copysignf(h.y, dp.y) : 0.f);
+    lo = make_float2(px ? copysignf(l.x, dp.x) : 0.f, py ? copysignf(l.y, dp.y) : 0.f);
+  } else {
+    float2 s;
+    if constexpr (LIM == AMRVAC_LIM_VANLEER) {
+      s = mul2(prod, rcp2(sub2(c, a)));  // dm dp / (dm + dp): half the slope
+    } else if constexpr (LIM == -3) {    // albada
+      const float2 den = fma2(dm, dm, mul2(dp, dp));
+      s = mul2(mul2(prod, mul2(sp2(0.5f), add2(dm, dp))), rcp2(den));
+    } else {
+      const float2 am = abs2(dm), ap = abs2(dp);
+      const float2 mn = min2(am, ap);
+      float2 g;
+      if constexpr (LIM == AMRVAC_LIM_MINMOD) g = mul2(sp2(0.5f), mn);
+      else g = min2(mul2(sp2(0.5f * sl.beta), mn),
+                    fma2(sp2(0.5f * sl.c1), max2(am, ap), mul2(sp2(0.5f * sl.c2), mn)));
+      s = make_float2(copysignf(g.x, dp.x), copysignf(g.y, dp.y));
+    }
+    lo = hi = sel2(px, py, s, sp2(0.f));
+  }
+}
+
+// local component c of a y face -> primitive variable (normal y, tangential
+// (z, x)); an x face uses the identity
+__device__ __forceinline__ constexpr int yface_var(int c) {
+  return c == 1 ? 2 : c == 2 ? 3 : c == 3 ? 1 : c == 5 ? 6 : c == 6 ? 7 : c == 7 ? 5 : c;
+}
+
+// ---------------------------------------------------------------- Riemann
+// one face, its left and right states in the lanes
+
+// squares of the fast speeds of both sides; bt = B_t^2, bx2 = B_n^2
 __device__ __forceinline__ float2 fast2(float g, float2 rho, float2 p, float2 bt, float bx2) {
   float2 ir = rcp2(rho);
   float2 a2 = mul2(mul2(sp2(g), p), ir);
@@ -30,7 +111,7 @@ __device__ __forceinline__ float2 fast2(float g, float2 rho, float2 p, float2 bt
   float2 bb = mul2(add2(sp2(bx2), bt), ir);
   float2 dd = sub2(a2, bb);
   float2 sq = sqrt2(fma2(dd, dd, mul2(mul2(sp2(4.f), a2), bt2)));
-  return sqrt2(mul2(sp2(0.5f), add2(add2(a2, bb), sq)));
+  return mul2(sp2(0.5f), add2(add2(a2, bb), sq));
 }
 
 // local frame pairs: rho, u, v, w, p, by, bz (x = left, y = right); bx shared
@@ -75,7 +156,7 @@ __device__ __forceinline__ void hll_pair(float g, float ig1, const Side2& q, flo
   const float bx2 = bx * bx;
   float2 pt, e, bt;
   pt_e2(q, bx2, ig1, pt, e, bt);
-  float2 cf = fast2(g, q.rho, q.p, bt, bx2);
+  float2 cf = sqrt2(fast2(g, q.rho, q.p, bt, bx2));
   float sl = fminf(q.u.x - cf.x, q.u.y - cf.y);
   float sr = fmaxf(q.u.x + cf.x, q.u.y + cf.y);
   float UL[8], FL[8], UR[8], FR[8];
@@ -102,7 +183,7 @@ __device__ __forceinline__ void tvdlf_pair(float g, float ig1, const Side2& q, f
   const float bx2 = bx * bx;
   float2 pt, e, bt;
   pt_e2(q, bx2, ig1, pt, e, bt);
-  const float2 cf = fast2(g, q.rho, q.p, bt, bx2);
+  const float2 cf = sqrt2(fast2(g, q.rho, q.p, bt, bx2));
   const float cmax = fmaxf(fabsf(q.u.x) + cf.x, fabsf(q.u.y) + cf.y);
   float UL[8], FL[8], UR[8], FR[8];
   side_flux(q.rho.x, q.u.x, q.v.x, q.w.x, q.by.x, q.bz.x, bx, pt.x, e.x, UL, FL);
@@ -117,195 +198,169 @@ __device__ __forceinline__ void tvdlf_pair(float g, float ig1, const Side2& q, f
   }
 }
 
+// HLLD (MK05).  Up to the single-star states the two sides share the lanes; from
+// there on the lanes are the tangential components (v, w) and (By, Bz) of one
+// side: the degeneracy selects write that layout, so that no register has to be
+// moved to change it.
 __device__ __forceinline__ void hlld_pair(float g, float ig1, const Side2& q, float bx, float* f) {
   const float bx2 = bx * bx;
-  float2 pt, e, bt;
-  pt_e2(q, bx2, ig1, pt, e, bt);
-  float2 cf = fast2(g, q.rho, q.p, bt, bx2);
-  const float cmax = fmaxf(cf.x, cf.y);
+  const float2 bxp = sp2(bx), bx2p = sp2(bx2);
+  const float2 bt = fma2(q.bz, q.bz, mul2(q.by, q.by));
+  const float2 b2 = add2(bt, bx2p);
+  const float2 hb = mul2(b2, sp2(0.5f));
+  const float2 pt = add2(q.p, hb);
+  const float2 uu = fma2(q.w, q.w, fma2(q.v, q.v, mul2(q.u, q.u)));
+  const float2 e = fma2(q.p, sp2(ig1), fma2(mul2(sp2(0.5f), q.rho), uu, hb));
+  // fast speeds (see local_fast2); one root for both sides: the larger square
+  const float2 ir = rcp2(q.rho);
+  const float2 a2 = mul2(mul2(sp2(g), q.p), ir), bb = mul2(b2, ir);
+  const float2 dd = sub2(a2, bb);
+  const float2 rad = fma2(dd, dd, mul2(mul2(sp2(4.f), a2), mul2(bt, ir)));
+  const float2 cf2 = add2(add2(a2, bb), sqrt2(rad));
+  const float cmax = sqrtf(0.5f * fmaxf(cf2.x, cf2.y));
   const float sl = fminf(q.u.x, q.u.y) - cmax;
   const float sr = fmaxf(q.u.x, q.u.y) + cmax;
   const float2 S = make_float2(sl, sr);
   const float2 su = sub2(S, q.u);              // (S_L - u_L, S_R - u_R)
   const float2 A = mul2(su, q.rho);            // rho (S - u)
   const float iden = 1.f / (A.y - A.x);
-  const float2 Au = mul2(A, q.u);
-  const float sm = (Au.y - Au.x - pt.y + pt.x) * iden;
-  const float pts =
-      (A.y * pt.x - A.x * pt.y + q.rho.x * q.rho.y * su.y * su.x * (q.u.y - q.u.x)) * iden;
+  const float sm = ((A.y * q.u.y + pt.x) - (A.x * q.u.x + pt.y)) * iden;
+  const float pts = ((A.y * pt.x - A.x * pt.y) + A.x * A.y * (q.u.y - q.u.x)) * iden;
+  const float psm = pts * sm, sbx = sm * bx;
   // single-star states of both sides
-  const float2 ssm = sub2(S, sp2(sm));         // S - S_M
+  const float2 smp = sp2(sm);
+  const float2 ssm = sub2(S, smp);             // S - S_M
   const float2 isd = rcp2(ssm);
   const float2 rs = mul2(A, isd);
   const float2 big = mul2(A, ssm);
-  const float2 den = sub2(big, sp2(bx2));
+  const float2 den = sub2(big, bx2p);
   const float2 iden2 = rcp2(den);
-  const float2 tv = mul2(mul2(sp2(bx), sub2(sp2(sm), q.u)), iden2);
-  const float2 tb = mul2(sub2(mul2(A, su), sp2(bx2)), iden2);
-  const float2 ntv = mul2(tv, sp2(-1.f));
-  float2 vs = fma2(q.by, ntv, q.v);
-  float2 ws = fma2(q.bz, ntv, q.w);
-  float2 bys = mul2(q.by, tb);
-  float2 bzs = mul2(q.bz, tb);
+  const float2 ntv = mul2(mul2(bxp, sub2(q.u, smp)), iden2);
+  const float2 tb = mul2(sub2(mul2(A, su), bx2p), iden2);
+  const float2 vs = fma2(q.by, ntv, q.v), ws = fma2(q.bz, ntv, q.w);
+  const float2 bys = mul2(q.by, tb), bzs = mul2(q.bz, tb);
   const float eps = Num<float>::hlld_eps;
-  if (fabsf(den.x) <= eps * fmaxf(fabsf(big.x), bx2)) {
-    vs.x = q.v.x;
-    ws.x = q.w.x;
-    bys.x = q.by.x;
-    bzs.x = q.bz.x;
-  }
-  if (fabsf(den.y) <= eps * fmaxf(fabsf(big.y), bx2)) {
-    vs.y = q.v.y;
-    ws.y = q.w.y;
-    bys.y = q.by.y;
-    bzs.y = q.bz.y;
-  }
-  const float2 vb = fma2(q.w, q.bz, fma2(q.v, q.by, mul2(q.u, sp2(bx))));
-  const float2 vbs = fma2(ws, bzs, fma2(vs, bys, sp2(sm * bx)));
-  float2 t = sub2(mul2(su, e), mul2(pt, q.u));
-  t = fma2(sp2(bx), sub2(vb, vbs), add2(t, sp2(pts * sm)));
-  const float2 es = mul2(t, isd);
-  // double-star states (averages of the two sides, packed over (v, w) / (By, Bz))
-  const float2 isq = make_float2(rsqrtf(rs.x), rsqrtf(rs.y));  // 1/sqrt(rho*)
-  const float2 sqr = mul2(rs, isq);
+  const bool dl = fabsf(den.x) <= eps * fmaxf(fabsf(big.x), bx2);
+  const bool dr = fabsf(den.y) <= eps * fmaxf(fabsf(big.y), bx2);
+  const float2 VL = make_float2(dl ? q.v.x : vs.x, dl ? q.w.x : ws.x);
+  const float2 VR = make_float2(dr ? q.v.y : vs.y, dr ? q.w.y : ws.y);
+  const float2 BL = make_float2(dl ? q.by.x : bys.x, dl ? q.bz.x : bzs.x);
+  const float2 BR = make_float2(dr ? q.by.y : bys.y, dr ? q.bz.y : bzs.y);
+  const float2 vb = fma2(q.w, q.bz, fma2(q.v, q.by, mul2(q.u, bxp)));
+  const float2 vbl = mul2(VL, BL), vbr = mul2(VR, BR);
+  const float2 vbs = make_float2(sbx + (vbl.x + vbl.y), sbx + (vbr.x + vbr.y));
+  const float2 t = sub2(mul2(su, e), mul2(pt, q.u));
+  const float2 es = mul2(fma2(bxp, sub2(vb, vbs), add2(t, sp2(psm))), isd);
+  // double-star states (averages of the two sides)
+  const float isl = rsqrtf(rs.x), isr = rsqrtf(rs.y);  // 1/sqrt(rho*)
+  const float sql = rs.x * isl, sqr = rs.y * isr;
   const float abx = fabsf(bx);
-  const float ssl = sm - abx * isq.x, ssr = sm + abx * isq.y;
-  const float sb = sgnT(bx);
-  const float issum = 1.f / (sqr.x + sqr.y);
-  const float2 VL = make_float2(vs.x, ws.x), VR = make_float2(vs.y, ws.y);
-  const float2 BL = make_float2(bys.x, bzs.x), BR = make_float2(bys.y, bzs.y);
-  const float2 VSS = mul2(fma2(sub2(BR, BL), sp2(sb), fma2(sp2(sqr.y), VR, mul2(sp2(sqr.x), VL))),
-                          sp2(issum));
-  const float2 BSS = mul2(fma2(sub2(VR, VL), sp2(sqr.x * sqr.y * sb),
-                               fma2(sp2(sqr.y), BL, mul2(sp2(sqr.x), BR))),
-                          sp2(issum));
-  const float vbss = sm * bx + VSS.x * BSS.x + VSS.y * BSS.y;
-  // e** = e* -/+ sqrt(rho*) (v*.B* - v**.B**) sgn(Bx)
-  const float2 ess = fma2(make_float2(-sqr.x * sb, sqr.y * sb), sub2(vbs, sp2(vbss)), es);
+  const float ssl = sm - abx * isl, ssr = sm + abx * isr;
+  const float sb = bx == 0.f ? 0.f : copysignf(1.f, bx);
+  const float issum = 1.f / (sql + sqr);
+  const float wl = sql * issum, wr = sqr * issum;
+  const float2 wlp = sp2(wl), wrp = sp2(wr);
+  const float2 VSS = fma2(sub2(BR, BL), sp2(sb * issum), fma2(wrp, VR, mul2(wlp, VL)));
+  const float2 BSS = fma2(sub2(VR, VL), sp2(sql * wr * sb), fma2(wrp, BL, mul2(wlp, BR)));
+  const float2 vbd = mul2(VSS, BSS);
+  const float vbss = sbx + (vbd.x + vbd.y);
   // region containing x/t = 0 (same tie rules as the scalar solver)
   const bool left = sm >= 0.f;
   const bool outer = left ? (sl > 0.f) : (sr < 0.f);
   const bool single = left ? (ssl >= 0.f) : !(ssr >= 0.f);
-  float U[8], F[8];
-  side_flux(left ? q.rho.x : q.rho.y, left ? q.u.x : q.u.y, left ? q.v.x : q.v.y,
-            left ? q.w.x : q.w.y, left ? q.by.x : q.by.y, left ? q.bz.x : q.bz.y, bx,
-            left ? pt.x : pt.y, left ? e.x : e.y, U, F);
-  const float r = left ? rs.x : rs.y;
+  // the upwind side of S_M
+  const float rho = left ? q.rho.x : q.rho.y, u = left ? q.u.x : q.u.y;
+  const float pu = left ? pt.x : pt.y, eu = left ? e.x : e.y;
+  const float r = left ? rs.x : rs.y, eS = left ? es.x : es.y, vbS = left ? vbs.x : vbs.y;
+  const float vbu = left ? vb.x : vb.y, sq = left ? -sql : sqr;
   const float c1 = left ? sl : sr, c2 = left ? ssl : ssr;
-  const float US[8] = {r, r * sm, r * (left ? vs.x : vs.y), r * (left ? ws.x : ws.y),
-                       left ? es.x : es.y, bx, left ? bys.x : bys.y, left ? bzs.x : bzs.y};
-  const float USS[8] = {r, r * sm, r * VSS.x, r * VSS.y, left ? ess.x : ess.y, bx, BSS.x, BSS.y};
-#pragma unroll
-  for (int c = 0; c < 8; c += 2) {
-    const float2 Fp = make_float2(F[c], F[c + 1]);
-    const float2 Up = make_float2(U[c], U[c + 1]);
-    const float2 Sp = make_float2(US[c], US[c + 1]);
-    const float2 SSp = make_float2(USS[c], USS[c + 1]);
-    const float2 fs = fma2(sp2(c1), sub2(Sp, Up), Fp);
-    const float2 fss = fma2(sp2(c2), sub2(SSp, Sp), fs);
-    f[c] = outer ? F[c] : (single ? fs.x : fss.x);
-    f[c + 1] = outer ? F[c + 1] : (single ? fs.y : fss.y);
+  const float2 V = make_float2(left ? q.v.x : q.v.y, left ? q.w.x : q.w.y);
+  const float2 B = make_float2(left ? q.by.x : q.by.y, left ? q.bz.x : q.bz.y);
+  const float2 VS = make_float2(left ? VL.x : VR.x, left ? VL.y : VR.y);
+  const float2 BS = make_float2(left ? BL.x : BR.x, left ? BL.y : BR.y);
+  // F + c1 (U* - U) + c2 (U** - U*); the double star keeps rho* and S_M, and
+  // e** - e* = -/+ sqrt(rho*) (v*.B* - v**.B**) sgn(Bx)
+  const float mu = rho * u;
+  const float F1 = mu * u + (pu - bx2), F4 = (eu + pu) * u - bx * vbu;
+  const float2 F23 = sub2(mul2(sp2(mu), V), mul2(bxp, B));
+  const float2 F67 = sub2(mul2(sp2(u), B), mul2(bxp, V));
+  const float2 c1p = sp2(c1);
+  const float2 fs23 = fma2(c1p, sub2(mul2(sp2(r), VS), mul2(sp2(rho), V)), F23);
+  const float2 fs67 = fma2(c1p, sub2(BS, B), F67);
+  const float fs4 = F4 + c1 * (eS - eu);
+  const float fss4 = fs4 + c2 * ((sq * sb) * (vbS - vbss));
+  const float2 fss23 = fma2(sp2(c2 * r), sub2(VSS, VS), fs23);
+  const float2 fss67 = fma2(sp2(c2), sub2(BSS, BS), fs67);
+  f[0] = outer ? mu : mu + c1 * (r - rho);
+  f[1] = outer ? F1 : F1 + c1 * (r * sm - mu);
+  f[2] = outer ? F23.x : (single ? fs23.x : fss23.x);
+  f[3] = outer ? F23.y : (single ? fs23.y : fss23.y);
+  f[4] = outer ? F4 : (single ? fs4 : fss4);
+  f[5] = 0.f;
+  f[6] = outer ? F67.x : (single ? fs67.x : fss67.x);
+  f[7] = outer ? F67.y : (single ? fs67.y : fss67.y);
+}
+
+// constants of a face flux: gamma, 1/(gamma - 1), c_h, 1/(2 c_h)
+struct FaceConst2 {
+  float g, ig1, ch, hich;
+  int glm;
+};
+__device__ __forceinline__ FaceConst2 face_const2(float g, float ch, int glm) {
+  return {g, 1.f / (g - 1.f), ch, 0.5f / ch, glm};
+}
+
+// glm solve and Riemann flux along D from the face states w[v] = (left, right)
+template <int D, int FLUX>
+__device__ __forceinline__ void face_flux2(const float2* w, const FaceConst2& fc, float* f) {
+  constexpr int t1 = D == 2 ? 0 : D + 1, t2 = D == 0 ? 2 : D - 1;
+  const float bnl = w[5 + D].x, bnr = w[5 + D].y;
+  float bns = 0.5f * (bnl + bnr), psis = 0.f, fpsi = 0.f;
+  if (fc.glm) {
+    bns = fmaf(w[8].x - w[8].y, fc.hich, bns);
+    psis = fmaf(bnl - bnr, 0.5f * fc.ch, 0.5f * (w[8].x + w[8].y));
+    fpsi = fc.ch * fc.ch * bns;
   }
-}
-
-// vanleer face values of the face between cells b and c from the stencil
-// (a, b, c, e): x = left state (from cell b), y = right state (from cell c)
-__device__ __forceinline__ float2 vanleer_pair(float a, float b, float c, float e) {
-  const float2 X = make_float2(b, c);
-  const float2 dm = sub2(X, make_float2(a, b));
-  const float2 dp = sub2(make_float2(c, e), X);
-  const float2 prod = mul2(dm, dp);
-  const float2 s = mul2(mul2(sp2(2.f), prod), rcp2(add2(dm, dp)));
-  const float2 v = fma2(make_float2(0.5f, -0.5f), s, X);
-  return make_float2(prod.x > 0.f ? v.x : b, prod.y > 0.f ? v.y : c);
-}
-
-// The symmetric limiters of the runtime-limiter instantiation, both face
-// states of the face between cells b and c at once (x: left state from cell b
-// with stencil (a, b, c); y: right state from cell c with (b, c, e)); slope =
-// sgn(dp) G(|dm|, |dp|) where dm dp > 0, else first order.
-//   monotonized central family: G = min(beta |dm|, (|dm| + |dp|)/2, beta |dp|)
-//     (woodward beta = 2, mcbeta beta = 1.4)
-//   superbee: G = max(min(2 |dm|, |dp|), min(|dm|, 2 |dp|))
-//   albada:   slope = dm dp (dm + dp) / (dm^2 + dp^2)
-template <int KIND>  // 0 monotonized central (beta), 1 superbee, 2 albada
-__device__ __forceinline__ float2 sym_pair(float a, float b, float c, float e, float beta) {
-  const float2 X = make_float2(b, c);
-  const float2 dm = sub2(X, make_float2(a, b));
-  const float2 dp = sub2(make_float2(c, e), X);
-  const float2 prod = mul2(dm, dp);
-  float2 s;
-  if (KIND == 2) {
-    const float2 den = fma2(dm, dm, mul2(dp, dp));
-    s = mul2(mul2(prod, add2(dm, dp)), rcp2(den));
+  const Side2 q = {w[0], w[1 + D], w[1 + t1], w[1 + t2], w[4], w[5 + t1], w[5 + t2]};
+  float fl[8];
+  if constexpr (FLUX == AMRVAC_FLUX_HLL) {
+    hll_pair(fc.g, fc.ig1, q, bns, fl);
+  } else if constexpr (FLUX == AMRVAC_FLUX_HLLD) {
+    hlld_pair(fc.g, fc.ig1, q, bns, fl);
+  } else if constexpr (FLUX == AMRVAC_FLUX_TVDLF) {
+    tvdlf_pair(fc.g, fc.ig1, q, bns, fl);
   } else {
-    const float am0 = fabsf(dm.x), ap0 = fabsf(dp.x), am1 = fabsf(dm.y), ap1 = fabsf(dp.y);
-    float g0, g1;
-    if (KIND == 1) {
-      g0 = fmaxf(fminf(2.f * am0, ap0), fminf(am0, 2.f * ap0));
-      g1 = fmaxf(fminf(2.f * am1, ap1), fminf(am1, 2.f * ap1));
-    } else {
-      g0 = fminf(fminf(beta * am0, 0.5f * (am0 + ap0)), beta * ap0);
-      g1 = fminf(fminf(beta * am1, 0.5f * (am1 + ap1)), beta * ap1);
-    }
-    s = make_float2(copysignf(g0, dp.x), copysignf(g1, dp.y));
+    // HLLC: the scalar three-wave solver on the unpacked face states
+    const float ql[8] = {q.rho.x, q.u.x, q.v.x, q.w.x, q.p.x, bns, q.by.x, q.bz.x};
+    const float qr[8] = {q.rho.y, q.u.y, q.v.y, q.w.y, q.p.y, bns, q.by.y, q.bz.y};
+    hllc_local<float>(fc.g, fc.ig1, ql, qr, bns, fl);
   }
-  const float2 v = fma2(make_float2(0.5f, -0.5f), s, X);
-  return make_float2(prod.x > 0.f ? v.x : b, prod.y > 0.f ? v.y : c);
+  f[0] = fl[0];
+  f[1 + D] = fl[1];
+  f[1 + t1] = fl[2];
+  f[1 + t2] = fl[3];
+  f[4] = fl[4];
+  f[5 + D] = psis;
+  f[5 + t1] = fl[6];
+  f[5 + t2] = fl[7];
+  f[8] = fpsi;
 }
 
-// cada3 (see cada3_half) for both face states of the face between cells b and
-// c: x = left state from cell b with (dm, dp) = (b - a, c - b); y = right state
-// from cell c, the mirrored rule with (dm, dp) = (c - e, b - c)
-__device__ __forceinline__ float2 cada3_pair(float a, float b, float c, float e) {
-  const float2 X = make_float2(b, c);
-  const float2 dm = sub2(X, make_float2(a, e));
-  const float2 dp = sub2(make_float2(c, b), X);
-  const float s0 = sgnT(dp.x), s1 = sgnT(dp.y);
-  const float2 A = make_float2(fabsf(dp.x), fabsf(dp.y));
-  const float2 t = mul2(make_float2(s0, s1), dm);
-  const float2 p3 = mul2(fma2(sp2(2.f), A, t), sp2(1.f / 3.f));
-  const float2 tt = mul2(sp2(2.f), t), ca = mul2(sp2(1.6f), A), ht = mul2(sp2(-0.5f), t);
-  const float i0 = fminf(fminf(tt.x, p3.x), ca.x), i1 = fminf(fminf(tt.y, p3.y), ca.y);
-  const float pa0 = fmaxf(0.f, fminf(p3.x, fmaxf(ht.x, i0)));
-  const float pa1 = fmaxf(0.f, fminf(p3.y, fmaxf(ht.y, i1)));
-  return fma2(mul2(sp2(0.5f), make_float2(s0, s1)), make_float2(pa0, pa1), X);
+// a face state is not positive (or NaN): the face takes the cell values
+__device__ __forceinline__ bool not_positive2(const float2* w) {
+  return !(w[0].x > 0.f) || !(w[4].x > 0.f) || !(w[0].y > 0.f) || !(w[4].y > 0.f);
 }
 
-// ---------------------------------------------------------------------------
-// Two faces per thread, one per float2 lane: lane x the x face of a cell and
-// lane y its y face.  Each lane loads the stencil of its own face already in
-// the face's local frame (normal velocity and field first), so the packed
-// operands need no register shuffling, and the per-face work of HLLD (wave
-// speeds, double-star states, fan region) runs once for both faces.  The
-// formulas are those of hlld_pair / hlld_local (MK05 with the degeneracy
-// threshold, sgn(0) = 0 and the same region ties); only the packing differs.
+// ---------------------------------------------------------------- Riemann, two faces
+// lane x the x face of a cell and lane y its y face, each in its local frame
+// (normal velocity and field first): every operation is packed, and the solver's
+// latency is paid once for both faces
 
-__device__ __forceinline__ float2 min2(float2 a, float2 b) {
-  return make_float2(fminf(a.x, b.x), fminf(a.y, b.y));
-}
-__device__ __forceinline__ float2 max2(float2 a, float2 b) {
-  return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y));
-}
-__device__ __forceinline__ float2 abs2(float2 a) { return make_float2(fabsf(a.x), fabsf(a.y)); }
-__device__ __forceinline__ float2 sel2(bool px, bool py, float2 a, float2 b) {
-  return make_float2(px ? a.x : b.x, py ? a.y : b.y);
-}
-
-// primitive face states of both faces in their local frames
 struct Prim2 {
   float2 rho, u, v, w, p, by, bz;
 };
 
-// van Leer slopes of two cells at once from their one-sided differences:
-// 2 dm dp / (dm + dp) where dm dp > 0, else 0
-__device__ __forceinline__ float2 vl_slope2(float2 dm, float2 dp) {
-  const float2 prod = mul2(dm, dp);
-  const float2 s = mul2(mul2(sp2(2.f), prod), rcp2(add2(dm, dp)));
-  return make_float2(prod.x > 0.f ? s.x : 0.f, prod.y > 0.f ? s.y : 0.f);
-}
-
-// fast speeds (cancellation-free form) from rho, p, B_t^2 and B_n^2
+// squares of the fast speeds (cancellation-free form) from rho, p, B_t^2, B_n^2
 __device__ __forceinline__ float2 fast_xy(float g, float2 rho, float2 p, float2 bt, float2 bx2) {
   const float2 ir = rcp2(rho);
   const float2 a2 = mul2(mul2(sp2(g), p), ir);
@@ -313,17 +368,134 @@ __device__ __forceinline__ float2 fast_xy(float g, float2 rho, float2 p, float2 
   const float2 bb = mul2(add2(bx2, bt), ir);
   const float2 dd = sub2(a2, bb);
   const float2 sq = sqrt2(fma2(dd, dd, mul2(mul2(sp2(4.f), a2), bt2)));
-  return sqrt2(mul2(sp2(0.5f), add2(add2(a2, bb), sq)));
+  return mul2(sp2(0.5f), add2(add2(a2, bb), sq));
 }
 
-// single-star state of one side (MK05 eqs. 43-48) for both faces
+// B_t^2, total pressure and total energy
+__device__ __forceinline__ void pt_e_xy(const Prim2& q, float2 bx2, float ig1, float2& bt,
+                                      float2& pt, float2& e) {
+  bt = fma2(q.bz, q.bz, mul2(q.by, q.by));
+  const float2 b2 = add2(bt, bx2);
+  pt = fma2(b2, sp2(0.5f), q.p);
+  const float2 uu = fma2(q.w, q.w, fma2(q.v, q.v, mul2(q.u, q.u)));
+  e = fma2(q.p, sp2(ig1), fma2(mul2(sp2(0.5f), q.rho), uu, mul2(sp2(0.5f), b2)));
+}
+
+// conserved state and physical flux (component 5, the normal field, is left to
+// the glm solve)
+__device__ __forceinline__ void state_flux2(const Prim2& q, float2 bx, float2 bx2, float2 pt,
+                                            float2 e, float2* U, float2* F) {
+  const float2 mu = mul2(q.rho, q.u), nbx = neg2(bx);
+  const float2 vb = fma2(q.w, q.bz, fma2(q.v, q.by, mul2(q.u, bx)));
+  U[0] = q.rho;
+  U[1] = mu;
+  U[2] = mul2(q.rho, q.v);
+  U[3] = mul2(q.rho, q.w);
+  U[4] = e;
+  U[5] = bx;
+  U[6] = q.by;
+  U[7] = q.bz;
+  F[0] = mu;
+  F[1] = fma2(mu, q.u, sub2(pt, bx2));
+  F[2] = fma2(mu, q.v, mul2(nbx, q.by));
+  F[3] = fma2(mu, q.w, mul2(nbx, q.bz));
+  F[4] = fma2(add2(e, pt), q.u, mul2(nbx, vb));
+  F[5] = sp2(0.f);
+  F[6] = fma2(q.by, q.u, mul2(nbx, q.v));
+  F[7] = fma2(q.bz, q.u, mul2(nbx, q.w));
+}
+
+// HLL and TVD Lax-Friedrichs
+template <int FLUX>
+__device__ __forceinline__ void hll2(float g, float ig1, const Prim2& L, const Prim2& R,
+                                     float2 bx, float2* f) {
+  const float2 bx2 = mul2(bx, bx);
+  float2 btL, ptL, eL, btR, ptR, eR, UL[8], FL[8], UR[8], FR[8];
+  pt_e_xy(L, bx2, ig1, btL, ptL, eL);
+  pt_e_xy(R, bx2, ig1, btR, ptR, eR);
+  const float2 cL = sqrt2(fast_xy(g, L.rho, L.p, btL, bx2));
+  const float2 cR = sqrt2(fast_xy(g, R.rho, R.p, btR, bx2));
+  state_flux2(L, bx, bx2, ptL, eL, UL, FL);
+  state_flux2(R, bx, bx2, ptR, eR, UR, FR);
+  if (FLUX == AMRVAC_FLUX_TVDLF) {
+    const float2 c = mul2(sp2(-0.5f), max2(add2(abs2(L.u), cL), add2(abs2(R.u), cR)));
+#pragma unroll
+    for (int k = 0; k < 8; k++)
+      f[k] = fma2(c, sub2(UR[k], UL[k]), mul2(sp2(0.5f), add2(FL[k], FR[k])));
+    return;
+  }
+  const float2 sl = min2(sub2(L.u, cL), sub2(R.u, cR)), sr = max2(add2(L.u, cL), add2(R.u, cR));
+  const float2 inv = rcp2(sub2(sr, sl)), nsl = neg2(sl), slsr = mul2(sl, sr);
+  const bool lx = sl.x >= 0.f, ly = sl.y >= 0.f, rx = sr.x <= 0.f, ry = sr.y <= 0.f;
+#pragma unroll
+  for (int k = 0; k < 8; k++) {
+    if (k == 5) continue;
+    const float2 t = fma2(sr, FL[k], mul2(nsl, FR[k]));
+    const float2 m = mul2(fma2(slsr, sub2(UR[k], UL[k]), t), inv);
+    f[k] = sel2(lx, ly, FL[k], sel2(rx, ry, FR[k], m));
+  }
+  f[5] = sp2(0.f);
+}
+
+// HLLC (see hllc_local)
+__device__ __forceinline__ void hllc2(float g, float ig1, const Prim2& L, const Prim2& R,
+                                      float2 bx, float2* f) {
+  const float2 bx2 = mul2(bx, bx);
+  float2 btL, ptL, eL, btR, ptR, eR, UL[8], FL[8], UR[8], FR[8];
+  pt_e_xy(L, bx2, ig1, btL, ptL, eL);
+  pt_e_xy(R, bx2, ig1, btR, ptR, eR);
+  const float2 cL = sqrt2(fast_xy(g, L.rho, L.p, btL, bx2));
+  const float2 cR = sqrt2(fast_xy(g, R.rho, R.p, btR, bx2));
+  state_flux2(L, bx, bx2, ptL, eL, UL, FL);
+  state_flux2(R, bx, bx2, ptR, eR, UR, FR);
+  const float2 sl = min2(sub2(L.u, cL), sub2(R.u, cR)), sr = max2(add2(L.u, cL), add2(R.u, cR));
+  const float2 inv = rcp2(sub2(sr, sl)), nsl = neg2(sl);
+  float2 uh[8];
+#pragma unroll
+  for (int k = 0; k < 8; k++)
+    uh[k] = mul2(add2(fma2(sr, UR[k], mul2(nsl, UL[k])), sub2(FL[k], FR[k])), inv);
+  const float2 ih = rcp2(uh[0]);
+  const float2 sm = mul2(uh[1], ih), vy = mul2(uh[2], ih), vz = mul2(uh[3], ih);
+  const float2 by = uh[6], bz = uh[7];
+  const float2 pts =
+      fma2(mul2(L.rho, sub2(sl, L.u)), sub2(sm, L.u), ptL);
+  const float2 vbs = fma2(vz, bz, fma2(vy, by, mul2(sm, bx)));
+  const bool lx = sm.x >= 0.f, ly = sm.y >= 0.f;
+  const Prim2 q = {sel2(lx, ly, L.rho, R.rho), sel2(lx, ly, L.u, R.u), sel2(lx, ly, L.v, R.v),
+                   sel2(lx, ly, L.w, R.w),     sel2(lx, ly, L.p, R.p), sel2(lx, ly, L.by, R.by),
+                   sel2(lx, ly, L.bz, R.bz)};
+  const float2 S = sel2(lx, ly, sl, sr), pt = sel2(lx, ly, ptL, ptR), e = sel2(lx, ly, eL, eR);
+  const float2 su = sub2(S, q.u), isd = rcp2(sub2(S, sm));
+  const float2 vb = fma2(q.w, q.bz, fma2(q.v, q.by, mul2(q.u, bx)));
+  const float2 nbx = neg2(bx);
+  float2 Us[8];
+  const float2 ru = mul2(q.rho, su);
+  Us[0] = mul2(ru, isd);
+  Us[1] = mul2(Us[0], sm);
+  Us[2] = mul2(fma2(ru, q.v, mul2(nbx, sub2(by, q.by))), isd);
+  Us[3] = mul2(fma2(ru, q.w, mul2(nbx, sub2(bz, q.bz))), isd);
+  Us[4] = mul2(fma2(nbx, sub2(vbs, vb), fma2(pts, sm, sub2(mul2(e, su), mul2(pt, q.u)))), isd);
+  Us[6] = by;
+  Us[7] = bz;
+  const bool olx = sl.x >= 0.f, oly = sl.y >= 0.f, orx = sr.x <= 0.f, ory = sr.y <= 0.f;
+#pragma unroll
+  for (int k = 0; k < 8; k++) {
+    if (k == 5) continue;
+    const float2 U = sel2(lx, ly, UL[k], UR[k]), F = sel2(lx, ly, FL[k], FR[k]);
+    const float2 m = fma2(S, sub2(Us[k], U), F);
+    f[k] = sel2(olx, oly, FL[k], sel2(orx, ory, FR[k], m));
+  }
+  f[5] = sp2(0.f);
+}
+
+// single-star state of one side (MK05 eqs. 43-48)
 struct Star2 {
   float2 rs, vs, ws, bys, bzs, es, vbs;
 };
 
-__device__ __forceinline__ Star2 hlld_star_xy(const Prim2& q, float2 S, float2 su, float2 A,
-                                              float2 pt, float2 e, float2 sm, float2 pts,
-                                              float2 bx, float2 bx2) {
+__device__ __forceinline__ Star2 hlld_star2(const Prim2& q, float2 S, float2 su, float2 A,
+                                            float2 pt, float2 e, float2 sm, float2 psm,
+                                            float2 sbx, float2 bx, float2 bx2) {
   Star2 r;
   const float2 ssm = sub2(S, sm);
   const float2 isd = rcp2(ssm);
@@ -331,9 +503,8 @@ __device__ __forceinline__ Star2 hlld_star_xy(const Prim2& q, float2 S, float2 s
   const float2 big = mul2(A, ssm);
   const float2 den = sub2(big, bx2);
   const float2 iden = rcp2(den);
-  const float2 tv = mul2(mul2(bx, sub2(sm, q.u)), iden);
+  const float2 ntv = mul2(mul2(bx, sub2(q.u, sm)), iden);
   const float2 tb = mul2(sub2(mul2(A, su), bx2), iden);
-  const float2 ntv = mul2(tv, sp2(-1.f));
   const float eps = Num<float>::hlld_eps;
   const bool dgx = fabsf(den.x) <= eps * fmaxf(fabsf(big.x), bx2.x);
   const bool dgy = fabsf(den.y) <= eps * fmaxf(fabsf(big.y), bx2.y);
@@ -342,80 +513,73 @@ __device__ __forceinline__ Star2 hlld_star_xy(const Prim2& q, float2 S, float2 s
   r.bys = sel2(dgx, dgy, q.by, mul2(q.by, tb));
   r.bzs = sel2(dgx, dgy, q.bz, mul2(q.bz, tb));
   const float2 vb = fma2(q.w, q.bz, fma2(q.v, q.by, mul2(q.u, bx)));
-  r.vbs = fma2(r.ws, r.bzs, fma2(r.vs, r.bys, mul2(sm, bx)));
+  r.vbs = fma2(r.ws, r.bzs, fma2(r.vs, r.bys, sbx));
   float2 t = sub2(mul2(su, e), mul2(pt, q.u));
-  t = fma2(bx, sub2(vb, r.vbs), fma2(pts, sm, t));
+  t = fma2(bx, sub2(vb, r.vbs), add2(psm, t));
   r.es = mul2(t, isd);
   return r;
 }
 
-// HLLD flux of two faces; f[c] for the local components c = 0..7 (c = 5, the
-// normal field, is left to the glm solve)
-__device__ __forceinline__ void hlld_xy(float g, float ig1, const Prim2& L, const Prim2& R,
-                                        float2 bx, float2* f) {
+// HLLD (MK05)
+__device__ __forceinline__ void hlld2(float g, float ig1, const Prim2& L, const Prim2& R,
+                                      float2 bx, float2* f) {
   const float2 bx2 = mul2(bx, bx);
-  const float2 btL = fma2(L.bz, L.bz, mul2(L.by, L.by));
-  const float2 btR = fma2(R.bz, R.bz, mul2(R.by, R.by));
-  const float2 b2L = add2(btL, bx2), b2R = add2(btR, bx2);
-  const float2 ptL = fma2(b2L, sp2(0.5f), L.p), ptR = fma2(b2R, sp2(0.5f), R.p);
-  const float2 uuL = fma2(L.w, L.w, fma2(L.v, L.v, mul2(L.u, L.u)));
-  const float2 uuR = fma2(R.w, R.w, fma2(R.v, R.v, mul2(R.u, R.u)));
-  const float2 eL = fma2(L.p, sp2(ig1), fma2(mul2(sp2(0.5f), L.rho), uuL, mul2(sp2(0.5f), b2L)));
-  const float2 eR = fma2(R.p, sp2(ig1), fma2(mul2(sp2(0.5f), R.rho), uuR, mul2(sp2(0.5f), b2R)));
-  const float2 cmax = max2(fast_xy(g, L.rho, L.p, btL, bx2), fast_xy(g, R.rho, R.p, btR, bx2));
+  float2 btL, ptL, eL, btR, ptR, eR;
+  pt_e_xy(L, bx2, ig1, btL, ptL, eL);
+  pt_e_xy(R, bx2, ig1, btR, ptR, eR);
+  // one root for both sides: the larger of the squared fast speeds
+  const float2 cmax =
+      sqrt2(max2(fast_xy(g, L.rho, L.p, btL, bx2), fast_xy(g, R.rho, R.p, btR, bx2)));
   const float2 sl = sub2(min2(L.u, R.u), cmax), sr = add2(max2(L.u, R.u), cmax);
   const float2 suL = sub2(sl, L.u), suR = sub2(sr, R.u);
   const float2 AL = mul2(suL, L.rho), AR = mul2(suR, R.rho);
   const float2 iden = rcp2(sub2(AR, AL));
   // S_M and p_T* from the HLL-averaged normal momentum (MK05 eqs. 38, 41)
   const float2 sm = mul2(sub2(fma2(AR, R.u, ptL), fma2(AL, L.u, ptR)), iden);
-  const float2 pts = mul2(fma2(mul2(mul2(L.rho, R.rho), mul2(suR, suL)), sub2(R.u, L.u),
-                               sub2(mul2(AR, ptL), mul2(AL, ptR))),
-                          iden);
-  const Star2 SL = hlld_star_xy(L, sl, suL, AL, ptL, eL, sm, pts, bx, bx2);
-  const Star2 SR = hlld_star_xy(R, sr, suR, AR, ptR, eR, sm, pts, bx, bx2);
+  const float2 pts =
+      mul2(fma2(mul2(AL, AR), sub2(R.u, L.u), sub2(mul2(AR, ptL), mul2(AL, ptR))), iden);
+  const float2 psm = mul2(pts, sm), sbx = mul2(sm, bx);
+  const Star2 SL = hlld_star2(L, sl, suL, AL, ptL, eL, sm, psm, sbx, bx, bx2);
+  const Star2 SR = hlld_star2(R, sr, suR, AR, ptR, eR, sm, psm, sbx, bx, bx2);
   // double-star states (MK05 eqs. 59-63)
   const float2 isqL = make_float2(rsqrtf(SL.rs.x), rsqrtf(SL.rs.y));
   const float2 isqR = make_float2(rsqrtf(SR.rs.x), rsqrtf(SR.rs.y));
   const float2 sqrL = mul2(SL.rs, isqL), sqrR = mul2(SR.rs, isqR);
   const float2 abx = abs2(bx);
   const float2 ssl = sub2(sm, mul2(abx, isqL)), ssr = fma2(abx, isqR, sm);
-  const float2 sb = make_float2(sgnT(bx.x), sgnT(bx.y));
+  const float2 sb = make_float2(bx.x == 0.f ? 0.f : copysignf(1.f, bx.x),
+                                bx.y == 0.f ? 0.f : copysignf(1.f, bx.y));
   const float2 issum = rcp2(add2(sqrL, sqrR));
-  const float2 vss = mul2(fma2(sub2(SR.bys, SL.bys), sb, fma2(sqrR, SR.vs, mul2(sqrL, SL.vs))), issum);
-  const float2 wss = mul2(fma2(sub2(SR.bzs, SL.bzs), sb, fma2(sqrR, SR.ws, mul2(sqrL, SL.ws))), issum);
-  const float2 sqq = mul2(mul2(sqrL, sqrR), sb);
-  const float2 byss = mul2(fma2(sub2(SR.vs, SL.vs), sqq, fma2(sqrL, SR.bys, mul2(sqrR, SL.bys))), issum);
-  const float2 bzss = mul2(fma2(sub2(SR.ws, SL.ws), sqq, fma2(sqrL, SR.bzs, mul2(sqrR, SL.bzs))), issum);
-  const float2 vbss = fma2(wss, bzss, fma2(vss, byss, mul2(sm, bx)));
-  // e** = e* -/+ sqrt(rho*) (v*.B* - v**.B**) sgn(Bx)
-  const float2 essL = fma2(mul2(sqrL, sb), sub2(vbss, SL.vbs), SL.es);
-  const float2 essR = fma2(mul2(sqrR, sb), sub2(SR.vbs, vbss), SR.es);
+  const float2 wL = mul2(sqrL, issum), wR = mul2(sqrR, issum), wS = mul2(sb, issum);
+  const float2 wQ = mul2(mul2(sqrL, wR), sb);
+  const float2 vss = fma2(sub2(SR.bys, SL.bys), wS, fma2(wR, SR.vs, mul2(wL, SL.vs)));
+  const float2 wss = fma2(sub2(SR.bzs, SL.bzs), wS, fma2(wR, SR.ws, mul2(wL, SL.ws)));
+  const float2 byss = fma2(sub2(SR.vs, SL.vs), wQ, fma2(wL, SR.bys, mul2(wR, SL.bys)));
+  const float2 bzss = fma2(sub2(SR.ws, SL.ws), wQ, fma2(wL, SR.bzs, mul2(wR, SL.bzs)));
+  const float2 vbss = fma2(wss, bzss, fma2(vss, byss, sbx));
   // fan region containing x/t = 0, per face (ties as in the scalar solver)
   const bool lx = sm.x >= 0.f, ly = sm.y >= 0.f;
   const bool ox = lx ? (sl.x > 0.f) : (sr.x < 0.f), oy = ly ? (sl.y > 0.f) : (sr.y < 0.f);
   const bool sx = lx ? (ssl.x >= 0.f) : !(ssr.x >= 0.f);
   const bool sy = ly ? (ssl.y >= 0.f) : !(ssr.y >= 0.f);
   // the upwind side of S_M
-  const float2 rho = sel2(lx, ly, L.rho, R.rho), u = sel2(lx, ly, L.u, R.u);
-  const float2 v = sel2(lx, ly, L.v, R.v), w = sel2(lx, ly, L.w, R.w);
-  const float2 by = sel2(lx, ly, L.by, R.by), bz = sel2(lx, ly, L.bz, R.bz);
+  const Prim2 q = {sel2(lx, ly, L.rho, R.rho), sel2(lx, ly, L.u, R.u), sel2(lx, ly, L.v, R.v),
+                   sel2(lx, ly, L.w, R.w),     sp2(0.f),               sel2(lx, ly, L.by, R.by),
+                   sel2(lx, ly, L.bz, R.bz)};
   const float2 pt = sel2(lx, ly, ptL, ptR), e = sel2(lx, ly, eL, eR);
   const float2 rs = sel2(lx, ly, SL.rs, SR.rs), vs = sel2(lx, ly, SL.vs, SR.vs);
   const float2 ws = sel2(lx, ly, SL.ws, SR.ws), bys = sel2(lx, ly, SL.bys, SR.bys);
   const float2 bzs = sel2(lx, ly, SL.bzs, SR.bzs), es = sel2(lx, ly, SL.es, SR.es);
-  const float2 ess = sel2(lx, ly, essL, essR);
+  const float2 vbs = sel2(lx, ly, SL.vbs, SR.vbs);
+  const float2 sq = sel2(lx, ly, neg2(sqrL), sqrR);
   const float2 c1 = sel2(lx, ly, sl, sr), c2 = sel2(lx, ly, ssl, ssr);
-  const float2 mu = mul2(rho, u);
-  const float2 vb = fma2(w, bz, fma2(v, by, mul2(u, bx)));
-  // physical flux F, state U, star U* and double-star U** of that side
-  const float2 F[8] = {mu, fma2(mu, u, sub2(pt, bx2)), fma2(mu, v, mul2(mul2(bx, by), sp2(-1.f))),
-                       fma2(mu, w, mul2(mul2(bx, bz), sp2(-1.f))),
-                       sub2(mul2(add2(e, pt), u), mul2(bx, vb)), sp2(0.f),
-                       sub2(mul2(by, u), mul2(bx, v)), sub2(mul2(bz, u), mul2(bx, w))};
-  const float2 U[8] = {rho, mu, mul2(rho, v), mul2(rho, w), e, bx, by, bz};
+  float2 U[8], F[8];
+  state_flux2(q, bx, bx2, pt, e, U, F);
+  // flux F + c1 (U* - U) + c2 (U** - U*): the double star keeps rho* and S_M,
+  // and e** - e* = -/+ sqrt(rho*) (v*.B* - v**.B**) sgn(Bx)
+  const float2 c2r = mul2(c2, rs);
   const float2 US[8] = {rs, mul2(rs, sm), mul2(rs, vs), mul2(rs, ws), es, bx, bys, bzs};
-  const float2 USS[8] = {rs, mul2(rs, sm), mul2(rs, vss), mul2(rs, wss), ess, bx, byss, bzss};
+  const float2 de = mul2(mul2(sq, sb), sub2(vbs, vbss));
 #pragma unroll
   for (int c = 0; c < 8; c++) {
     if (c == 5) {
@@ -423,131 +587,44 @@ __device__ __forceinline__ void hlld_xy(float g, float ig1, const Prim2& L, cons
       continue;
     }
     const float2 fs = fma2(c1, sub2(US[c], U[c]), F[c]);
-    // the double-star and star states differ in the tangential and energy parts only
-    const float2 fss = (c == 0 || c == 1) ? fs : fma2(c2, sub2(USS[c], US[c]), fs);
-    f[c] = make_float2(ox ? F[c].x : (sx ? fs.x : fss.x), oy ? F[c].y : (sy ? fs.y : fss.y));
+    float2 fss = fs;
+    if (c == 2) fss = fma2(c2r, sub2(vss, vs), fs);
+    if (c == 3) fss = fma2(c2r, sub2(wss, ws), fs);
+    if (c == 4) fss = fma2(c2, de, fs);
+    if (c == 6) fss = fma2(c2, sub2(byss, bys), fs);
+    if (c == 7) fss = fma2(c2, sub2(bzss, bzs), fs);
+    f[c] = sel2(ox, oy, F[c], c < 2 ? fs : sel2(sx, sy, fs, fss));
   }
 }
 
-// local component c of the y face -> primitive variable (normal y, tangential
-// (z, x)); the x face uses the identity
-__device__ __forceinline__ constexpr int yface_var(int c) {
-  return c == 1 ? 2 : c == 2 ? 3 : c == 3 ? 1 : c == 5 ? 6 : c == 6 ? 7 : c == 7 ? 5 : c;
-}
-
-// x and y face fluxes of one cell with vanleer + HLLD: ax(v, t), ay(v, t) the
-// 4-cell stencils (cells f-2 .. f+1) of the x and y faces; positivity fallback
-// and glm as in stencil_flux_f2, per face
-template <class AX, class AY>
-__device__ __forceinline__ void stencil_flux_xy(AX ax, AY ay, int glm, float g, float ch,
-                                                float* fx, float* fy) {
-  float2 wl[NV], wr[NV];
-#pragma unroll
-  for (int c = 0; c < NV; c++) {
-    const int vy = yface_var(c);
-    const float2 A = make_float2(ax(c, 0), ay(vy, 0)), B = make_float2(ax(c, 1), ay(vy, 1));
-    const float2 C = make_float2(ax(c, 2), ay(vy, 2)), E = make_float2(ax(c, 3), ay(vy, 3));
-    const float2 d2 = sub2(C, B);
-    wl[c] = fma2(sp2(0.5f), vl_slope2(sub2(B, A), d2), B);
-    wr[c] = fma2(sp2(-0.5f), vl_slope2(d2, sub2(E, C)), C);
-  }
-  const bool bx_ = !(wl[0].x > 0.f) || !(wl[4].x > 0.f) || !(wr[0].x > 0.f) || !(wr[4].x > 0.f);
-  const bool by_ = !(wl[0].y > 0.f) || !(wl[4].y > 0.f) || !(wr[0].y > 0.f) || !(wr[4].y > 0.f);
-  if (bx_ || by_) {
-#pragma unroll
-    for (int c = 0; c < NV; c++) {
-      if (bx_) {
-        wl[c].x = ax(c, 1);
-        wr[c].x = ax(c, 2);
-      }
-      if (by_) {
-        wl[c].y = ay(yface_var(c), 1);
-        wr[c].y = ay(yface_var(c), 2);
-      }
-    }
-  }
+// fluxes of an x face (lane x) and a y face (lane y) from their left and right
+// states in the local frames (component c of lane y is variable yface_var(c));
+// component 5 is the flux of the normal field
+template <int FLUX>
+__device__ __forceinline__ void face_flux_xy(const float2* wl, const float2* wr,
+                                             const FaceConst2& fc, float2* f) {
   const float2 bnl = wl[5], bnr = wr[5];
-  float2 bns, psis;
-  if (glm) {
-    const float ih = 0.5f / ch;
-    bns = sub2(mul2(sp2(0.5f), add2(bnl, bnr)), mul2(sp2(ih), sub2(wr[8], wl[8])));
-    psis = sub2(mul2(sp2(0.5f), add2(wl[8], wr[8])), mul2(sp2(0.5f * ch), sub2(bnr, bnl)));
-  } else {
-    bns = mul2(sp2(0.5f), add2(bnl, bnr));
-    psis = sp2(0.f);
+  float2 bns = mul2(sp2(0.5f), add2(bnl, bnr)), psis = sp2(0.f), fpsi = sp2(0.f);
+  if (fc.glm) {
+    bns = fma2(sub2(wl[8], wr[8]), sp2(fc.hich), bns);
+    psis = fma2(sub2(bnl, bnr), sp2(0.5f * fc.ch), mul2(sp2(0.5f), add2(wl[8], wr[8])));
+    fpsi = mul2(sp2(fc.ch * fc.ch), bns);
   }
-  float2 fl[8];
   const Prim2 L = {wl[0], wl[1], wl[2], wl[3], wl[4], wl[6], wl[7]};
   const Prim2 R = {wr[0], wr[1], wr[2], wr[3], wr[4], wr[6], wr[7]};
-  hlld_xy(g, 1.f / (g - 1.f), L, R, bns, fl);
-  const float2 fpsi = glm ? mul2(sp2(ch * ch), bns) : sp2(0.f);
-  fl[5] = psis;
-#pragma unroll
-  for (int c = 0; c < 8; c++) {
-    fx[c] = fl[c].x;
-    fy[yface_var(c)] = fl[c].y;
-  }
-  fx[8] = fpsi.x;
-  fy[8] = fpsi.y;
-}
-
-template <int D, int FLUX>
-__device__ __forceinline__ void face_flux_f2(float2* w, int glm, float g, float ch, float* f);
-
-// Face flux along D from the 4-cell stencils of the 9 primitive variables:
-// st(v, t) for cells f-2, f-1, f, f+1.  Positivity fallback and glm as in
-// face_flux_d.
-// LIM < 0: the limiter is the runtime value lim.
-template <int D, int LIM, int FLUX, class Acc>
-__device__ __forceinline__ void stencil_flux_f2(Acc st, int glm, float g, float ch, float* f,
-                                                int lim) {
-  float2 w[NV];
-  if constexpr (LIM >= 0) {
-#pragma unroll
-    for (int v = 0; v < NV; v++) {
-      float a = st(v, 0), b = st(v, 1), c = st(v, 2), e = st(v, 3);
-      if (LIM == AMRVAC_LIM_VANLEER) w[v] = vanleer_pair(a, b, c, e);
-      else w[v] = make_float2(recon_plus<float>(LIM, a, b, c), recon_minus<float>(LIM, b, c, e));
-    }
-  } else {
-    // runtime limiter: one switch per face, the variable loop inside (not
-    // unrolled: four limiters inlined at three faces would otherwise crowd the
-    // instruction cache)
-    if (lim == AMRVAC_LIM_SUPERBEE) {
-#pragma unroll 1
-      for (int v = 0; v < NV; v++) w[v] = sym_pair<1>(st(v, 0), st(v, 1), st(v, 2), st(v, 3), 0.f);
-    } else if (lim == AMRVAC_LIM_ALBADA) {
-#pragma unroll 1
-      for (int v = 0; v < NV; v++) w[v] = sym_pair<2>(st(v, 0), st(v, 1), st(v, 2), st(v, 3), 0.f);
-    } else if (lim == AMRVAC_LIM_CADA3) {
-#pragma unroll 1
-      for (int v = 0; v < NV; v++) w[v] = cada3_pair(st(v, 0), st(v, 1), st(v, 2), st(v, 3));
-    } else if (lim == AMRVAC_LIM_VENK) {
-#pragma unroll 1
-      for (int v = 0; v < NV; v++) {
-        const float a = st(v, 0), b = st(v, 1), c = st(v, 2), e = st(v, 3);
-        w[v] = make_float2(b + venk_increment(a, b, c), c - venk_increment(b, c, e));
-      }
-    } else {
-      const float beta = lim == AMRVAC_LIM_WOODWARD ? 2.f : 1.4f;
-#pragma unroll 1
-      for (int v = 0; v < NV; v++)
-        w[v] = sym_pair<0>(st(v, 0), st(v, 1), st(v, 2), st(v, 3), beta);
-    }
-  }
-  if (!(w[0].x > 0.f) || !(w[4].x > 0.f) || !(w[0].y > 0.f) || !(w[4].y > 0.f)) {
-#pragma unroll
-    for (int v = 0; v < NV; v++) w[v] = make_float2(st(v, 1), st(v, 2));
-  }
-  face_flux_f2<D, FLUX>(w, glm, g, ch, f);
+  if constexpr (FLUX == AMRVAC_FLUX_HLLD) hlld2(fc.g, fc.ig1, L, R, bns, f);
+  else if constexpr (FLUX == AMRVAC_FLUX_HLLC) hllc2(fc.g, fc.ig1, L, R, bns, f);
+  else hll2<FLUX>(fc.g, fc.ig1, L, R, bns, f);
+  f[5] = psis;
+  f[8] = fpsi;
 }
 
 // Five-point limiters (mp5, weno5, wenoz5, wenozp5; lim at run time, lam the
 // wenozp5 lambda): st(v, t) for the six cells f-3 .. f+2 around the face
 // f-1/2; each face state reconstructed in float as on the plain path
 template <int D, int FLUX, class Acc>
-__device__ __forceinline__ void stencil_flux5_f2(Acc st, int lim, float lam, int glm, float g,
-                                                 float ch, float* f) {
+__device__ __forceinline__ void stencil_flux5_f2(Acc st, int lim, float lam, const FaceConst2& fc,
+                                                 float* f) {
   float2 w[NV];
   // one copy of the reconstruction for the nine variables (not unrolled): the
   // limiters' code, four of them behind the runtime switch and inlined at the
@@ -557,54 +634,11 @@ __device__ __forceinline__ void stencil_flux5_f2(Acc st, int lim, float lam, int
     const float c[6] = {st(v, 0), st(v, 1), st(v, 2), st(v, 3), st(v, 4), st(v, 5)};
     w[v] = make_float2(recon5_plus<float>(lim, c, lam), recon5_minus<float>(lim, c + 1, lam));
   }
-  if (!(w[0].x > 0.f) || !(w[4].x > 0.f) || !(w[0].y > 0.f) || !(w[4].y > 0.f)) {
+  if (not_positive2(w)) {
 #pragma unroll
     for (int v = 0; v < NV; v++) w[v] = make_float2(st(v, 2), st(v, 3));
   }
-  face_flux_f2<D, FLUX>(w, glm, g, ch, f);
-}
-
-// glm solve and Riemann flux along D from the face states w[v] = (left, right)
-template <int D, int FLUX>
-__device__ __forceinline__ void face_flux_f2(float2* w, int glm, float g, float ch, float* f) {
-  constexpr int t1 = D == 2 ? 0 : D + 1, t2 = D == 0 ? 2 : D - 1;
-  const float bnl = w[5 + D].x, bnr = w[5 + D].y;
-  float bns, psis;
-  if (glm) {
-    bns = 0.5f * (bnl + bnr) - (w[8].y - w[8].x) / (2.f * ch);
-    psis = 0.5f * (w[8].x + w[8].y) - 0.5f * ch * (bnr - bnl);
-  } else {
-    bns = 0.5f * (bnl + bnr);
-    psis = 0.f;
-  }
-  Side2 q;
-  q.rho = w[0];
-  q.u = w[1 + D];
-  q.v = w[1 + t1];
-  q.w = w[1 + t2];
-  q.p = w[4];
-  q.by = w[5 + t1];
-  q.bz = w[5 + t2];
-  float fl[8];
-  const float ig1 = 1.f / (g - 1.f);
-  if (FLUX == AMRVAC_FLUX_HLL) hll_pair(g, ig1, q, bns, fl);
-  else if (FLUX == AMRVAC_FLUX_HLLD) hlld_pair(g, ig1, q, bns, fl);
-  else if (FLUX == AMRVAC_FLUX_TVDLF) tvdlf_pair(g, ig1, q, bns, fl);
-  else {
-    // HLLC: the scalar three-wave solver on the unpacked face states
-    const float ql[8] = {q.rho.x, q.u.x, q.v.x, q.w.x, q.p.x, bns, q.by.x, q.bz.x};
-    const float qr[8] = {q.rho.y, q.u.y, q.v.y, q.w.y, q.p.y, bns, q.by.y, q.bz.y};
-    hllc_local<float>(g, ig1, ql, qr, bns, fl);
-  }
-  f[0] = fl[0];
-  f[1 + D] = fl[1];
-  f[1 + t1] = fl[2];
-  f[1 + t2] = fl[3];
-  f[4] = fl[4];
-  f[5 + D] = glm ? psis : 0.f;
-  f[5 + t1] = fl[6];
-  f[5 + t2] = fl[7];
-  f[8] = glm ? ch * ch * bns : 0.f;
+  face_flux2<D, FLUX>(w, fc, f);
 }
 
 }  // namespace amrvac
