@@ -356,8 +356,8 @@ Layout make_layout(const amrvac_config* c, int ninst, int nblocks, const Tables&
     L.flags = take((size_t)ncell * nblocks);
     L.fixcount = take(sizeof(unsigned long long));
   }
-  L.lcf = take(sizeof(float) * LC_N * MAXLEV * ninst);
-  L.lcd = take(sizeof(double) * LC_N * MAXLEV * ninst);
+  L.lcf = take(sizeof(float) * LC_N * MAXLEV * ninst * MAXSTAGE);
+  L.lcd = take(sizeof(double) * LC_N * MAXLEV * ninst * MAXSTAGE);
   // regridding: per-block estimator and flag, and the transfer table
   L.est = take(sizeof(double) * nblocks);
   L.eflags = take((size_t)nblocks);
@@ -418,6 +418,8 @@ amrvac_status enqueue_stage(amrvac_state* s, int k, int epilogue, int* count) {
 
 amrvac_status enqueue_step(amrvac_state* s, int* count) {
   const int ns = num_stages(s->cfg.time);
+  if (launch_level_consts(s, 0, ns) < 0) return AMRVAC_E_CUDA;
+  *count += 1;
   for (int k = 0; k < ns; k++) {
     amrvac_status st = enqueue_stage(s, k, k == ns - 1, count);
     if (st) return st;
@@ -811,7 +813,8 @@ amrvac_status amrvac_cfl_dt(amrvac_state* s, int32_t buffer, double* h_dt_out) {
 amrvac_status amrvac_stage(amrvac_state* s, int32_t stage) {
   if (!s || stage < 0 || stage >= num_stages(s->cfg.time)) return AMRVAC_E_INVALID;
   if (!s->dt_valid) return AMRVAC_E_STATE;
-  int count = 0;
+  int count = 1;
+  if (launch_level_consts(s, stage, 1) < 0) return AMRVAC_E_CUDA;
   amrvac_status st = enqueue_stage(s, stage, stage == num_stages(s->cfg.time) - 1, &count);
   s->launches += count;
   return st;

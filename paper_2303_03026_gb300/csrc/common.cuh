@@ -14,6 +14,7 @@ constexpr int NV = 9;       // rho, m_x, m_y, m_z, e, B_x, B_y, B_z, psi
 constexpr int NG = 2;       // ghost cells per face of the two-ghost-cell limiters
 constexpr int NG5 = 3;      // ghost cells per face of the five-point limiters (plain path)
 constexpr int MAXLEV = AMRVAC_MAX_LEVELS;
+constexpr int MAXSTAGE = 5;  // stages of the longest scheme
 constexpr int NPART = 12;   // per-block partials: smax, chmax, sums[9], pad
 
 // the limiters that reconstruct from five cells (three ghost layers)
@@ -21,8 +22,8 @@ __host__ __device__ inline bool five_point_limiter(int lim) {
   return lim == AMRVAC_LIM_MP5 || lim == AMRVAC_LIM_WENO5 || lim == AMRVAC_LIM_WENOZ5 ||
          lim == AMRVAC_LIM_WENOZP5;
 }
-// per-(instance, level) stage constants of the fused kernels, refreshed from
-// InstRT before every fused stage: c dt (the stage's Euler step), ch, psi
+// per-(instance, level) stage constants, refreshed from InstRT before every step
+// (or single stage): c dt (the stage's Euler step), ch, psi
 // damping factor over c dt, dx[3], 1/dx[3], finished flag (dt == 0), gamma,
 // gamma - 1, and c2 dt with its damping factor (second output)
 constexpr int LC_N = 16;
@@ -70,8 +71,8 @@ struct DevMesh {
   double* part;           // [nblocks][NPART]
   double* sums;           // [ninst][NV]
   int* err;               // [4] code, block, cell, var
-  float* lcf;             // [ninst][MAXLEV][LC_N] stage constants, float (FP32 bulk)
-  double* lcd;            // [ninst][MAXLEV][LC_N] stage constants, double (FP64)
+  float* lcf;             // [stage][ninst][MAXLEV][LC_N] stage constants, float
+  double* lcd;            // the same in double (a kernel gets its stage's part of both)
 };
 
 template <class T> __device__ __forceinline__ const T* level_consts(const DevMesh& M);

@@ -45,6 +45,9 @@ constexpr int FB = 16;          // block edge handled by the fused kernel
 // (the 32 faces on the +x/+y block boundary).  The 2D kernel uses the same
 // roles with threads 0 .. 64G-1 copying and converting the halo.
 constexpr int FT = FB * FB + FB;
+// ghost layers of a tile for a limiter template value (-2: the five-point
+// limiters, chosen at run time)
+__host__ __device__ constexpr int tile_ghosts(int lim) { return lim == -2 ? NG5 : NG; }
 // Double with a two-ghost-cell limiter: every cell's limited slopes are
 // evaluated once (its two face states handed to the neighbouring face through
 // the face-flux array) instead of once per face, since the FP64 pipe bounds
@@ -53,15 +56,14 @@ constexpr int FT = FB * FB + FB;
 // With the refined approximations of fp64.cuh for division and square root: a
 // step of the 3D AMR blast in double (6.0 M cells) 85.6 -> 42.0 ms, of the 1024^2
 // vortex with koren 10.3 -> 5.3 ms. 
-template <class T, int LIM> constexpr bool share_slopes() { return sizeof(T) == 8 && LIM != -2; }
+template <class T, int LIM> constexpr bool share_slopes() {
+  return sizeof(T) == 8 && tile_ghosts(LIM) == NG;
+}
 template <class T, int LIM> constexpr int fused_threads() {
   return share_slopes<T, LIM>() ? FB * FB + 2 * FB : FT;
 }
 constexpr int FXW = 20;           // row stride of the face-flux arrays
 
-// ghost layers of a tile for a limiter template value (-2: the five-point
-// limiters, chosen at run time)
-__host__ __device__ constexpr int tile_ghosts(int lim) { return lim == -2 ? NG5 : NG; }
 
 // Thread (x, y) of a warp: lanes 0-15 take row r, lanes 16-31 row r + 4, so the
 // two half-warps of a row-stride-20 array fall on disjoint banks (4*20 = 16 mod 32;
@@ -110,39 +112,6 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.wait_group 0;\n" ::: "memory");
 }
 
-// deterministic CTA reduction of the owners' partials (warps 0..7; the partial
-// helper warp only joins the barriers); thread 0..NPART-1 store part_b
-__device__ __forceinline__ void cta_reduce_store(double (*red)[NPART], Partial& p, bool owner,
-                                                 double* part_b) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __syncthreads();
-  if (owner) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      p.smax = fmax(p.smax, __shfl_xor_sync(0xffffffffu, p.smax, o));
-      p.chm = fmax(p.chm, __shfl_xor_sync(0xffffffffu, p.chm, o));
-#pragma unroll
-      for (int v = 0; v < NV; v++) p.sum[v] += __shfl_xor_sync(0xffffffffu, p.sum[v], o);
-    }
-    if (lane == 0) {
-      red[warp][0] = p.smax;
-      red[warp][1] = p.chm;
-#pragma unroll
-      for (int v = 0; v < NV; v++) red[warp][2 + v] = p.sum[v];
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < NPART) {
-    double acc = red[0][threadIdx.x];
-    for (int w = 1; w < 8; w++) {
-      double x = red[w][threadIdx.x];
-      acc = threadIdx.x < 2 ? fmax(acc, x) : acc + x;
-    }
-    part_b[threadIdx.x] = threadIdx.x < 2 + NV ? acc : 0.0;
-  }
-  __syncthreads();
-}
-
 // CTA maximum of the owners' two CFL terms into part_b[0], part_b[1]
 __device__ __forceinline__ void cta_reduce_max2(double (*red)[NPART], double smax, double cmax,
                                                 bool owner, double* part_b) {
@@ -165,32 +134,6 @@ __device__ __forceinline__ void cta_reduce_max2(double (*red)[NPART], double sma
     for (int w = 1; w < 8; w++) acc = fmax(acc, red[w][threadIdx.x]);
     part_b[threadIdx.x] = acc;
   }
-}
-
-// CFL terms of a conserved cell: running max of sum_d (|v_d| + c_f,d)/dx_d and
-// of |v_d| + c_f,d.  The fast speed of each direction is the cancellation-free
-// form with 1/rho, a^2 = gamma p/rho and b^2 = B^2/rho shared by the
-// directions (b_t^2 = b^2 - B_d^2/rho, kept >= 0).
-template <class T, int DIM>
-__device__ __forceinline__ void cfl_terms(const T* u, double gammad, T g, bool ff, float gm1f,
-                                          const T* idx, T& smx, T& cmx) {
-  T w[NV];
-  cons2prim(gammad, u, w, ff, gm1f);
-  const T ir = rcp_T(w[0]);
-  const T a2 = g * w[4] * ir;
-  const T bb = (w[5] * w[5] + w[6] * w[6] + w[7] * w[7]) * ir;
-  const T dd = a2 - bb, sab = a2 + bb;
-  T s = T(0);
-#pragma unroll
-  for (int d = 0; d < DIM; d++) {
-    const T bt = bb - w[5 + d] * w[5 + d] * ir;
-    const T bt2 = gt0(bt) ? bt : T(0);  // no negative rounding
-    const T cf = sqrt_T(T(0.5) * (sab + sqrt_T(dd * dd + T(4) * a2 * bt2)));
-    const T spd = fabs(w[1 + d]) + cf;
-    s += spd * idx[d];
-    cmx = fmax(cmx, spd);
-  }
-  smx = fmax(smx, s);
 }
 
 // refluxing: the flux f of cell `idx` of level-change face `face` of the block
@@ -828,7 +771,7 @@ template <class T, int DIM, int LIM, int FLUX, bool FULL> struct FusedKernel {
 };
 
 template <class T, int DIM, int LIM, int FLUX, bool FULL>
-static int launch_one(amrvac_state* s, const T* U0, const T* Uk, const T* U2, T* out, T* out2,
+static int launch_one(amrvac_state* s, int k, const T* U0, const T* Uk, const T* U2, T* out, T* out2,
                       const int* work, int nwork, int* counter, StageParams sp) {
   static_assert(DIM == 2 || LIM != -2 || sizeof(T) == 4,
                 "five-point limiters in 3D: FP32 bulk only (a double 6-plane ring does not fit)");
@@ -854,7 +797,7 @@ static int launch_one(amrvac_state* s, const T* U0, const T* Uk, const T* U2, T*
   if (s->tune.dynamic) {
     if (cudaMemsetAsync(counter, 0, sizeof(int), s->stream) != cudaSuccess) return -1;
   }
-  kern<<<grid, NT, smem, s->stream>>>(s->mesh, U0, Uk, U2, out, out2, work, nwork,
+  kern<<<grid, NT, smem, s->stream>>>(stage_mesh(s, k), U0, Uk, U2, out, out2, work, nwork,
                                        (const T*)s->gslab, s->tune.dynamic ? counter : nullptr,
                                        sp);
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
@@ -862,7 +805,7 @@ static int launch_one(amrvac_state* s, const T* U0, const T* Uk, const T* U2, T*
 
 // Stage k for scheme group g (the blocks of the levels sharing this
 // limiter and the group's flux); group 0 also launches the per-stage passes
-// every group shares: the stage constants and the ghost slabs.
+// every group shares, the ghost slabs.
 template <class T, int DIM, int LIM>
 int launch_fused_l(amrvac_state* s, int k, int epilogue, int g) {
   const StageBuffers sb = stage_buffers(s->cfg.time, k);
@@ -876,8 +819,6 @@ int launch_fused_l(amrvac_state* s, int k, int epilogue, int g) {
   T* out2 = sb.out2 >= 0 ? (T*)s->U[sb.out2] : nullptr;
   int n = 0;
   if (g == 0) {
-    if (launch_level_consts(s, k) < 0) return -1;
-    n++;
     if (s->ngen > 0) {
       // ghost slabs of the level-change faces of the stage input (as many
       // layers as the mesh's tiles have ghost cells)
@@ -901,24 +842,24 @@ int launch_fused_l(amrvac_state* s, int k, int epilogue, int g) {
   const int flux = s->grp_flux[g];
   int m;
   if (flux == AMRVAC_FLUX_HLLD)
-    m = full ? launch_one<T, DIM, LIM, AMRVAC_FLUX_HLLD, true>(s, U0, Uk, U2, out, out2, work,
+    m = full ? launch_one<T, DIM, LIM, AMRVAC_FLUX_HLLD, true>(s, k, U0, Uk, U2, out, out2, work,
                                                                nwork, counter, sp)
-             : launch_one<T, DIM, LIM, AMRVAC_FLUX_HLLD, false>(s, U0, Uk, U2, out, out2, work,
+             : launch_one<T, DIM, LIM, AMRVAC_FLUX_HLLD, false>(s, k, U0, Uk, U2, out, out2, work,
                                                                 nwork, counter, sp);
   else if (flux == AMRVAC_FLUX_HLL)
-    m = full ? launch_one<T, DIM, LIM, AMRVAC_FLUX_HLL, true>(s, U0, Uk, U2, out, out2, work,
+    m = full ? launch_one<T, DIM, LIM, AMRVAC_FLUX_HLL, true>(s, k, U0, Uk, U2, out, out2, work,
                                                               nwork, counter, sp)
-             : launch_one<T, DIM, LIM, AMRVAC_FLUX_HLL, false>(s, U0, Uk, U2, out, out2, work,
+             : launch_one<T, DIM, LIM, AMRVAC_FLUX_HLL, false>(s, k, U0, Uk, U2, out, out2, work,
                                                                nwork, counter, sp);
   else if (flux == AMRVAC_FLUX_TVDLF)
-    m = full ? launch_one<T, DIM, LIM, AMRVAC_FLUX_TVDLF, true>(s, U0, Uk, U2, out, out2, work,
+    m = full ? launch_one<T, DIM, LIM, AMRVAC_FLUX_TVDLF, true>(s, k, U0, Uk, U2, out, out2, work,
                                                                 nwork, counter, sp)
-             : launch_one<T, DIM, LIM, AMRVAC_FLUX_TVDLF, false>(s, U0, Uk, U2, out, out2, work,
+             : launch_one<T, DIM, LIM, AMRVAC_FLUX_TVDLF, false>(s, k, U0, Uk, U2, out, out2, work,
                                                                  nwork, counter, sp);
   else
-    m = full ? launch_one<T, DIM, LIM, AMRVAC_FLUX_HLLC, true>(s, U0, Uk, U2, out, out2, work,
+    m = full ? launch_one<T, DIM, LIM, AMRVAC_FLUX_HLLC, true>(s, k, U0, Uk, U2, out, out2, work,
                                                                nwork, counter, sp)
-             : launch_one<T, DIM, LIM, AMRVAC_FLUX_HLLC, false>(s, U0, Uk, U2, out, out2, work,
+             : launch_one<T, DIM, LIM, AMRVAC_FLUX_HLLC, false>(s, k, U0, Uk, U2, out, out2, work,
                                                                 nwork, counter, sp);
   return m < 0 ? -1 : n + m;
 }

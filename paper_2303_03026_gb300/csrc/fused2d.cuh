@@ -19,24 +19,6 @@
 
 namespace amrvac {
 
-// Per-warp maxima of the owners' two CFL terms merged into part_b[0..1] with
-// atomicMax on the bit patterns (order-independent for values >= 0; NaN is
-// dropped as fmax drops it).  part_b[0..1] are zeroed before the block's first
-// barrier, the atomics come after its last one.
-__device__ __forceinline__ void warp_max2_atomic(double smax, double cmax, double* part_b) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, o));
-    cmax = fmax(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
-  }
-  if ((threadIdx.x & 31) == 0) {
-    if (smax == smax)
-      atomicMax((unsigned long long*)&part_b[0], (unsigned long long)__double_as_longlong(smax));
-    if (cmax == cmax)
-      atomicMax((unsigned long long*)&part_b[1], (unsigned long long)__double_as_longlong(cmax));
-  }
-}
-
 // G: ghost layers of the tile (2, or 3 for the five-point limiters)
 template <class T, int G = NG> struct Fused2dSmem {
   static constexpr int PW = FB + 2 * G;  // padded tile width

@@ -44,40 +44,17 @@ __global__ void __launch_bounds__(256) k_cfl_partials_static(DevMesh M, const T*
                                                              double dx1, double dx2, int ff,
                                                              double* __restrict__ partials) {
   const size_t vs = (size_t)M.nblocks * M.ncell;
-  const double dx[3] = {dx0, dx1, dx2};
+  const T idx[3] = {(T)(1.0 / dx0), (T)(1.0 / dx1), (T)(1.0 / dx2)};
   for (int b = blockIdx.x; b < M.nblocks; b += gridDim.x) {
-    Partial p;
-    partial_zero(p);
+    T smx = T(0), cmx = T(0);
     for (int c = threadIdx.x; c < M.ncell; c += blockDim.x) {
       T u[NV];
       const T* src = U + (size_t)b * M.ncell + c;
 #pragma unroll
       for (int v = 0; v < NV; v++) u[v] = src[(size_t)v * vs];
-      accumulate_cell(M, u, gamma, dx, p, ff != 0);
+      cfl_terms_nd(M.ndim, u, gamma, (T)gamma, ff != 0, (float)(gamma - 1.0), idx, smx, cmx);
     }
-    // block maximum: warp shuffles, then the warps' maxima in a fixed order
-    __shared__ double sh[32][2];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      p.smax = fmax(p.smax, __shfl_xor_sync(0xffffffffu, p.smax, o));
-      p.chm = fmax(p.chm, __shfl_xor_sync(0xffffffffu, p.chm, o));
-    }
-    if (lane == 0) {
-      sh[warp][0] = p.smax;
-      sh[warp][1] = p.chm;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double m0 = sh[0][0], m1 = sh[0][1];
-      for (int w = 1; w < (int)(blockDim.x >> 5); w++) {
-        m0 = fmax(m0, sh[w][0]);
-        m1 = fmax(m1, sh[w][1]);
-      }
-      partials[2 * b] = m0;
-      partials[2 * b + 1] = m1;
-    }
-    __syncthreads();
+    cta_max2(smx, cmx, false, partials + 2 * (size_t)b);
   }
 }
 

@@ -22,6 +22,16 @@ static inline int grid_for(size_t work, int threads) {
   return (int)g;
 }
 
+// Threads per CTA of the passes over cells and faces: one SM evaluates 2 double
+// lanes a clock, so a small mesh is spread over the SMs in CTAs of one to four
+// warps (a 512-cell shock tube's face pass: 33 us in 3 CTAs of 256, the work of a
+// face being some 400 double operations), a large one takes 256.
+static inline int threads_for(size_t work) {
+  int t = 32;
+  while (t < 256 && work > (size_t)t * 152 * 2) t *= 2;
+  return t;
+}
+
 // ------------------------------------------------------------------ k_prim
 
 template <class T>
@@ -36,6 +46,8 @@ __global__ void __launch_bounds__(256) k_prim(DevMesh M, const T* __restrict__ U
        t += (size_t)gridDim.x * blockDim.x) {
     int b = (int)(t / np);
     int pc = (int)(t - (size_t)b * np);
+    // the CFL maxima of the block, merged by the CTAs of k_update
+    if (sp.epilogue && pc == 0) M.part[(size_t)b * NPART] = M.part[(size_t)b * NPART + 1] = 0.0;
     int i = pc % P0 - g0, j = (pc / P0) % P1 - g1, k = pc / (P0 * P1) - g2;
     int outside = (i < 0 || i >= M.nx[0]) + (j < 0 || j >= M.nx[1]) + (k < 0 || k >= M.nx[2]);
     if (outside > 1) continue;
@@ -120,60 +132,60 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh M, const T* __restrict__ W
 
 // ------------------------------------------------------------------ k_update
 
+// one CTA per chunk of blockDim.x cells of a block (nchunk chunks a block), so that
+// few large blocks fill the chip too; the stage constants from the level's table
+// (every thread formed 1/dx and two double exponentials before: a third of the
+// pass on 12^2 blocks).  With the spread of threads_for: four steps of a 512-cell
+// shock tube 158 -> 104 us, a step of the 2D mesh of 12^2 blocks 1.75 -> 1.55 ms.
 template <class T>
 __global__ void __launch_bounds__(256) k_update(DevMesh M, const T* U0,
                                                 const T* Uk, const T* U2, T* out, T* out2,
                                                 const T* __restrict__ F0,
                                                 const T* __restrict__ F1,
-                                                const T* __restrict__ F2, StageParams sp) {
+                                                const T* __restrict__ F2, int nchunk,
+                                                StageParams sp) {
   const size_t vs = (size_t)M.nblocks * M.ncell;
   const int nx0 = M.nx[0], nx1 = M.nx[1], nx2 = M.nx[2];
   const size_t nf0 = (size_t)(nx0 + 1) * nx1 * nx2;
   const size_t nf1 = (size_t)nx0 * (nx1 + 1) * nx2;
   const size_t nf2 = (size_t)nx0 * nx1 * (nx2 + 1);
-  for (int b = blockIdx.x; b < M.nblocks; b += gridDim.x) {
-    const int* bi = M.blk + b * 5;
-    const int q = bi[0], L = bi[1];
-    const InstRT rt = M.rt[q];
-    const double* dxl = M.dx + (q * MAXLEV + L) * 3;
-    double dx[3] = {dxl[0], dxl[1], dxl[2]};
-    Partial p;
-    partial_zero(p);
-    const double gamma = M.gamma[q];
-    double dxmin = dx[0];
-    for (int d = 1; d < M.ndim; d++) dxmin = fmin(dxmin, dx[d]);
-    const double dt1 = sp.c * rt.dt, dt2 = sp.c2 * rt.dt;
-    const T damp = sp.glm ? (T)exp(-sp.glm_alpha * rt.ch * dt1 / dxmin) : T(1);
-    const T damp2 = sp.glm ? (T)exp(-sp.glm_alpha * rt.ch * dt2 / dxmin) : T(1);
-    const T dt = (T)dt1, dtb = (T)dt2, a = (T)sp.a, bb = (T)sp.b;
+  const size_t nitem = (size_t)M.nblocks * nchunk;
+  for (size_t item = blockIdx.x; item < nitem; item += gridDim.x) {
+    const int b = (int)(item / nchunk);
+    const int c = (int)(item - (size_t)b * nchunk) * blockDim.x + threadIdx.x;
+    const int q = M.blk[b * 5], L = M.blk[b * 5 + 1];
+    const double* lc = M.lcd + (q * MAXLEV + L) * LC_N;
+    const T idx[3] = {(T)lc[LC_IDX], (T)lc[LC_IDX + 1], (T)lc[LC_IDX + 2]};
+    const T damp = (T)lc[LC_DAMP], damp2 = (T)lc[LC_DAMP2];
+    const T dt = (T)lc[LC_DT], dtb = (T)lc[LC_DT2], a = (T)sp.a, bb = (T)sp.b;
     const T a2 = (T)sp.a2, b2 = (T)sp.b2;
-    const T idx0 = (T)(1.0 / dx[0]), idx1 = (T)(1.0 / dx[1]), idx2 = (T)(1.0 / dx[2]);
-    for (int c = threadIdx.x; c < M.ncell; c += blockDim.x) {
-      int i = c % nx0, j = (c / nx0) % nx1, k = c / (nx0 * nx1);
+    T smx = T(0), cmx = T(0);
+    if (c < M.ncell) {
+      const int i = c % nx0, j = (c / nx0) % nx1, k = c / (nx0 * nx1);
       T un[NV], u2n[NV];
-      if (rt.dt == 0.0) {
+      if (lc[LC_SKIP] != 0.0) {
 #pragma unroll
         for (int v = 0; v < NV; v++) {
           un[v] = Uk[(size_t)v * vs + (size_t)b * M.ncell + c];
           u2n[v] = un[v];
         }
       } else {
-        size_t f0 = ((size_t)k * nx1 + j) * (nx0 + 1) + i;
-        size_t f1 = ((size_t)k * (nx1 + 1) + j) * nx0 + i;
-        size_t f2 = ((size_t)k * nx1 + j) * nx0 + i;
+        const size_t f0 = ((size_t)k * nx1 + j) * (nx0 + 1) + i;
+        const size_t f1 = ((size_t)k * (nx1 + 1) + j) * nx0 + i;
+        const size_t f2 = ((size_t)k * nx1 + j) * nx0 + i;
 #pragma unroll
         for (int v = 0; v < NV; v++) {
           const T* g0 = F0 + ((size_t)b * NV + v) * nf0;
-          T acc = (g0[f0 + 1] - g0[f0]) * idx0;
+          T acc = (g0[f0 + 1] - g0[f0]) * idx[0];
           if (M.ndim > 1) {
             const T* g1 = F1 + ((size_t)b * NV + v) * nf1;
-            acc += (g1[f1 + nx0] - g1[f1]) * idx1;
+            acc += (g1[f1 + nx0] - g1[f1]) * idx[1];
           }
           if (M.ndim > 2) {
             const T* g2 = F2 + ((size_t)b * NV + v) * nf2;
-            acc += (g2[f2 + (size_t)nx0 * nx1] - g2[f2]) * idx2;
+            acc += (g2[f2 + (size_t)nx0 * nx1] - g2[f2]) * idx[2];
           }
-          size_t at = (size_t)v * vs + (size_t)b * M.ncell + c;
+          const size_t at = (size_t)v * vs + (size_t)b * M.ncell + c;
           T ut = Uk[at] - dt * acc;
           if (v == 8) ut = ut * damp;
           un[v] = sp.plain ? ut : a * U0[at] + bb * ut;
@@ -190,87 +202,74 @@ __global__ void __launch_bounds__(256) k_update(DevMesh M, const T* U0,
         out[(size_t)v * vs + (size_t)b * M.ncell + c] = un[v];
         if (sp.has2) out2[(size_t)v * vs + (size_t)b * M.ncell + c] = u2n[v];
       }
-      if (sp.epilogue) accumulate_cell(M, un, gamma, dx, p, sp.pressure_ff != 0);
+      if (sp.epilogue)
+        cfl_terms_nd(M.ndim, un, lc[LC_G], (T)lc[LC_G], sp.pressure_ff != 0, (float)lc[LC_GM1],
+                     idx, smx, cmx);
     }
-    if (sp.epilogue) block_reduce_store(p, M.part + (size_t)b * NPART);
+    if (sp.epilogue) cta_max2(smx, cmx, true, M.part + (size_t)b * NPART);
   }
 }
 
 // ------------------------------------------------------------------ k_cfl
 
+// CFL maxima of every block of U, a CTA per chunk of `chunk` cells of a block
+// (one chunk a block: stored; else merged into part, zeroed before).  Only the two
+// maxima are reduced, and 1/dx and the terms shared by the directions are formed
+// once.
 template <class T>
-__global__ void __launch_bounds__(256) k_cfl(DevMesh M, const T* __restrict__ U, int ff) {
+__global__ void __launch_bounds__(256) k_cfl(DevMesh M, const T* __restrict__ U, int ff,
+                                             int nchunk, int chunk) {
   const size_t vs = (size_t)M.nblocks * M.ncell;
-  for (int b = blockIdx.x; b < M.nblocks; b += gridDim.x) {
-    const int* bi = M.blk + b * 5;
-    const int q = bi[0], L = bi[1];
-    const double* dxl = M.dx + (q * MAXLEV + L) * 3;
-    double dx[3] = {dxl[0], dxl[1], dxl[2]};
-    Partial p;
-    partial_zero(p);
-    for (int c = threadIdx.x; c < M.ncell; c += blockDim.x) {
+  const size_t nitem = (size_t)M.nblocks * nchunk;
+  for (size_t item = blockIdx.x; item < nitem; item += gridDim.x) {
+    const int b = (int)(item / nchunk), c0 = (int)(item - (size_t)b * nchunk) * chunk;
+    const int q = M.blk[b * 5], L = M.blk[b * 5 + 1];
+    const double* dx = M.dx + (q * MAXLEV + L) * 3;
+    const T idx[3] = {(T)(1.0 / dx[0]), (T)(1.0 / dx[1]), (T)(1.0 / dx[2])};
+    const double gamma = M.gamma[q];
+    T smx = T(0), cmx = T(0);
+    const int c1 = c0 + chunk < M.ncell ? c0 + chunk : M.ncell;
+#pragma unroll 2
+    for (int c = c0 + threadIdx.x; c < c1; c += blockDim.x) {
       T u[NV];
       read_cell(M, U, vs, b, c, u);
-      accumulate_cell(M, u, M.gamma[q], dx, p, ff != 0);
+      cfl_terms_nd(M.ndim, u, gamma, (T)gamma, ff != 0, (float)(gamma - 1.0), idx, smx, cmx);
     }
-    block_reduce_store(p, M.part + (size_t)b * NPART);
+    cta_max2(smx, cmx, nchunk > 1, M.part + (size_t)b * NPART);
   }
 }
 
 // ------------------------------------------------------------------ finalize
 
-__global__ void __launch_bounds__(256) k_finalize(DevMesh M, double courant, int advance) {
+// per instance: the maxima over its blocks, the clock and the next dt and c_h
+// (18,304 blocks of one instance: 163 us with 256 threads that also summed the
+// nine unused partials)
+__global__ void __launch_bounds__(1024) k_finalize(DevMesh M, double courant, int advance) {
   const int q = blockIdx.x;
   if (q >= M.ninst) return;
-  __shared__ double sh[8][NPART];
-  double smax = 0.0, chm = 0.0, sum[NV];
-#pragma unroll
-  for (int v = 0; v < NV; v++) sum[v] = 0.0;
-  const int b0 = M.inst_start[q], b1 = M.inst_start[q + 1];
-  for (int n = b0 + threadIdx.x; n < b1; n += blockDim.x) {
-    int b = M.inst_blocks[n];
-    const double* pb = M.part + (size_t)b * NPART;
-    const int L = M.blk[b * 5 + 1];
-    const double* dxl = M.dx + (q * MAXLEV + L) * 3;
-    double dv = dxl[0];
-    for (int d = 1; d < M.ndim; d++) dv *= dxl[d];
-    smax = fmax(smax, pb[0]);
-    chm = fmax(chm, pb[1]);
-#pragma unroll
-    for (int v = 0; v < NV; v++) sum[v] += pb[2 + v] * dv;
+  __shared__ double out[2];
+  double smax = 0.0, chm = 0.0;
+  const int b1 = M.inst_start[q + 1];
+#pragma unroll 4
+  for (int n = M.inst_start[q] + threadIdx.x; n < b1; n += blockDim.x) {
+    const double2 p =
+        *reinterpret_cast<const double2*>(M.part + (size_t)M.inst_blocks[n] * NPART);
+    smax = fmax(smax, p.x);
+    chm = fmax(chm, p.y);
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, o));
-    chm = fmax(chm, __shfl_xor_sync(0xffffffffu, chm, o));
-#pragma unroll
-    for (int v = 0; v < NV; v++) sum[v] += __shfl_xor_sync(0xffffffffu, sum[v], o);
-  }
-  if (lane == 0) {
-    sh[warp][0] = smax;
-    sh[warp][1] = chm;
-#pragma unroll
-    for (int v = 0; v < NV; v++) sh[warp][2 + v] = sum[v];
-  }
-  __syncthreads();
+  cta_max2(smax, chm, false, out);
   if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); w++) {
-      sh[0][0] = fmax(sh[0][0], sh[w][0]);
-      sh[0][1] = fmax(sh[0][1], sh[w][1]);
-      for (int v = 0; v < NV; v++) sh[0][2 + v] += sh[w][2 + v];
-    }
     InstRT r = M.rt[q];
     if (advance) {
       if (r.dt > 0.0 && r.dt >= r.t_end - r.t) r.t = r.t_end;
       else r.t += r.dt;
     }
-    double d = courant / sh[0][0];
+    double d = courant / out[0];
     double left = r.t_end - r.t;
     if (left <= 0.0) d = 0.0;
     else if (d >= left) d = left;
     r.dt = d;
-    r.ch = sh[0][1];
+    r.ch = out[1];
     M.rt[q] = r;
   }
 }
@@ -433,31 +432,37 @@ StageParams make_stage_params(const amrvac_state* s, int k, int epilogue) {
   return sp;
 }
 
-// per-(instance, level) stage constants of the fused kernels from InstRT and
-// the level's cell size (one thread per level)
-__global__ void k_level_consts(DevMesh M, double glm_alpha, int glm, double c, double c2) {
-  const int q = blockIdx.x, L = threadIdx.x;
+struct StageSteps {
+  double c[MAXSTAGE], c2[MAXSTAGE];
+};
+
+// per-(stage, instance, level) constants from InstRT and the level's cell size
+// (one thread per level; CTA y the stage k0 + y): c dt and its psi damping factor
+// (float bulk: exp of the float-rounded argument), and the same for the second
+// output's c2 dt
+__global__ void k_level_consts(DevMesh M, double glm_alpha, int glm, int k0, StageSteps ss) {
+  const int q = blockIdx.x, L = threadIdx.x, k = k0 + blockIdx.y;
   if (q >= M.ninst || L >= MAXLEV) return;
   const InstRT rt = M.rt[q];
   const double* dx = M.dx + (q * MAXLEV + L) * 3;
-  double dxmin = fmin(dx[0], dx[1]);
-  if (M.ndim == 3) dxmin = fmin(dxmin, dx[2]);
+  double dxmin = dx[0];
+  for (int d = 1; d < M.ndim; d++) dxmin = fmin(dxmin, dx[d]);
   const double g = M.gamma[q];
-  float* f = M.lcf + (q * MAXLEV + L) * LC_N;
-  double* d = M.lcd + (q * MAXLEV + L) * LC_N;
-  // the stage's Euler step c dt and its psi damping factor (float bulk: exp of
-  // the float-rounded argument); the same for the second output's c2 dt
-  const double dt1 = c * rt.dt, dt2 = c2 * rt.dt;
+  const size_t at = (((size_t)k * M.ninst + q) * MAXLEV + L) * LC_N;
+  float* f = M.lcf + at;
+  double* d = M.lcd + at;
+  const double dt1 = ss.c[k] * rt.dt, dt2 = ss.c2[k] * rt.dt;
+  const double a1 = -glm_alpha * rt.ch * dt1 / dxmin, a2 = -glm_alpha * rt.ch * dt2 / dxmin;
   d[LC_DT] = dt1;
   f[LC_DT] = (float)dt1;
   d[LC_CH] = rt.ch;
   f[LC_CH] = (float)rt.ch;
-  d[LC_DAMP] = glm ? exp(-glm_alpha * rt.ch * dt1 / dxmin) : 1.0;
-  f[LC_DAMP] = glm ? expf((float)(-glm_alpha * rt.ch * dt1 / dxmin)) : 1.0f;
+  d[LC_DAMP] = glm ? exp(a1) : 1.0;
+  f[LC_DAMP] = glm ? expf((float)a1) : 1.0f;
   d[LC_DT2] = dt2;
   f[LC_DT2] = (float)dt2;
-  d[LC_DAMP2] = glm ? exp(-glm_alpha * rt.ch * dt2 / dxmin) : 1.0;
-  f[LC_DAMP2] = glm ? expf((float)(-glm_alpha * rt.ch * dt2 / dxmin)) : 1.0f;
+  d[LC_DAMP2] = glm ? exp(a2) : 1.0;
+  f[LC_DAMP2] = glm ? expf((float)a2) : 1.0f;
   for (int e = 0; e < 3; e++) {
     d[LC_DX + e] = dx[e];
     f[LC_DX + e] = (float)dx[e];
@@ -472,30 +477,49 @@ __global__ void k_level_consts(DevMesh M, double glm_alpha, int glm, double c, d
   f[LC_GM1] = (float)(g - 1.0);
 }
 
-int launch_level_consts(amrvac_state* s, int k) {
-  const StageCoeffs co = stage_coeffs(s->cfg.time, k);
-  k_level_consts<<<s->ninst, MAXLEV, 0, s->stream>>>(s->mesh, s->cfg.glm_alpha, s->cfg.glm,
-                                                      co.c, co.c2);
+// constants of stages k0 .. k0 + nk - 1 (dt and c_h stay the same within a step:
+// a step computes those of all its stages in one launch)
+int launch_level_consts(amrvac_state* s, int k0, int nk) {
+  StageSteps ss{};
+  for (int k = k0; k < k0 + nk; k++) {
+    const StageCoeffs co = stage_coeffs(s->cfg.time, k);
+    ss.c[k] = co.c;
+    ss.c2[k] = co.c2;
+  }
+  k_level_consts<<<dim3(s->ninst, nk), MAXLEV, 0, s->stream>>>(s->mesh, s->cfg.glm_alpha,
+                                                                s->cfg.glm, k0, ss);
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
+}
+
+DevMesh stage_mesh(const amrvac_state* s, int k) {
+  DevMesh M = s->mesh;
+  M.lcf += (size_t)k * s->ninst * MAXLEV * LC_N;
+  M.lcd += (size_t)k * s->ninst * MAXLEV * LC_N;
+  return M;
 }
 
 template <class T> static int plain_stage_t(amrvac_state* s, int k, int epilogue) {
   const StageBuffers sb = stage_buffers(s->cfg.time, k);
   const int uin = sb.uin;
   StageParams sp = make_stage_params(s, k, epilogue);
-  const DevMesh& M = s->mesh;
+  const DevMesh M = stage_mesh(s, k);
   size_t work = s->npad * s->nblocks;
-  k_prim<T><<<grid_for(work, 256), 256, 0, s->stream>>>(M, (const T*)s->U[uin], (T*)s->W,
+  int nt = threads_for(work);
+  k_prim<T><<<grid_for(work, nt), nt, 0, s->stream>>>(M, (const T*)s->U[uin], (T*)s->W,
                                                         s->P[0], s->P[1], s->P[2], sp);
-  for (int d = 0; d < s->ndim; d++)
-    k_flux<T><<<grid_for(s->nface[d] * s->nblocks, 256), 256, 0, s->stream>>>(
+  for (int d = 0; d < s->ndim; d++) {
+    work = s->nface[d] * s->nblocks;
+    nt = threads_for(work);
+    k_flux<T><<<grid_for(work, nt), nt, 0, s->stream>>>(
         M, (const T*)s->W, (T*)s->F[d], d, s->P[0], s->P[1], s->P[2], sp);
-  int grid = s->nblocks < 152 * 16 ? s->nblocks : 152 * 16;
-  k_update<T><<<grid, 256, 0, s->stream>>>(
+  }
+  nt = threads_for((size_t)s->ncell * s->nblocks);
+  const int nchunk = (s->ncell + nt - 1) / nt;
+  k_update<T><<<grid_for((size_t)nchunk * s->nblocks, 1), nt, 0, s->stream>>>(
       M, (const T*)s->U[sb.u0], (const T*)s->U[uin],
       sb.u2 >= 0 ? (const T*)s->U[sb.u2] : nullptr, (T*)s->U[sb.out],
       sb.out2 >= 0 ? (T*)s->U[sb.out2] : nullptr, (const T*)s->F[0], (const T*)s->F[1],
-      (const T*)s->F[2], sp);
+      (const T*)s->F[2], nchunk, sp);
   if (cudaPeekAtLastError() != cudaSuccess) return -1;
   return 2 + s->ndim;
 }
@@ -506,17 +530,26 @@ int launch_plain_stage(amrvac_state* s, int k, int epilogue) {
 }
 
 int launch_cfl_partials(amrvac_state* s, int buffer) {
-  int grid = s->nblocks < 152 * 16 ? s->nblocks : 152 * 16;
+  // a CTA per block, or per 256 cells where the blocks alone would not fill the chip
+  const int nchunk = s->nblocks < 152 * 8 ? (s->ncell + 255) / 256 : 1;
+  const int chunk = nchunk > 1 ? 256 : s->ncell;
+  const int grid = grid_for((size_t)nchunk * s->nblocks, 1);
+  if (nchunk > 1 && cudaMemsetAsync(s->mesh.part, 0, sizeof(double) * NPART * s->nblocks,
+                                    s->stream) != cudaSuccess)
+    return -1;
   const int ff = s->cfg.precision == AMRVAC_FP32_BULK && s->cfg.pressure == AMRVAC_PRESSURE_FF;
   if (s->cfg.precision == AMRVAC_FP64)
-    k_cfl<double><<<grid, 256, 0, s->stream>>>(s->mesh, (const double*)s->U[buffer], 0);
+    k_cfl<double><<<grid, 256, 0, s->stream>>>(s->mesh, (const double*)s->U[buffer], 0, nchunk,
+                                               chunk);
   else
-    k_cfl<float><<<grid, 256, 0, s->stream>>>(s->mesh, (const float*)s->U[buffer], ff);
+    k_cfl<float><<<grid, 256, 0, s->stream>>>(s->mesh, (const float*)s->U[buffer], ff, nchunk,
+                                              chunk);
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 
 int launch_finalize(amrvac_state* s, int advance) {
-  k_finalize<<<s->ninst, 256, 0, s->stream>>>(s->mesh, s->cfg.courant, advance);
+  const int nt = s->nblocks >= 1024 * s->ninst ? 1024 : 256;
+  k_finalize<<<s->ninst, nt, 0, s->stream>>>(s->mesh, s->cfg.courant, advance);
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 

@@ -1,100 +1,96 @@
-// Per-block partials of the CFL reduction and the conservation sums, and their
-// deterministic CTA reduction (fixed shuffle tree, fixed warp order).
+// CFL terms of a cell and the reductions of their maxima: per block into part
+// (fixed layout, maxima are independent of the order), per instance in k_finalize.
 #pragma once
 
 #include "physics.cuh"
 
 namespace amrvac {
 
-struct Partial {
-  double smax, chm, sum[NV];
-};
-
-__device__ __forceinline__ void partial_zero(Partial& p) {
-  p.smax = 0.0;
-  p.chm = 0.0;
-#pragma unroll
-  for (int v = 0; v < NV; v++) p.sum[v] = 0.0;
-}
-
-// deterministic block reduction (fixed shuffle tree + fixed warp order) of a
-// Partial; thread 0 writes it to part[b]
-static __device__ void block_reduce_store(Partial& p, double* part_b) {
-  __shared__ double sh[32][NPART];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    p.smax = fmax(p.smax, __shfl_xor_sync(0xffffffffu, p.smax, o));
-    p.chm = fmax(p.chm, __shfl_xor_sync(0xffffffffu, p.chm, o));
-#pragma unroll
-    for (int v = 0; v < NV; v++) p.sum[v] += __shfl_xor_sync(0xffffffffu, p.sum[v], o);
-  }
-  if (lane == 0) {
-    sh[warp][0] = p.smax;
-    sh[warp][1] = p.chm;
-#pragma unroll
-    for (int v = 0; v < NV; v++) sh[warp][2 + v] = p.sum[v];
-  }
-  __syncthreads();
-  if (threadIdx.x < NPART) {
-    const int nw = blockDim.x >> 5;
-    double acc = sh[0][threadIdx.x];
-    for (int w = 1; w < nw; w++) {
-      double x = sh[w][threadIdx.x];
-      acc = threadIdx.x < 2 ? fmax(acc, x) : acc + x;
-    }
-    part_b[threadIdx.x] = threadIdx.x < 2 + NV ? acc : 0.0;
-  }
-  __syncthreads();
-}
-
-// per-cell CFL terms: sum_d (|v_d| + c_f,d)/dx_d and max_d (|v_d| + c_f,d), in the
-// bulk precision (inverse cell sizes precomputed); conservation sums in double
-template <class T>
-__device__ __forceinline__ void accumulate_cell(const DevMesh& M, const T* u, double gamma,
-                                                const double* dx, Partial& p, bool ff = false) {
-  // CFL terms only (the conservation sums are reduced on demand by k_sums);
-  // ff: float-float pressure recovery of FP32-bulk states
+// CFL terms of a conserved cell: running max of sum_d (|v_d| + c_f,d)/dx_d and
+// of |v_d| + c_f,d.  The fast speed of each direction is the cancellation-free
+// form with 1/rho, a^2 = gamma p/rho and b^2 = B^2/rho shared by the
+// directions (b_t^2 = b^2 - B_d^2/rho, kept >= 0).
+template <class T, int DIM>
+__device__ __forceinline__ void cfl_terms(const T* u, double gammad, T g, bool ff, float gm1f,
+                                          const T* idx, T& smx, T& cmx) {
   T w[NV];
-  cons2prim(gamma, u, w, ff, (float)(gamma - 1.0));
-  T s = T(0), cm = T(0);
-  for (int d = 0; d < M.ndim; d++) {
-    T spd = fabs(w[1 + d]) + fast_speed((T)gamma, w, d);
-    s += spd / (T)dx[d];
-    cm = fmax(cm, spd);
+  cons2prim(gammad, u, w, ff, gm1f);
+  const T ir = rcp_T(w[0]);
+  const T a2 = g * w[4] * ir;
+  const T bb = (w[5] * w[5] + w[6] * w[6] + w[7] * w[7]) * ir;
+  const T dd = a2 - bb, sab = a2 + bb;
+  T s = T(0);
+#pragma unroll
+  for (int d = 0; d < DIM; d++) {
+    const T bt = bb - w[5 + d] * w[5 + d] * ir;
+    const T bt2 = gt0(bt) ? bt : T(0);  // no negative rounding
+    const T cf = sqrt_T(T(0.5) * (sab + sqrt_T(dd * dd + T(4) * a2 * bt2)));
+    const T spd = fabs(w[1 + d]) + cf;
+    s += spd * idx[d];
+    cmx = fmax(cmx, spd);
   }
-  p.smax = fmax(p.smax, (double)s);
-  p.chm = fmax(p.chm, (double)cm);
+  smx = fmax(smx, s);
 }
 
-// same reduction with caller-provided shared scratch red[>= nwarps][NPART]
-__device__ __forceinline__ void block_reduce_red(double (*red)[NPART], Partial& p, double* part_b) {
+// Per-warp maxima of the owners' two CFL terms merged into part_b[0..1] with
+// atomicMax on the bit patterns (order-independent for values >= 0; NaN is
+// dropped as fmax drops it).  part_b[0..1] are zeroed before the block's first
+// barrier, the atomics come after its last one.
+__device__ __forceinline__ void warp_max2_atomic(double smax, double cmax, double* part_b) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, o));
+    cmax = fmax(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    if (smax == smax)
+      atomicMax((unsigned long long*)&part_b[0], (unsigned long long)__double_as_longlong(smax));
+    if (cmax == cmax)
+      atomicMax((unsigned long long*)&part_b[1], (unsigned long long)__double_as_longlong(cmax));
+  }
+}
+
+// the same of the two CFL terms for a number of dimensions known at run time
+template <class T>
+__device__ __forceinline__ void cfl_terms_nd(int nd, const T* u, double gammad, T g, bool ff,
+                                             float gm1f, const T* idx, T& smx, T& cmx) {
+  if (nd == 3) cfl_terms<T, 3>(u, gammad, g, ff, gm1f, idx, smx, cmx);
+  else if (nd == 2) cfl_terms<T, 2>(u, gammad, g, ff, gm1f, idx, smx, cmx);
+  else cfl_terms<T, 1>(u, gammad, g, ff, gm1f, idx, smx, cmx);
+}
+
+// CTA maximum of the two CFL terms (every thread of the CTA takes part): thread 0
+// stores it to part_b[0..1], or merges it there when several CTAs share a block
+// (merge: part_b zeroed before; values >= 0, NaN dropped as fmax drops it)
+__device__ __forceinline__ void cta_max2(double smax, double cmax, bool merge, double* part_b) {
+  __shared__ double sh[32][2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    p.smax = fmax(p.smax, __shfl_xor_sync(0xffffffffu, p.smax, o));
-    p.chm = fmax(p.chm, __shfl_xor_sync(0xffffffffu, p.chm, o));
-#pragma unroll
-    for (int v = 0; v < NV; v++) p.sum[v] += __shfl_xor_sync(0xffffffffu, p.sum[v], o);
+    smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, o));
+    cmax = fmax(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
   }
-  __syncthreads();
   if (lane == 0) {
-    red[warp][0] = p.smax;
-    red[warp][1] = p.chm;
-#pragma unroll
-    for (int v = 0; v < NV; v++) red[warp][2 + v] = p.sum[v];
+    sh[warp][0] = smax;
+    sh[warp][1] = cmax;
   }
   __syncthreads();
-  if (threadIdx.x < NPART) {
-    const int nw = blockDim.x >> 5;
-    double acc = red[0][threadIdx.x];
-    for (int w = 1; w < nw; w++) {
-      double x = red[w][threadIdx.x];
-      acc = threadIdx.x < 2 ? fmax(acc, x) : acc + x;
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < (int)(blockDim.x >> 5); w++) {
+      smax = fmax(smax, sh[w][0]);
+      cmax = fmax(cmax, sh[w][1]);
     }
-    part_b[threadIdx.x] = threadIdx.x < 2 + NV ? acc : 0.0;
+    if (!merge) {
+      part_b[0] = smax;
+      part_b[1] = cmax;
+    } else {
+      if (smax == smax)
+        atomicMax((unsigned long long*)&part_b[0], (unsigned long long)__double_as_longlong(smax));
+      if (cmax == cmax)
+        atomicMax((unsigned long long*)&part_b[1], (unsigned long long)__double_as_longlong(cmax));
+    }
   }
-  __syncthreads();
+  __syncthreads();  // sh is reused
 }
 
 }  // namespace amrvac

@@ -145,12 +145,10 @@ template <class T> int reflux_t(amrvac_state* s, int k) {
                                                     s->d_glist, s->ngen);
       n++;
     }
-    if (launch_level_consts(s, k) < 0) return -1;
-    n++;
   }
   if (s->nrlist > 0) {
     const int g = s->nrlist < 152 * 8 ? s->nrlist : 152 * 8;
-    k_reflux<T><<<g, 256, 0, s->stream>>>(s->mesh, (T*)s->U[sb.out],
+    k_reflux<T><<<g, 256, 0, s->stream>>>(stage_mesh(s, k), (T*)s->U[sb.out],
                                            sb.out2 >= 0 ? (T*)s->U[sb.out2] : nullptr,
                                            s->d_rlist, s->nrlist, sp);
     n++;

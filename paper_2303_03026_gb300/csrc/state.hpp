@@ -162,7 +162,8 @@ int launch_plain_stage(amrvac_state* s, int k, int epilogue);
 int launch_cfl_partials(amrvac_state* s, int buffer);
 int launch_finalize(amrvac_state* s, int advance);
 int launch_sums(amrvac_state* s, int buffer);
-int launch_level_consts(amrvac_state* s, int k);
+int launch_level_consts(amrvac_state* s, int k0, int nk);
+DevMesh stage_mesh(const amrvac_state* s, int k);  // with stage k's constants
 int launch_fix_small(amrvac_state* s, int buffer);
 int launch_reflux(amrvac_state* s, int k);
 int launch_fill_ghosts(amrvac_state* s, int buffer, void* out);
