@@ -21,10 +21,11 @@ SOURCES = ["api.cu", "plain.cu", "fused.cu", "noalloc.cu", "fix.cu", "reflux.cu"
 # the fused kernel source is compiled once per (precision, dimension, limiter)
 # limiter groups: minmod, vanleer, koren as compile-time limiters, -1 = the
 # other two-ghost-cell limiters at run time (FP32: superbee, woodward, mcbeta; -3
-# the rest), -2 = the five-point limiters at run time
+# the rest); five points: mp5, weno5, wenoz5, wenozp5 one by one in FP32, -2 = at
+# run time in double (2D)
 FUSED_GROUPS = ([(t, d, l) for t in ("float", "double") for d in (2, 3) for l in (0, 1, 2, -1)] +
                 [("float", d, -3) for d in (2, 3)] +
-                [(t, 2, -2) for t in ("float", "double")] + [("float", 3, -2)])
+                [("float", d, l) for d in (2, 3) for l in (7, 8, 9, 11)] + [("double", 2, -2)])
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xptxas", "-v",
               "--expt-relaxed-constexpr"]

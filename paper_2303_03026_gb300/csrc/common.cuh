@@ -18,7 +18,7 @@ constexpr int MAXSTAGE = 5;  // stages of the longest scheme
 constexpr int NPART = 12;   // per-block partials: smax, chmax, sums[9], pad
 
 // the limiters that reconstruct from five cells (three ghost layers)
-__host__ __device__ inline bool five_point_limiter(int lim) {
+__host__ __device__ constexpr bool five_point_limiter(int lim) {
   return lim == AMRVAC_LIM_MP5 || lim == AMRVAC_LIM_WENO5 || lim == AMRVAC_LIM_WENOZ5 ||
          lim == AMRVAC_LIM_WENOZP5;
 }

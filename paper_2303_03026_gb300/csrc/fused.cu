@@ -27,9 +27,19 @@ bool fused_supported5(const amrvac_config* c) {
 
 template <class T, int DIM> static int by_limiter(amrvac_state* s, int k, int epilogue, int g) {
   if (five_point_limiter(s->grp_lim[g])) {
-    // the five-point limiters share one instantiation (three ghost layers;
-    // 3D in FP32 bulk only)
-    if constexpr (DIM == 2 || sizeof(T) == 4) return launch_fused_l<T, DIM, -2>(s, k, epilogue, g);
+    // three ghost layers (3D in FP32 bulk only): in FP32 one instantiation a
+    // limiter, so that its unrolled code alone is in the instruction cache; in
+    // double they share one
+    if constexpr (sizeof(T) == 4) {
+      switch (s->grp_lim[g]) {
+        case AMRVAC_LIM_MP5: return launch_fused_l<T, DIM, AMRVAC_LIM_MP5>(s, k, epilogue, g);
+        case AMRVAC_LIM_WENO5: return launch_fused_l<T, DIM, AMRVAC_LIM_WENO5>(s, k, epilogue, g);
+        case AMRVAC_LIM_WENOZ5: return launch_fused_l<T, DIM, AMRVAC_LIM_WENOZ5>(s, k, epilogue, g);
+        default: return launch_fused_l<T, DIM, AMRVAC_LIM_WENOZP5>(s, k, epilogue, g);
+      }
+    } else if constexpr (DIM == 2) {
+      return launch_fused_l<T, DIM, -2>(s, k, epilogue, g);
+    }
     return -1;
   }
   switch (s->grp_lim[g]) {

@@ -45,9 +45,12 @@ constexpr int FB = 16;          // block edge handled by the fused kernel
 // (the 32 faces on the +x/+y block boundary).  The 2D kernel uses the same
 // roles with threads 0 .. 64G-1 copying and converting the halo.
 constexpr int FT = FB * FB + FB;
-// ghost layers of a tile for a limiter template value (-2: the five-point
-// limiters, chosen at run time)
-__host__ __device__ constexpr int tile_ghosts(int lim) { return lim == -2 ? NG5 : NG; }
+// limiter template values: a limiter, or in double -2 = the five-point ones at run
+// time (-1, -3: see fused.cu); ghost layers of the tile
+__host__ __device__ constexpr bool five_tile(int lim) {
+  return lim == -2 || (lim >= 0 && five_point_limiter(lim));
+}
+__host__ __device__ constexpr int tile_ghosts(int lim) { return five_tile(lim) ? NG5 : NG; }
 // Double with a two-ghost-cell limiter: every cell's limited slopes are
 // evaluated once (its two face states handed to the neighbouring face through
 // the face-flux array) instead of once per face, since the FP64 pipe bounds
@@ -162,11 +165,11 @@ __device__ __forceinline__ void limited_flux(T* wl, T* wr, CL cl, CR cr, int glm
 
 // face flux from the six-cell stencil S(v, t), t = 0..5 for cells f-3 .. f+2
 // around the face f-1/2, with a five-point limiter lim (lam: wenozp5's lambda)
-template <class T, int D, int FLUX, class Acc>
+template <class T, int D, int LIM, int FLUX, class Acc>
 __device__ __forceinline__ void stencil_flux5(Acc S, int lim, T lam, int glm,
                                               const FaceConst<T>& fc, T* f) {
   if constexpr (sizeof(T) == 4) {
-    stencil_flux5_f2<D, FLUX>(S, lim, lam, FaceConst2{fc.g, fc.ig1, fc.ch, fc.hich, glm}, f);
+    stencil_flux5_f2<D, LIM, FLUX>(S, lam, FaceConst2{fc.g, fc.ig1, fc.ch, fc.hich, glm}, f);
   } else {
     T wl[NV], wr[NV];
 #pragma unroll
@@ -387,8 +390,8 @@ __global__ void __launch_bounds__(256)
 // mirrored reads of symmetric walls are compiled in (they are runtime-uniform
 // branches that still cost the hot loop registers and scheduling freedom, so
 // the lean instantiation runs otherwise)
-// LIM -2: the five-point limiters (runtime limiter, three ghost layers: a
-// 6-plane ring of 22 x 22 planes and 192 halo cells a plane, one CTA per SM)
+// Five-point limiters: three ghost layers (a 6-plane ring of 22 x 22 planes and
+// 192 halo cells a plane, one CTA per SM)
 template <class T, int DIM, int LIM, int FLUX, bool FULL>
 __global__ void __launch_bounds__(fused_threads<T, LIM>(), 1)
     k_fused(DevMesh M, const T* U0, const T* __restrict__ Uk, const T* U2, T* out, T* out2,
@@ -396,7 +399,7 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), 1)
             int* __restrict__ counter, StageParams sp) {
   extern __shared__ __align__(16) unsigned char smraw[];
   static_assert(DIM == 3, "16x16 blocks in 2D use k_fused2d");
-  static_assert(sizeof(T) == 8 || LIM == -2, "FP32 with two ghost layers: k_fused_f2");
+  static_assert(sizeof(T) == 8 || five_tile(LIM), "FP32 with two ghost layers: k_fused_f2");
   constexpr int G = tile_ghosts(LIM);
   using Smem = FusedSmem<T, DIM, G>;
   Smem& S = *reinterpret_cast<Smem*>(smraw);
@@ -607,7 +610,7 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), 1)
 #pragma unroll
         for (int t = 0; t < 6; t++) sl6[t] = (zc - 3 + t + 2 * NSLOT) % NSLOT;
         auto acc = [&](int v, int t) -> T { return zcell(sl6[t], v); };
-        stencil_flux5<T, 2, FLUX>(acc, sp.limiter, lam[2], sp.glm, fc, f);
+        stencil_flux5<T, 2, LIM, FLUX>(acc, sp.limiter, lam[2], sp.glm, fc, f);
       }
     };
 
@@ -672,14 +675,14 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), 1)
         T f[NV];
         auto ax = [&](int v, int t) -> T { return S.plane[sl][v][fxr + G][fxc + t]; };
         auto ay = [&](int v, int t) -> T { return S.plane[sl][v][fyr + t][fyc + G]; };
-        stencil_flux5<T, 0, FLUX>(ax, sp.limiter, lam[0], sp.glm, fc, f);
+        stencil_flux5<T, 0, LIM, FLUX>(ax, sp.limiter, lam[0], sp.glm, fc, f);
 #pragma unroll
         for (int v = 0; v < NV; v++) S.fx[fb][v][fxr][fxc] = f[v];
         if (FULL && sp.reflux) {
           const int face = owner ? (x == 0 ? 0 : -1) : 1;
           if (face >= 0 && nb[face] <= -3) keep_face_flux(M, nb[face], z * FB + fxr, f);
         }
-        stencil_flux5<T, 1, FLUX>(ay, sp.limiter, lam[1], sp.glm, fc, f);
+        stencil_flux5<T, 1, LIM, FLUX>(ay, sp.limiter, lam[1], sp.glm, fc, f);
 #pragma unroll
         for (int v = 0; v < NV; v++) S.fy[fb][v][fyr][fyc] = f[v];
         if (FULL && sp.reflux) {
@@ -754,7 +757,7 @@ namespace amrvac {
 // the kernel of a dimension and precision (the others are not instantiated), its
 // threads and shared memory
 template <class T, int DIM, int LIM, int FLUX, bool FULL> struct FusedKernel {
-  static constexpr bool F2 = sizeof(T) == 4 && LIM != -2;
+  static constexpr bool F2 = sizeof(T) == 4 && !five_tile(LIM);
   static constexpr int threads = F2 ? F2_T : fused_threads<T, LIM>();
   static constexpr auto kernel() {
     if constexpr (F2 && DIM == 3) return &k_fused_f2<LIM, FLUX, FULL>;
@@ -773,7 +776,7 @@ template <class T, int DIM, int LIM, int FLUX, bool FULL> struct FusedKernel {
 template <class T, int DIM, int LIM, int FLUX, bool FULL>
 static int launch_one(amrvac_state* s, int k, const T* U0, const T* Uk, const T* U2, T* out, T* out2,
                       const int* work, int nwork, int* counter, StageParams sp) {
-  static_assert(DIM == 2 || LIM != -2 || sizeof(T) == 4,
+  static_assert(DIM == 2 || !five_tile(LIM) || sizeof(T) == 4,
                 "five-point limiters in 3D: FP32 bulk only (a double 6-plane ring does not fit)");
   using K = FusedKernel<T, DIM, LIM, FLUX, FULL>;
   const auto kern = K::kernel();

@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), sizeof(T) == 4 ? 2 : 
               const int* __restrict__ work, int nwork, const T* __restrict__ gslab,
               int* __restrict__ counter, StageParams sp) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  static_assert(sizeof(T) == 8 || LIM == -2, "FP32 with two ghost layers: k_fused2d_f2");
+  static_assert(sizeof(T) == 8 || five_tile(LIM), "FP32 with two ghost layers: k_fused2d_f2");
   constexpr int G = tile_ghosts(LIM);
   Fused2dSmem<T, G>& S = *reinterpret_cast<Fused2dSmem<T, G>*>(smraw);
   constexpr int SLAB_FACE = NV * G * FB;  // one face: [v][layer][t1]
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), sizeof(T) == 4 ? 2 : 
         // five-point limiters: six-cell stencils (three ghost layers)
         const int lv = M.blk[b * 5 + 1];
         const T lamx = (T)M.wzlam[(q * MAXLEV + lv) * 3], lamy = (T)M.wzlam[(q * MAXLEV + lv) * 3 + 1];
-        stencil_flux5<T, 0, FLUX>(ax, sp.limiter, lamx, sp.glm, fc, f);
+        stencil_flux5<T, 0, LIM, FLUX>(ax, sp.limiter, lamx, sp.glm, fc, f);
 #pragma unroll
         for (int v = 0; v < NV; v++) S.fx[v][fxr][fxc] = f[v];
         if (FULL && sp.reflux) {
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), sizeof(T) == 4 ? 2 : 
           const int code = face >= 0 ? M.nbr[b * 6 + face] : 0;
           if (code == NBR_GENERAL) keep_face_flux(M, -3 - M.gface[b * 6 + face], fxr, f);
         }
-        stencil_flux5<T, 1, FLUX>(ay, sp.limiter, lamy, sp.glm, fc, f);
+        stencil_flux5<T, 1, LIM, FLUX>(ay, sp.limiter, lamy, sp.glm, fc, f);
 #pragma unroll
         for (int v = 0; v < NV; v++) S.fy[v][fyr][fyc] = f[v];
         if (FULL && sp.reflux) {

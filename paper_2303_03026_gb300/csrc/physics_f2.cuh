@@ -619,20 +619,96 @@ __device__ __forceinline__ void face_flux_xy(const float2* wl, const float2* wr,
   f[8] = fpsi;
 }
 
-// Five-point limiters (mp5, weno5, wenoz5, wenozp5; lim at run time, lam the
-// wenozp5 lambda): st(v, t) for the six cells f-3 .. f+2 around the face
-// f-1/2; each face state reconstructed in float as on the plain path
-template <int D, int FLUX, class Acc>
-__device__ __forceinline__ void stencil_flux5_f2(Acc st, int lim, float lam, const FaceConst2& fc,
+// ---------------------------------------------------------------- five points
+// Both states of a face from its six cells (lane x: the left state, from cells
+// 0 .. 4; lane y: the right state, the mirrored stencil 5 .. 1), as increments
+// to the cell value next to the face: with s1 .. s4 the differences along the
+// stencil every formula of physics.cuh becomes free of the cell value itself
+// (and exact on constant data).  Minima and selects are per lane.
+__device__ __forceinline__ float minmod_f(float a, float b) {
+  return fmaxf(fminf(a, b), 0.f) + fminf(fmaxf(a, b), 0.f);
+}
+__device__ __forceinline__ float minmod4_f(float w, float x, float y, float z) {
+  return fmaxf(fminf(fminf(w, x), fminf(y, z)), 0.f) + fminf(fmaxf(fmaxf(w, x), fmaxf(y, z)), 0.f);
+}
+
+// the limited part of mp5 (one lane): q = the fifth-order increment
+__device__ __forceinline__ float mp5_clip(float q, float s1, float s2, float s3, float s4) {
+  const float djm = s2 - s1, dj = s3 - s2, djp = s4 - s3;
+  const float dp = minmod4_f(4.f * dj - djp, 4.f * djp - dj, dj, djp);
+  const float dm = minmod4_f(4.f * dj - djm, 4.f * djm - dj, dj, djm);
+  const float ul = 4.f * s2, md = 0.5f * s3 - 0.5f * dp, lc = 0.5f * s2 + (4.f / 3.f) * dm;
+  const float lo = fmaxf(fminf(fminf(0.f, s3), md), fminf(fminf(0.f, ul), lc));
+  const float hi = fminf(fmaxf(fmaxf(0.f, s3), md), fmaxf(fmaxf(0.f, ul), lc));
+  return q + minmod_f(lo - q, hi - q);
+}
+
+template <int LIM>
+__device__ __forceinline__ float2 recon5_pair(const float* c, float lam) {
+  if constexpr (LIM == AMRVAC_LIM_WENOZP5) {
+    // weights from a near-cancellation: the explicitly rounded scalar form
+    return make_float2(weno5_face(2, c[0], c[1], c[2], c[3], c[4], lam),
+                       weno5_face(2, c[5], c[4], c[3], c[2], c[1], lam));
+  } else {
+    const float2 C = make_float2(c[2], c[3]);
+    const float d0 = c[1] - c[0], d1 = c[2] - c[1], d2 = c[3] - c[2], d3 = c[4] - c[3],
+                d4 = c[5] - c[4];
+    const float2 s1 = make_float2(d0, -d4), s2 = make_float2(d1, -d3), s3 = make_float2(d2, -d2),
+                 s4 = make_float2(d3, -d1);
+    if constexpr (LIM == AMRVAC_LIM_MP5) {
+      // (2 a - 13 b + 47 c + 27 d - 3 e)/60 - c
+      float2 q = fma2(sp2(-2.f / 60.f), s1, mul2(sp2(11.f / 60.f), s2));
+      q = fma2(sp2(24.f / 60.f), s3, fma2(sp2(-3.f / 60.f), s4, q));
+      // kept where it lies between c and c + minmod(s3, 4 s2)
+      const float mx = minmod_f(s3.x, 4.f * s2.x), my = minmod_f(s3.y, 4.f * s2.y);
+      const bool kx = q.x * (q.x - mx) <= 0.f, ky = q.y * (q.y - my) <= 0.f;
+      if (!kx) q.x = mp5_clip(q.x, s1.x, s2.x, s3.x, s4.x);
+      if (!ky) q.y = mp5_clip(q.y, s1.y, s2.y, s3.y, s4.y);
+      return add2(C, q);
+    } else {
+      const float2 t0 = sub2(s2, s1), u0 = fma2(sp2(3.f), s2, neg2(s1));
+      const float2 t1 = sub2(s3, s2), u1 = add2(s2, s3);
+      const float2 t2 = sub2(s4, s3), u2 = fma2(sp2(-3.f), s3, s4);
+      const float2 k13 = sp2(13.f / 12.f), k14 = sp2(0.25f);
+      const float2 b0 = fma2(mul2(k13, t0), t0, mul2(mul2(k14, u0), u0));
+      const float2 b1 = fma2(mul2(k13, t1), t1, mul2(mul2(k14, u1), u1));
+      const float2 b2 = fma2(mul2(k13, t2), t2, mul2(mul2(k14, u2), u2));
+      const float2 q0 = mul2(fma2(sp2(5.f), s2, mul2(sp2(-2.f), s1)), sp2(1.f / 6.f));
+      const float2 q1 = mul2(fma2(sp2(2.f), s3, s2), sp2(1.f / 6.f));
+      const float2 q2 = mul2(fma2(sp2(4.f), s3, neg2(s4)), sp2(1.f / 6.f));
+      float2 a0, a1, a2;
+      if constexpr (LIM == AMRVAC_LIM_WENOZ5) {
+        // scaled weights (see weno5_face): a_k = d_k (bm + bm/(b_k + eps) tau)/(bm + tau)
+        const float2 eps = sp2(1e-36f), tau = abs2(sub2(b0, b2));
+        const float2 bm = add2(min2(min2(b0, b1), b2), eps);
+        // (in this order: bm tau alone may underflow)
+        const float2 iden = rcp2(add2(bm, tau));
+        a0 = mul2(sp2(0.1f), mul2(fma2(mul2(bm, rcp2(add2(b0, eps))), tau, bm), iden));
+        a1 = mul2(sp2(0.6f), mul2(fma2(mul2(bm, rcp2(add2(b1, eps))), tau, bm), iden));
+        a2 = mul2(sp2(0.3f), mul2(fma2(mul2(bm, rcp2(add2(b2, eps))), tau, bm), iden));
+      } else {
+        const float2 eps = sp2(1e-6f);
+        const float2 e0 = rcp2(add2(b0, eps)), e1 = rcp2(add2(b1, eps)), e2 = rcp2(add2(b2, eps));
+        a0 = mul2(mul2(sp2(0.1f), e0), e0);
+        a1 = mul2(mul2(sp2(0.6f), e1), e1);
+        a2 = mul2(mul2(sp2(0.3f), e2), e2);
+      }
+      const float2 num = fma2(a2, q2, fma2(a1, q1, mul2(a0, q0)));
+      return fma2(num, rcp2(add2(add2(a0, a1), a2)), C);
+    }
+  }
+}
+
+// Face flux along D with the five-point limiter LIM (lam the wenozp5 lambda):
+// st(v, t) for the six cells f-3 .. f+2 around the face f-1/2
+template <int D, int LIM, int FLUX, class Acc>
+__device__ __forceinline__ void stencil_flux5_f2(Acc st, float lam, const FaceConst2& fc,
                                                  float* f) {
   float2 w[NV];
-  // one copy of the reconstruction for the nine variables (not unrolled): the
-  // limiters' code, four of them behind the runtime switch and inlined at the
-  // three faces, otherwise overflows the instruction cache
-#pragma unroll 1
+#pragma unroll
   for (int v = 0; v < NV; v++) {
     const float c[6] = {st(v, 0), st(v, 1), st(v, 2), st(v, 3), st(v, 4), st(v, 5)};
-    w[v] = make_float2(recon5_plus<float>(lim, c, lam), recon5_minus<float>(lim, c + 1, lam));
+    w[v] = recon5_pair<LIM>(c, lam);
   }
   if (not_positive2(w)) {
 #pragma unroll
