@@ -64,6 +64,42 @@ __device__ __forceinline__ void est_cell(const DevMesh& M, const T* U, size_t vs
   }
 }
 
+// estimate of cell ci of block b in double: sum over the weighted quantities of
+// w sqrt(num/den)
+template <class T>
+__device__ double est_double(const DevMesh& M, const T* U, size_t vs, int b, const int* ci,
+                             const EstWeights& ew, double g) {
+  const int nq = ew.prim ? NV : 1;
+  double q0[NV], num[NV], den[NV];
+  est_cell(M, U, vs, b, ci[0], ci[1], ci[2], ew, g, q0);
+  for (int v = 0; v < nq; v++) num[v] = den[v] = 0.0;
+  for (int d = 0; d < M.ndim; d++) {
+    int p[3] = {ci[0], ci[1], ci[2]}, m[3] = {ci[0], ci[1], ci[2]};
+    p[d] += 1;
+    m[d] -= 1;
+    double qp[NV], qm[NV];
+    est_cell(M, U, vs, b, p[0], p[1], p[2], ew, g, qp);
+    est_cell(M, U, vs, b, m[0], m[1], m[2], ew, g, qm);
+    for (int v = 0; v < nq; v++) {
+      if (ew.w[v] == 0.0) continue;
+      const double rp = qp[v], r0 = q0[v], rm = qm[v];
+      const double s2 = __dadd_rn(__dsub_rn(rp, 2.0 * r0), rm);
+      num[v] = __dadd_rn(num[v], __dmul_rn(s2, s2));
+      const double a = __dadd_rn(fabs(__dsub_rn(rp, r0)), fabs(__dsub_rn(r0, rm)));
+      const double f = __dadd_rn(__dadd_rn(fabs(rp), 2.0 * fabs(r0)), fabs(rm));
+      const double dd = __dadd_rn(a, __dmul_rn(LOEHNER_EPS, f));
+      den[v] = __dadd_rn(den[v], __dmul_rn(dd, dd));
+    }
+  }
+  double e = 0.0;
+  for (int v = 0; v < nq; v++) {
+    if (ew.w[v] == 0.0) continue;
+    const double r = den[v] > 0.0 ? num[v] / den[v] : 0.0;
+    e = __dadd_rn(e, __dmul_rn(ew.w[v], sqrt(r)));
+  }
+  return e;
+}
+
 template <class T>
 __global__ void __launch_bounds__(256) k_regrid_estimate(DevMesh M, const T* __restrict__ U,
                                                          EstWeights ew, double thr, double dthr,
@@ -71,39 +107,12 @@ __global__ void __launch_bounds__(256) k_regrid_estimate(DevMesh M, const T* __r
                                                          signed char* flags) {
   __shared__ double red[256 / 32];
   const size_t vs = (size_t)M.nblocks * M.ncell;
-  const int nq = ew.prim ? NV : 1;
   for (int b = blockIdx.x; b < M.nblocks; b += gridDim.x) {
     const double g = M.gamma[M.blk[b * 5]];
     double emax = 0.0;
     for (int c = threadIdx.x; c < M.ncell; c += blockDim.x) {
       const int ci[3] = {c % M.nx[0], (c / M.nx[0]) % M.nx[1], c / (M.nx[0] * M.nx[1])};
-      double q0[NV], num[NV], den[NV];
-      est_cell(M, U, vs, b, ci[0], ci[1], ci[2], ew, g, q0);
-      for (int v = 0; v < nq; v++) num[v] = den[v] = 0.0;
-      for (int d = 0; d < M.ndim; d++) {
-        int p[3] = {ci[0], ci[1], ci[2]}, m[3] = {ci[0], ci[1], ci[2]};
-        p[d] += 1;
-        m[d] -= 1;
-        double qp[NV], qm[NV];
-        est_cell(M, U, vs, b, p[0], p[1], p[2], ew, g, qp);
-        est_cell(M, U, vs, b, m[0], m[1], m[2], ew, g, qm);
-        for (int v = 0; v < nq; v++) {
-          if (ew.w[v] == 0.0) continue;
-          const double rp = qp[v], r0 = q0[v], rm = qm[v];
-          const double s2 = __dadd_rn(__dsub_rn(rp, 2.0 * r0), rm);
-          num[v] = __dadd_rn(num[v], __dmul_rn(s2, s2));
-          const double a = __dadd_rn(fabs(__dsub_rn(rp, r0)), fabs(__dsub_rn(r0, rm)));
-          const double f = __dadd_rn(__dadd_rn(fabs(rp), 2.0 * fabs(r0)), fabs(rm));
-          const double dd = __dadd_rn(a, __dmul_rn(LOEHNER_EPS, f));
-          den[v] = __dadd_rn(den[v], __dmul_rn(dd, dd));
-        }
-      }
-      double e = 0.0;
-      for (int v = 0; v < nq; v++) {
-        if (ew.w[v] == 0.0) continue;
-        const double r = den[v] > 0.0 ? num[v] / den[v] : 0.0;
-        e = __dadd_rn(e, __dmul_rn(ew.w[v], sqrt(r)));
-      }
+      const double e = est_double(M, U, vs, b, ci, ew, g);
       emax = e > emax ? e : emax;
     }
 #pragma unroll
@@ -136,6 +145,7 @@ __global__ void __launch_bounds__(256) k_regrid_estimate(DevMesh M, const T* __r
 // cell's estimate is +0 (also where den is 0 or the values are not finite,
 // which the quotient's guard turns into 0).
 constexpr int EST_TILED_THREADS = 512;
+constexpr double EST_TODO = -1.0;  // est of a block that the screening left (an estimate is >= 0)
 
 template <class T> __device__ __forceinline__ bool same_bits(T a, T b);
 template <> __device__ __forceinline__ bool same_bits<float>(float a, float b) {
@@ -148,7 +158,7 @@ template <> __device__ __forceinline__ bool same_bits<double>(double a, double b
 template <class T>
 __global__ void __launch_bounds__(EST_TILED_THREADS, 1)
     k_regrid_estimate_tiled(DevMesh M, const T* __restrict__ U, EstWeights ew, int nch,
-                            double thr, double dthr, int maxlev, double* est,
+                            double thr, double dthr, int maxlev, bool todo_only, double* est,
                             signed char* flags) {
   extern __shared__ double tile[];
   __shared__ double red[EST_TILED_THREADS / 32];
@@ -162,6 +172,8 @@ __global__ void __launch_bounds__(EST_TILED_THREADS, 1)
     if (ew.w[v] != 0.0) vars[nw++] = v;
   const int stride[3] = {1, P0, P0 * P1};
   for (int b = blockIdx.x; b < M.nblocks; b += gridDim.x) {
+    if (todo_only && est[b] != EST_TODO) continue;
+    __syncthreads();  // est[b] is written below
     const double g = M.gamma[M.blk[b * 5]];
     // uniform block: every stencil cell equal to the first cell, bit for bit
     T ref[NV];
@@ -249,6 +261,383 @@ __global__ void __launch_bounds__(EST_TILED_THREADS, 1)
   }
 }
 
+// FP32 states: the same estimate with a float screening.  The double arithmetic
+// (some 170 operations a cell with density and pressure, on a pipe of 2 lanes a
+// clock and SM) is only needed where the maximum may lie, so per block
+//   1. a block of equal cells is recorded as 0 (as in k_regrid_estimate_tiled);
+//      else the weighted quantities of the block and its face halo are formed in
+//      float (velocities and pressure in two parts) in shared memory;
+//   2. every cell's estimate e is evaluated in float and the block maximum taken
+//      (cells whose stencil holds equal values are exactly 0 and dropped);
+//   3. the cells with e >= max - 2 tol are evaluated in double, the arithmetic of
+//      k_regrid_estimate, and their maximum is the block's estimate.
+// The cell of the true maximum is among them when |e - exact| <= tol.  A velocity
+// or pressure is kept as a sum hi + lo within 1e-8 of itself (the pressure up to a
+// constant factor, which the quotient does not see; one below 1e-4 of the cell's
+// energies is left out, see est_float), the other variables are exact.  The
+// differences of neighbours dp, dm are then within 1.2e-7 of themselves + 2e-8 f/4
+// (f = |rp| + 2 |r0| + |rm|), and so, relative to the denominator d = |dp| + |dm| +
+// 0.01 f, are the second difference and d itself: within 2.4e-7 + 2e-6.  The
+// quotient of the norms, at most 1, is within twice that and 5e-7 for the roundings
+// of squares, sums and roots: 5e-6.  tol = 6e-6 of the sum of |weights|.  Values that
+// are not finite and denominators below 1e-30 make a cell a candidate.
+constexpr float EST_TOL = 6e-6f;
+// 512 threads of 64 registers, two CTAs an SM: the loads' latency bounds the kernel.
+// The estimate of 26 M cells on three levels: 6.8 ms all in double, 2.0 ms so (256
+// threads of 128 registers 2.2 ms); the double pipe is then busy for a quarter of it.
+constexpr int EST_SCREEN_THREADS = 512;
+// worth it from this many cells (see launch_estimate)
+constexpr size_t EST_SCREEN_CELLS = 2048;
+constexpr int EST_SLOTS = 2 * 152;
+
+// the quantities of a conserved cell as hi + lo (lo of the velocities and the
+// pressure only, the others are exact): v = m/rho with its remainder; the pressure
+// over gamma - 1 with kinetic and magnetic energies as sums of exact products and
+// the subtraction compensated, within 1e-12 of e + ke + me; NaN where that exceeds
+// 1e-8 of it, and for a velocity that underflows (a zero means an exact one)
+__device__ __forceinline__ void sq_add(float x, float& hi, float& lo) {
+  const float h = __fmul_rn(x, x);
+  lo = __fadd_rn(lo, __fmaf_rn(x, x, -h));
+  const ff2 t = two_sum(hi, h);
+  hi = t.hi;
+  lo = __fadd_rn(lo, t.lo);
+}
+__device__ __forceinline__ void est_float(const float* u, float* q, float* lo) {
+  const float nan = __int_as_float(0x7fc00000);
+  const float ir = __frcp_rn(u[0]);
+  q[0] = u[0];
+#pragma unroll
+  for (int c = 1; c < 4; c++) {
+    const float h = __fmul_rn(u[c], ir);
+    lo[c] = __fmul_rn(__fmaf_rn(-h, u[0], u[c]), ir);
+    q[c] = u[c] != 0.f && !(fabsf(h) > 1e-30f) ? nan : h;
+  }
+  float mh = 0.f, ml = 0.f, bh = 0.f, bl = 0.f;
+#pragma unroll
+  for (int c = 1; c < 4; c++) {
+    sq_add(u[c], mh, ml);
+    sq_add(u[4 + c], bh, bl);
+  }
+  // m^2 / rho as k1 + k2
+  const float k1 = __fmul_rn(mh, ir);
+  const float k2 = __fmul_rn(__fadd_rn(__fmaf_rn(-k1, u[0], mh), ml), ir);
+  const ff2 a = two_sum(u[4], -0.5f * k1);
+  const ff2 b = two_sum(a.hi, -0.5f * bh);
+  const ff2 p =
+      two_sum(b.hi, __fadd_rn(__fadd_rn(a.lo, b.lo), -0.5f * __fadd_rn(k2, bl)));
+  const float scale = fabsf(u[4]) + 0.5f * (fabsf(k1) + bh);
+  q[4] = 1e-4f * scale < fabsf(p.hi) ? p.hi : nan;
+  lo[4] = p.lo;
+#pragma unroll
+  for (int c = 5; c < NV; c++) q[c] = u[c];
+}
+
+// out of line: its general lookups would be inlined at every use
+static __device__ __noinline__ void est_cell_call(const DevMesh& M, const float* U, size_t vs,
+                                                  int b, int i, int j, int k,
+                                                  const EstWeights& ew, double g, double* q) {
+  est_cell(M, U, vs, b, i, j, k, ew, g, q);
+}
+static __device__ __noinline__ void halo_cell_call(const DevMesh& M, const float* U, size_t vs,
+                                                   int b, int i, int j, int k, float* u) {
+  block_cell_value(M, U, vs, b, i, j, k, u);
+}
+
+__global__ void __launch_bounds__(EST_SCREEN_THREADS, 2)
+    k_regrid_estimate_screen(DevMesh M, const float* __restrict__ U, EstWeights ew, float tol,
+                             double thr, double dthr, int maxlev, double* est,
+                             signed char* flags) {
+  // [quantity][padded cell], then [cell] estimates, then the list of candidates
+  extern __shared__ float ftile[];
+  __shared__ double red[EST_SCREEN_THREADS / 32];
+  __shared__ float fred[EST_SCREEN_THREADS / 32];
+  __shared__ int ncand, nbr[6];
+  const size_t vs = (size_t)M.nblocks * M.ncell;
+  const int nd = M.ndim, h1 = nd > 1 ? 1 : 0, h2 = nd > 2 ? 1 : 0;
+  const int n0 = M.nx[0], n1 = M.nx[1], n2 = M.nx[2];
+  const int P0 = n0 + 2, P1 = n1 + 2 * h1, P2 = n2 + 2 * h2, PL = P0 * P1;
+  const int np = PL * P2;
+  const int stride[3] = {1, P0, PL};
+  // the halo's cells in slots, each face's rounded up to whole warps: a warp takes one
+  // path, and the faces (a chain of lookups where the level changes) run side by side
+  const int face[3] = {n1 * n2, nd > 1 ? n0 * n2 : 0, nd > 2 ? n0 * n1 : 0};
+  const int w0 = (face[0] + 31) & ~31, w1 = (face[1] + 31) & ~31, w2 = (face[2] + 31) & ~31;
+  const int nslots = 2 * (w0 + w1 + w2);
+  auto slot = [&](int t, int& f, int& r) -> bool {
+    const int d = t < 2 * w0 ? 0 : t < 2 * (w0 + w1) ? 1 : 2;
+    const int w = d == 0 ? w0 : d == 1 ? w1 : w2;
+    r = t - (d == 0 ? 0 : d == 1 ? 2 * w0 : 2 * (w0 + w1));
+    f = 2 * d + (r >= w ? 1 : 0);
+    if (r >= w) r -= w;
+    return r < face[d];
+  };
+  const float in0 = 1.f / (float)n0, in01 = 1.f / (float)(n0 * n1);
+  unsigned mask = 0;  // the weighted variables
+#pragma unroll
+  for (int v = 0; v < NV; v++)
+    if (v < (ew.prim ? NV : 1) && ew.w[v] != 0.0) mask |= 1u << v;
+  // the conserved variables that these depend on; only they are read and compared
+  unsigned dep = mask | (mask & 0xeu ? 1u : 0u) | (mask & 0x10u ? 0xffu : 0u);
+  const int ntile = __popc(mask) + __popc(mask & 0x1eu);  // a second one for the low parts
+  float* ecell = ftile + (size_t)ntile * np;
+  int* list = (int*)(ecell + M.ncell);
+  const int most = M.ncell / 4;  // candidates taken here
+  // padded cells that hold the first cell's values, bit for bit
+  unsigned char* as_first = (unsigned char*)(list + most);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int b = blockIdx.x; b < M.nblocks; b += gridDim.x) {
+    const double g = M.gamma[M.blk[b * 5]];
+    const float* Ub = U + (size_t)b * M.ncell;
+    float ref[NV];
+#pragma unroll
+    for (int v = 0; v < NV; v++) ref[v] = dep >> v & 1 ? Ub[(size_t)v * vs] : 0.f;
+    if (threadIdx.x == 0) ncand = 0;
+    if (threadIdx.x < 6) nbr[threadIdx.x] = M.nbr[b * 6 + threadIdx.x];
+    __syncthreads();
+    // conserved values of cell r of face f's halo and its index in the padded block
+    auto halo = [&](int f, int r, float* u) -> int {
+      const int d = f >> 1, code = nbr[f];
+      const int w = d == 0 ? n1 : n0;  // r = (second) w + (first)
+      const int q = (int)(((float)r + 0.5f) * (d == 0 ? 1.f / (float)n1 : in0));
+      const int p = r - q * w;
+      const int len = d == 0 ? n0 : d == 1 ? n1 : n2, out = f & 1 ? len : -1;
+      const int i = d == 0 ? out : p, j = d == 0 ? p : d == 1 ? out : q, k = d == 2 ? out : q;
+      if (code < 0 && code != NBR_OUTFLOW) {
+        halo_cell_call(M, U, vs, b, i, j, k, u);
+      } else {
+        // the same-level neighbour's cell, or the next one inside (outflow)
+        const int step = d == 0 ? 1 : d == 1 ? n0 : n0 * n1;
+        const int move = code >= 0 ? (f & 1 ? -len : len) : (f & 1 ? -1 : 1);
+        const float* src = U + (size_t)(code >= 0 ? code : b) * M.ncell +
+                           ((k * n1 + j) * n0 + i + move * step);
+#pragma unroll
+        for (int v = 0; v < NV; v++, src += vs) u[v] = dep >> v & 1 ? *src : 0.f;
+      }
+      return ((k + h2) * P1 + (j + h1)) * P0 + i + 1;
+    };
+    auto equal = [&](const float* u) {
+      bool eq = true;
+#pragma unroll
+      for (int v = 0; v < NV; v++) eq = eq && (!(dep >> v & 1) || same_bits(u[v], ref[v]));
+      return eq;
+    };
+    const int L = M.blk[b * 5 + 1];
+    bool same = true;
+    // (the loads' latency bounds this pass: four cells at a time where they are aligned)
+    const bool quads = M.ncell % 4 == 0 && ((size_t)U & 15) == 0;
+    if (quads) {
+#pragma unroll 1
+      for (int c = 4 * threadIdx.x; c < M.ncell && same; c += 4 * EST_SCREEN_THREADS) {
+        float4 u[NV];
+#pragma unroll
+        for (int v = 0; v < NV; v++)
+          u[v] = dep >> v & 1 ? *reinterpret_cast<const float4*>(Ub + v * vs + c)
+                              : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int v = 0; v < NV; v++)
+          same = same && same_bits(u[v].x, ref[v]) && same_bits(u[v].y, ref[v]) &&
+                 same_bits(u[v].z, ref[v]) && same_bits(u[v].w, ref[v]);
+      }
+    } else {
+#pragma unroll 1
+      for (int c = threadIdx.x; c < M.ncell && same; c += EST_SCREEN_THREADS) {
+        float u[NV];
+#pragma unroll
+        for (int v = 0; v < NV; v++) u[v] = dep >> v & 1 ? Ub[v * vs + c] : 0.f;
+        same = equal(u);
+      }
+    }
+    if (__syncthreads_and(same)) {
+#pragma unroll 1
+      for (int t = threadIdx.x; t < nslots && same; t += EST_SCREEN_THREADS) {
+        int f, r;
+        float u[NV];
+        if (!slot(t, f, r)) continue;
+        halo(f, r, u);
+        same = equal(u);
+      }
+      if (__syncthreads_and(same)) {
+        if (threadIdx.x == 0) {
+          est[b] = 0.0;
+          flags[b] = (0.0 > thr && L < maxlev) ? 1 : ((0.0 < dthr && L > 0) ? -1 : 0);
+        }
+        continue;  // uniform across the CTA
+      }
+    }
+    auto put = [&](int t, const float* u) {
+      float q[NV], lo[5];
+      as_first[t] = equal(u);
+      est_float(u, q, lo);
+      float* at = ftile + t;
+#pragma unroll
+      for (int v = 0; v < NV; v++) {
+        if (!(mask >> v & 1)) continue;
+        *at = q[v];
+        at += np;
+        if (v >= 1 && v <= 4) {
+          *at = lo[v];
+          at += np;
+        }
+      }
+    };
+    float next[NV];  // the following cell, loaded while this one is converted
+    if (threadIdx.x < M.ncell)
+#pragma unroll
+      for (int v = 0; v < NV; v++) next[v] = dep >> v & 1 ? Ub[v * vs + threadIdx.x] : 0.f;
+#pragma unroll 1
+    for (int c = threadIdx.x; c < M.ncell; c += EST_SCREEN_THREADS) {
+      float u[NV];
+#pragma unroll
+      for (int v = 0; v < NV; v++) u[v] = next[v];
+      if (c + EST_SCREEN_THREADS < M.ncell)
+#pragma unroll
+        for (int v = 0; v < NV; v++)
+          next[v] = dep >> v & 1 ? Ub[v * vs + c + EST_SCREEN_THREADS] : 0.f;
+      // c = (k n1 + j) n0 + i, exact: c < 2^18, half a unit from the next quotient
+      const int k = (int)(((float)c + 0.5f) * in01), r = c - k * n0 * n1;
+      const int j = (int)(((float)r + 0.5f) * in0), i = r - j * n0;
+      put(((k + h2) * P1 + (j + h1)) * P0 + i + 1, u);
+    }
+#pragma unroll 1
+    for (int t = threadIdx.x; t < nslots; t += EST_SCREEN_THREADS) {
+      int f, r;
+      float u[NV];
+      if (!slot(t, f, r)) continue;
+      const int at = halo(f, r, u);
+      put(at, u);
+    }
+    __syncthreads();
+    // float estimates and their maximum
+    float fmx = 0.f;
+    for (int c = threadIdx.x; c < M.ncell; c += EST_SCREEN_THREADS) {
+      {
+        const int k = (int)(((float)c + 0.5f) * in01), r = c - k * n0 * n1;
+        const int j = (int)(((float)r + 0.5f) * in0), i = r - j * n0;
+        const float* q = ftile + ((k + h2) * P1 + (j + h1)) * P0 + i + 1;
+        float e = 0.f;
+        for (unsigned m = mask; m; m &= m - 1, q += np) {
+          const int v = __ffs(m) - 1;
+          const bool two = v >= 1 && v <= 4;
+          const float* l = q + np;
+          const float r0 = q[0], l0 = two ? l[0] : 0.f;
+          float s2[3], dd[3], dm = 0.f;
+          bool nan = false;
+#pragma unroll
+          for (int d = 0; d < 3; d++) {
+            if (d >= nd) continue;
+            const float rp = q[stride[d]], rm = q[-stride[d]];
+            float dp = rp - r0, dn = r0 - rm;
+            if (two) {
+              dp += l[stride[d]] - l0;
+              dn += l0 - l[-stride[d]];
+            }
+            s2[d] = dp - dn;
+            dd[d] = (fabsf(dp) + fabsf(dn)) +
+                    (float)LOEHNER_EPS * ((fabsf(rp) + 2.f * fabsf(r0)) + fabsf(rm));
+            dm = dd[d] <= dm ? dm : dd[d];
+            nan = nan || dd[d] != dd[d];
+          }
+          if (two) q += np;
+          // squares relative to the largest denominator: no underflow
+          const float id = 1.f / dm;
+          float num = 0.f, den = 0.f;
+#pragma unroll
+          for (int d = 0; d < 3; d++) {
+            if (d >= nd) continue;
+            num += (s2[d] * id) * (s2[d] * id);
+            den += (dd[d] * id) * (dd[d] * id);
+          }
+          const float r = sqrtf(num / den);
+          e += (float)ew.w[v] * (!nan && dm == 0.f ? 0.f  // every value is exactly 0
+                                            : dm >= 1e-30f && !nan ? r : __int_as_float(0x7fc00000));
+        }
+        if (!(fabsf(e) < 1e30f)) e = 3e38f;
+        if (e < 4.f * tol) {
+          // near zero: exactly zero where the whole stencil holds equal values
+          const unsigned char* f = as_first + ((k + h2) * P1 + (j + h1)) * P0 + i + 1;
+          bool eq = f[0];
+          for (int d = 0; d < nd; d++) eq = eq && f[stride[d]] && f[-stride[d]];
+          if (eq) e = -3e38f;
+        }
+        ecell[c] = e;
+        // cells that must be evaluated do not raise the bar for the others
+        if (e < 1e30f) fmx = fmaxf(fmx, e);
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) fmx = fmaxf(fmx, __shfl_xor_sync(0xffffffffu, fmx, o));
+    if (lane == 0) fred[warp] = fmx;
+    __syncthreads();
+    fmx = fred[0];
+    for (int w = 1; w < EST_SCREEN_THREADS / 32; w++) fmx = fmaxf(fmx, fred[w]);
+    const float bar = fmaxf(fmx - 2.f * tol, -1e38f);
+    for (int c = threadIdx.x; c < M.ncell; c += blockDim.x)
+      if (ecell[c] >= bar) {
+        const int n = atomicAdd(&ncand, 1);
+        if (n < most) list[n] = c;
+      }
+    __syncthreads();
+    const int nc = ncand;
+    if (nc > most) {
+      // too many (a block of noise): left to the tiled kernel, which recovers a
+      // cell's primitives once, not for each of its stencils
+      if (threadIdx.x == 0) est[b] = EST_TODO;
+      __syncthreads();
+      continue;  // uniform across the CTA
+    }
+    // the candidates in double: eight lanes each, a stencil cell a lane (the cell
+    // itself, then +d, -d); the maximum does not depend on the list's order
+    double emax = 0.0;
+    const int sc = lane & 7, d0 = (sc - 1) >> 1;
+    for (int n0c = warp * 4; n0c < nc; n0c += EST_SCREEN_THREADS / 8) {
+      const int n = n0c + (lane >> 3);
+      const int c = list[n < nc ? n : n0c];
+      int ci[3] = {c % n0, (c / n0) % n1, c / (n0 * n1)};
+      const bool used = sc <= 2 * nd;
+      if (used && sc > 0) ci[d0] += (sc & 1) ? 1 : -1;
+      double q[NV];
+      if (used) est_cell_call(M, U, vs, b, ci[0], ci[1], ci[2], ew, g, q);
+      __syncwarp();
+      double e = 0.0;
+#pragma unroll
+      for (int v = 0; v < NV; v++) {
+        if (!(mask >> v & 1)) continue;
+        const int base = lane & 24;
+        const double r0 = __shfl_sync(0xffffffffu, q[v], base);
+        double num = 0.0, den = 0.0;
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+          if (d >= nd) continue;
+          const double rp = __shfl_sync(0xffffffffu, q[v], base + 1 + 2 * d);
+          const double rm = __shfl_sync(0xffffffffu, q[v], base + 2 + 2 * d);
+          const double s2 = __dadd_rn(__dsub_rn(rp, 2.0 * r0), rm);
+          num = __dadd_rn(num, __dmul_rn(s2, s2));
+          const double a = __dadd_rn(fabs(__dsub_rn(rp, r0)), fabs(__dsub_rn(r0, rm)));
+          const double f = __dadd_rn(__dadd_rn(fabs(rp), 2.0 * fabs(r0)), fabs(rm));
+          const double dd = __dadd_rn(a, __dmul_rn(LOEHNER_EPS, f));
+          den = __dadd_rn(den, __dmul_rn(dd, dd));
+        }
+        const double r = den > 0.0 ? num / den : 0.0;
+        e = __dadd_rn(e, __dmul_rn(ew.w[v], sqrt(r)));
+      }
+      emax = e > emax ? e : emax;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double other = __shfl_xor_sync(0xffffffffu, emax, o);
+      emax = other > emax ? other : emax;
+    }
+    if (lane == 0) red[warp] = emax;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < EST_SCREEN_THREADS / 32; w++) emax = red[w] > emax ? red[w] : emax;
+      est[b] = emax;
+      flags[b] = (emax > thr && L < maxlev) ? 1 : ((emax < dthr && L > 0) ? -1 : 0);
+    }
+    __syncthreads();  // the tile and the reductions are reused by the next block
+  }
+}
+
 template <class T>
 int launch_estimate(amrvac_state* s, const T* U, const EstWeights& ew, double thr, double dthr,
                     int maxlev) {
@@ -258,8 +647,52 @@ int launch_estimate(amrvac_state* s, const T* U, const EstWeights& ew, double th
   size_t np = 1;
   for (int d = 0; d < 3; d++) np *= (size_t)(M.nx[d] + (d < M.ndim ? 2 : 0));
   const size_t cells = sizeof(double) * (size_t)M.ncell;
+  bool todo_only = false;
+  int launched = 0;
   int nw = 0;
   for (int v = 0; v < (ew.prim ? NV : 1); v++) nw += ew.w[v] != 0.0;
+  if constexpr (sizeof(T) == 4) {
+    // float screening: two CTAs an SM where the tile allows
+    int nt = nw;
+    for (int v = 1; v < 5; v++) nt += ew.prim && ew.w[v] != 0.0;
+    const size_t smem = sizeof(float) * (np * (size_t)nt + (size_t)M.ncell) +
+                        sizeof(int) * (size_t)(M.ncell / 4) + np;
+    // It saves double arithmetic, which is in proportion to the cells that one CTA
+    // works off, and costs a second launch and a longer chain of latencies where levels
+    // meet.  For density and pressure, both ways in us: 2D 16^2, 1024 blocks 150 and 110,
+    // 16384 blocks 1633 and 849; 3D 8^3, 1024 blocks 275 and 129; 16^3, 16 blocks 248
+    // and 89, 1024 blocks 1493 and 266; but 288 blocks of 8^3 on three levels 89 and
+    // 141, 43 blocks of 8^2 64 and 80, 1024 blocks of 128 cells in 1D 102 and 105.
+    // (Blocks of nothing but rounding noise are worked twice: +12 % at 16^3.)
+    // 1128 blocks of 8^3 on three levels 177 and 198, 64 blocks of 16^3 on three 289 and
+    // 111: across levels the block itself has to be large enough.
+    size_t chain = (size_t)M.ncell;
+    if (chain < EST_SCREEN_CELLS) {
+      bool one = true;
+      for (int b = 1; b < s->nblocks && one; b++) one = s->meta[5 * b + 1] == s->meta[1];
+      if (one) chain *= (size_t)((s->nblocks + EST_SLOTS - 1) / EST_SLOTS);
+    }
+    if (chain >= EST_SCREEN_CELLS && smem <= SMEM_MAX &&
+        cells + sizeof(double) * np <= SMEM_MAX) {
+      double wsum = 0.0;
+      for (int v = 0; v < (ew.prim ? NV : 1); v++) wsum += fabs(ew.w[v]);
+      int dev = 0, nsm = 0, per = 0;
+      if (cudaFuncSetAttribute(k_regrid_estimate_screen,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+              cudaSuccess ||
+          cudaGetDevice(&dev) != cudaSuccess ||
+          cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_regrid_estimate_screen,
+                                                        EST_SCREEN_THREADS, smem) != cudaSuccess)
+        return -1;
+      const int g = s->nblocks < nsm * per * 2 ? s->nblocks : nsm * per * 2;
+      k_regrid_estimate_screen<<<g, EST_SCREEN_THREADS, smem, s->stream>>>(
+          M, U, ew, EST_TOL * (float)wsum, thr, dthr, maxlev, s->d_est, s->d_eflags);
+      if (cudaPeekAtLastError() != cudaSuccess) return -1;
+      todo_only = true;
+      launched = 1;
+    }
+  }
   if (cells + sizeof(double) * np <= SMEM_MAX) {
     int nch = (int)((SMEM_MAX - cells) / (sizeof(double) * np));
     if (nch > nw) nch = nw;
@@ -274,13 +707,13 @@ int launch_estimate(amrvac_state* s, const T* U, const EstWeights& ew, double th
       return -1;
     const int g = s->nblocks < nsm * 2 ? s->nblocks : nsm * 2;
     k_regrid_estimate_tiled<T><<<g, EST_TILED_THREADS, smem, s->stream>>>(
-        M, U, ew, nch, thr, dthr, maxlev, s->d_est, s->d_eflags);
+        M, U, ew, nch, thr, dthr, maxlev, todo_only, s->d_est, s->d_eflags);
   } else {
     k_regrid_estimate<T><<<grid_for(s->nblocks), 256, 0, s->stream>>>(M, U, ew, thr, dthr,
                                                                         maxlev, s->d_est,
                                                                         s->d_eflags);
   }
-  return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
+  return cudaPeekAtLastError() == cudaSuccess ? 1 + launched : -1;
 }
 
 // children of split blocks (kind 1 in the table): one thread per cell of the
