@@ -2,7 +2,9 @@
 the estimator's screening (amrvac_regrid_estimate finds the cells of the maximum in
 float and evaluates them in double) on blocks of equal values, of rounding noise, of
 single outliers, of vanishing velocities and of a pressure far below the magnetic
-one.
+one; and
+the restriction, whose mean is formed in float where that is exact, on values of all
+magnitudes.
 """
 import numpy as np
 import pytest
@@ -94,3 +96,37 @@ def test_screened_estimate(amr, orc, nd, bnx, blocks, weights):
     S.close()
     assert np.isfinite(E).all()
     assert np.abs(E - Eo).max() <= 5e-9, np.abs(E - Eo).max()
+
+
+@pytest.mark.parametrize("nd,bnx", [(1, 4), (1, 34), (2, 4), (2, 10), (3, 4), (3, 8)])
+def test_restriction_bits(amr, orc, nd, bnx):
+    # every block merges; each parent cell has the bits of the double sum of its 2^d
+    # cells, rounded once
+    blocks = tuple(2 if d < nd else 1 for d in range(3))
+    cfg, inst, _ = _mesh(nd, bnx, 1)
+    rng = np.random.Generator(np.random.PCG64(7 * nd + bnx))
+    meta = wl.uniform_meta(blocks)
+    meta[:, 1] = 1
+    shape = (9, len(meta), bnx ** nd)
+    with np.errstate(over="ignore", under="ignore"):
+        U = rng.uniform(0.5, 1.0, shape).astype(np.float32)             # ties
+        U[1] = rng.choice([-1, 1], shape[1:]) * U[1]                    # cancellation
+        U[2] *= (10.0 ** rng.uniform(-30, 30, shape[1:])).astype(np.float32)
+        U[3] = (1 + np.arange(bnx ** nd) % 2 * -2) * (1 + 1e-7 * U[3])  # all but cancelled
+        U[4] *= np.float32(1e-41)                                       # denormal
+        U[5] *= np.float32(3.4e38)                                      # the float sum overflows
+        U[6] = rng.choice([0.0, -0.0, 1e-45, 1.0], shape[1:])
+        U[7] *= (10.0 ** rng.uniform(-9, 0, shape[1:])).astype(np.float32)
+        U[8] = 0.3
+    W = wl.Workload("merge", cfg, [inst], meta, U.astype(np.float64))
+    new = wl.uniform_meta((1, 1, 1))
+    ref = rg.transfer(cfg, [inst], meta, W.U, orc.mesh_for(W), new).astype(np.float32)
+    S = amr.State.from_workload(W, kernel="plain")
+    S.set_conserved(U)
+    D = amr.State(cfg, [inst], new, kernel="plain")
+    S.regrid_transfer(D, 0, 0)
+    got = D.get_conserved(0)
+    S.close()
+    D.close()
+    assert got.dtype == np.float32
+    assert np.array_equal(got.view(np.uint32), ref.view(np.uint32))
