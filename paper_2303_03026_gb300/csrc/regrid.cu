@@ -7,13 +7,15 @@
 //       ghost operators of the update), and the block's refine / coarsen flag.
 //       The arithmetic is double with explicit round-to-nearest operations;
 //       the tiled form stages the quantities in shared memory.
+//   k_regrid_estimate_screen: the same for FP32 states, double only where the
+//       maximum may lie.
 //   amrvac_regrid_plan (host) and amrvac_regrid_plan_device: the new block
 //       list, closed under 2:1 balance.
 //   k_regrid_copy, k_regrid_restrict, k_regrid_transfer: fill a state built
 //       on the new list from the old one: copy (kept blocks, wide elements),
 //       restriction (mean of the 2^d children cells) or prolongation (coarse
-//       value plus minmod-limited slopes times +-1/4).  Sums are formed in double in a fixed order
-//       and rounded once to the state's precision.
+//       value plus minmod-limited slopes times +-1/4).  Sums are formed in double in a
+//       fixed order (or exactly) and rounded once to the state's precision.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -269,21 +271,25 @@ __global__ void __launch_bounds__(EST_TILED_THREADS, 1)
 //      float (velocities and pressure in two parts) in shared memory;
 //   2. every cell's estimate e is evaluated in float and the block maximum taken
 //      (cells whose stencil holds equal values are exactly 0 and dropped);
-//   3. the cells with e >= max - 2 tol are evaluated in double, the arithmetic of
+//   3. with a bound tol of |e - exact| per cell, the cells with e + tol >= the
+//      block's max(e - tol) are evaluated in double, the arithmetic of
 //      k_regrid_estimate, and their maximum is the block's estimate.
-// The cell of the true maximum is among them when |e - exact| <= tol.  A velocity
-// or pressure is kept as a sum hi + lo within 1e-8 of itself (the pressure up to a
-// constant factor, which the quotient does not see; one below 1e-4 of the cell's
-// energies is left out, see est_float), the other variables are exact.  The
-// differences of neighbours dp, dm are then within 1.2e-7 of themselves + 2e-8 f/4
-// (f = |rp| + 2 |r0| + |rm|), and so, relative to the denominator d = |dp| + |dm| +
-// 0.01 f, are the second difference and d itself: within 2.4e-7 + 2e-6.  The
-// quotient of the norms, at most 1, is within twice that and 5e-7 for the roundings
-// of squares, sums and roots: 5e-6.  tol = 6e-6 of the sum of |weights|.  Values that
-// are not finite and denominators below 1e-30 make a cell a candidate.
-constexpr float EST_TOL = 6e-6f;
+// The cell of the true maximum is among them.  The bound, with u = 2^-24, dp and dm
+// the differences of neighbours, a = |dp| + |dm|, f = |rp| + 2 |r0| + |rm| and
+// d = a + 0.01 f: a velocity or pressure is a sum hi + lo, a velocity within 1e-13 of
+// itself and a pressure within 1e-12 s of itself, where s is the largest ratio of a
+// cell's energies to its pressure in the block (up to a constant factor, which the
+// quotient does not see; s > 1e4 makes the cell a candidate, see est_float).  So the
+// second difference is within 3.2 u a + 1e-12 s f, and with the roundings of d, the
+// squares, sums and roots (23 u e, e <= |a|/|d| in norms) a quantity's e is within
+// 27 u |a|/|d| + 2e-10 s: tol = sum of |w| (2e-6 |a|/|d| + 4e-10 s), and never above
+// 8e-6 of the sum of |w|.  The first term is what lets a block of rounding noise
+// (|a|/|d| of 1e-5) be told apart; with 6e-6 throughout each of its cells was a
+// candidate.  Values that are not finite and denominators below 1e-30 make a cell a
+// candidate.
+constexpr float EST_TOL = 8e-6f;
 // 512 threads of 64 registers, two CTAs an SM: the loads' latency bounds the kernel.
-// The estimate of 26 M cells on three levels: 6.8 ms all in double, 2.0 ms so (256
+// The estimate of 26 M cells on three levels: 6.8 ms all in double, below 2.0 ms so (256
 // threads of 128 registers 2.2 ms); the double pipe is then busy for a quarter of it.
 constexpr int EST_SCREEN_THREADS = 512;
 // worth it from this many cells (see launch_estimate)
@@ -302,7 +308,8 @@ __device__ __forceinline__ void sq_add(float x, float& hi, float& lo) {
   hi = t.hi;
   lo = __fadd_rn(lo, t.lo);
 }
-__device__ __forceinline__ void est_float(const float* u, float* q, float* lo) {
+// ratio: energies over |pressure|, 0 where that is left out
+__device__ __forceinline__ void est_float(const float* u, float* q, float* lo, float& ratio) {
   const float nan = __int_as_float(0x7fc00000);
   const float ir = __frcp_rn(u[0]);
   q[0] = u[0];
@@ -326,7 +333,9 @@ __device__ __forceinline__ void est_float(const float* u, float* q, float* lo) {
   const ff2 p =
       two_sum(b.hi, __fadd_rn(__fadd_rn(a.lo, b.lo), -0.5f * __fadd_rn(k2, bl)));
   const float scale = fabsf(u[4]) + 0.5f * (fabsf(k1) + bh);
-  q[4] = 1e-4f * scale < fabsf(p.hi) ? p.hi : nan;
+  const bool kept = 1e-4f * scale < fabsf(p.hi);
+  q[4] = kept ? p.hi : nan;
+  ratio = kept ? 1.0001f * __fdividef(scale, fabsf(p.hi)) : 0.f;
   lo[4] = p.lo;
 #pragma unroll
   for (int c = 5; c < NV; c++) q[c] = u[c];
@@ -351,7 +360,7 @@ __global__ void __launch_bounds__(EST_SCREEN_THREADS, 2)
   extern __shared__ float ftile[];
   __shared__ double red[EST_SCREEN_THREADS / 32];
   __shared__ float fred[EST_SCREEN_THREADS / 32];
-  __shared__ int ncand, nbr[6];
+  __shared__ int ncand, rmax, nbr[6];
   const size_t vs = (size_t)M.nblocks * M.ncell;
   const int nd = M.ndim, h1 = nd > 1 ? 1 : 0, h2 = nd > 2 ? 1 : 0;
   const int n0 = M.nx[0], n1 = M.nx[1], n2 = M.nx[2];
@@ -381,7 +390,7 @@ __global__ void __launch_bounds__(EST_SCREEN_THREADS, 2)
   const int ntile = __popc(mask) + __popc(mask & 0x1eu);  // a second one for the low parts
   float* ecell = ftile + (size_t)ntile * np;
   int* list = (int*)(ecell + M.ncell);
-  const int most = M.ncell / 4;  // candidates taken here
+  const int most = M.ncell / 16;  // candidates taken here, seven cells' work each
   // padded cells that hold the first cell's values, bit for bit
   unsigned char* as_first = (unsigned char*)(list + most);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -391,7 +400,7 @@ __global__ void __launch_bounds__(EST_SCREEN_THREADS, 2)
     float ref[NV];
 #pragma unroll
     for (int v = 0; v < NV; v++) ref[v] = dep >> v & 1 ? Ub[(size_t)v * vs] : 0.f;
-    if (threadIdx.x == 0) ncand = 0;
+    if (threadIdx.x == 0) ncand = rmax = 0;
     if (threadIdx.x < 6) nbr[threadIdx.x] = M.nbr[b * 6 + threadIdx.x];
     __syncthreads();
     // conserved values of cell r of face f's halo and its index in the padded block
@@ -464,10 +473,12 @@ __global__ void __launch_bounds__(EST_SCREEN_THREADS, 2)
         continue;  // uniform across the CTA
       }
     }
+    float ratio = 1.f;  // the largest of this thread's cells
     auto put = [&](int t, const float* u) {
-      float q[NV], lo[5];
+      float q[NV], lo[5], mine;
       as_first[t] = equal(u);
-      est_float(u, q, lo);
+      est_float(u, q, lo, mine);
+      if (mask & 0x10u) ratio = fmaxf(ratio, mine);
       float* at = ftile + t;
 #pragma unroll
       for (int v = 0; v < NV; v++) {
@@ -506,21 +517,24 @@ __global__ void __launch_bounds__(EST_SCREEN_THREADS, 2)
       const int at = halo(f, r, u);
       put(at, u);
     }
+    const int rbits = __reduce_max_sync(0xffffffffu, __float_as_int(ratio));
+    if (lane == 0) atomicMax(&rmax, rbits);
     __syncthreads();
-    // float estimates and their maximum
+    const float floor_tol = tol * (4e-10f / EST_TOL) * __int_as_float(rmax);
+    // float estimates, and the least that the maximum can be
     float fmx = 0.f;
     for (int c = threadIdx.x; c < M.ncell; c += EST_SCREEN_THREADS) {
       {
         const int k = (int)(((float)c + 0.5f) * in01), r = c - k * n0 * n1;
         const int j = (int)(((float)r + 0.5f) * in0), i = r - j * n0;
         const float* q = ftile + ((k + h2) * P1 + (j + h1)) * P0 + i + 1;
-        float e = 0.f;
+        float e = 0.f, rel = 0.f;
         for (unsigned m = mask; m; m &= m - 1, q += np) {
           const int v = __ffs(m) - 1;
           const bool two = v >= 1 && v <= 4;
           const float* l = q + np;
           const float r0 = q[0], l0 = two ? l[0] : 0.f;
-          float s2[3], dd[3], dm = 0.f;
+          float s2[3], dd[3], dm = 0.f, as = 0.f;
           bool nan = false;
 #pragma unroll
           for (int d = 0; d < 3; d++) {
@@ -532,7 +546,9 @@ __global__ void __launch_bounds__(EST_SCREEN_THREADS, 2)
               dn += l0 - l[-stride[d]];
             }
             s2[d] = dp - dn;
-            dd[d] = (fabsf(dp) + fabsf(dn)) +
+            const float a = fabsf(dp) + fabsf(dn);
+            as += a;
+            dd[d] = a +
                     (float)LOEHNER_EPS * ((fabsf(rp) + 2.f * fabsf(r0)) + fabsf(rm));
             dm = dd[d] <= dm ? dm : dd[d];
             nan = nan || dd[d] != dd[d];
@@ -548,10 +564,13 @@ __global__ void __launch_bounds__(EST_SCREEN_THREADS, 2)
             den += (dd[d] * id) * (dd[d] * id);
           }
           const float r = sqrtf(num / den);
+          if (as > 0.f) rel += (float)ew.w[v] * (as * id);  // not below the quotient of the norms
           e += (float)ew.w[v] * (!nan && dm == 0.f ? 0.f  // every value is exactly 0
                                             : dm >= 1e-30f && !nan ? r : __int_as_float(0x7fc00000));
         }
         if (!(fabsf(e) < 1e30f)) e = 3e38f;
+        // NaN (a quantity of zeros only) gives the larger bound
+        const float off = fminf(tol, 2e-6f * rel + floor_tol);
         if (e < 4.f * tol) {
           // near zero: exactly zero where the whole stencil holds equal values
           const unsigned char* f = as_first + ((k + h2) * P1 + (j + h1)) * P0 + i + 1;
@@ -559,9 +578,9 @@ __global__ void __launch_bounds__(EST_SCREEN_THREADS, 2)
           for (int d = 0; d < nd; d++) eq = eq && f[stride[d]] && f[-stride[d]];
           if (eq) e = -3e38f;
         }
-        ecell[c] = e;
+        ecell[c] = e < 1e30f ? e + off : e;
         // cells that must be evaluated do not raise the bar for the others
-        if (e < 1e30f) fmx = fmaxf(fmx, e);
+        if (e < 1e30f) fmx = fmaxf(fmx, e - off);
       }
     }
 #pragma unroll
@@ -570,9 +589,8 @@ __global__ void __launch_bounds__(EST_SCREEN_THREADS, 2)
     __syncthreads();
     fmx = fred[0];
     for (int w = 1; w < EST_SCREEN_THREADS / 32; w++) fmx = fmaxf(fmx, fred[w]);
-    const float bar = fmaxf(fmx - 2.f * tol, -1e38f);
     for (int c = threadIdx.x; c < M.ncell; c += blockDim.x)
-      if (ecell[c] >= bar) {
+      if (ecell[c] >= fmx) {
         const int n = atomicAdd(&ncand, 1);
         if (n < most) list[n] = c;
       }
@@ -656,14 +674,17 @@ int launch_estimate(amrvac_state* s, const T* U, const EstWeights& ew, double th
     int nt = nw;
     for (int v = 1; v < 5; v++) nt += ew.prim && ew.w[v] != 0.0;
     const size_t smem = sizeof(float) * (np * (size_t)nt + (size_t)M.ncell) +
-                        sizeof(int) * (size_t)(M.ncell / 4) + np;
+                        sizeof(int) * (size_t)(M.ncell / 16) + np;
     // It saves double arithmetic, which is in proportion to the cells that one CTA
     // works off, and costs a second launch and a longer chain of latencies where levels
     // meet.  For density and pressure, both ways in us: 2D 16^2, 1024 blocks 150 and 110,
     // 16384 blocks 1633 and 849; 3D 8^3, 1024 blocks 275 and 129; 16^3, 16 blocks 248
     // and 89, 1024 blocks 1493 and 266; but 288 blocks of 8^3 on three levels 89 and
     // 141, 43 blocks of 8^2 64 and 80, 1024 blocks of 128 cells in 1D 102 and 105.
-    // (Blocks of nothing but rounding noise are worked twice: +12 % at 16^3.)
+    // Blocks that differ by less than the bounds tell apart are worked twice: 3106 such
+    // blocks among 6448 of 16^3 (the blast after 60 steps) 11.3 and 11.8 ms.  Noise of an ulp is told apart (1024
+    // blocks of 16^3 1647 and 487) unless many cells tie (2D, 64 blocks of 64^2, 235
+    // and 355).
     // 1128 blocks of 8^3 on three levels 177 and 198, 64 blocks of 16^3 on three 289 and
     // 111: across levels the block itself has to be large enough.
     size_t chain = (size_t)M.ncell;
@@ -782,8 +803,8 @@ template <> struct Pair<float> { using type = float2; };
 template <> struct Pair<double> { using type = double2; };
 
 // The mean of a parent cell's values, rounded once, without the double pipe (2 lanes
-// a clock and SM, where the 8 conversions and 8 sums of a value took 0.94 ms for 75 M
-// child cells): the sum as hi + lo of error-free additions (Knuth's TwoSum).  With no
+// a clock and SM, where the 8 conversions and 8 sums of a value took 0.94 ms in a
+// regrid of 26 M cells; now 0.21 ms, bound by memory): the sum as hi + lo of error-free additions (Knuth's TwoSum).  With no
 // error left over, hi + lo is the exact sum, the sum in double is exact as well, and
 // the one rounding is the same.  False where an error is left (values more than some
 // 20 binary digits apart), the result is near or beyond the range's ends, or not
