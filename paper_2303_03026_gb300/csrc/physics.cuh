@@ -114,20 +114,6 @@ __device__ __forceinline__ void cons2prim(double gamma, const T* u, T* w, bool f
   w[8] = u[8];
 }
 
-// fast speed along direction d of a primitive state (global frame)
-template <class T>
-__device__ __forceinline__ T fast_speed(T gamma, const T* w, int d) {
-  int t1 = d == 2 ? 0 : d + 1, t2 = d == 0 ? 2 : d - 1;
-  T ir = rcp_T(w[0]);
-  T a2 = gamma * w[4] * ir;
-  T bn = w[5 + d], b1 = w[5 + t1], b2 = w[5 + t2];
-  T bt = b1 * b1 + b2 * b2;
-  T bt2 = bt * ir;
-  T bb = (bn * bn + bt) * ir;
-  T dd = a2 - bb;
-  return sqrt_T(T(0.5) * (a2 + bb + sqrt_T(dd * dd + T(4) * a2 * bt2)));
-}
-
 // small values (Sect. 7.4): density or pressure below its floor, or not
 // positive at all (the floors default to 0)
 template <class T> __device__ __forceinline__ bool is_small_prim(T rho, T p, T rho_floor,
