@@ -813,28 +813,38 @@ template <> struct Pair<double> { using type = double2; };
 
 // The mean of a parent cell's values, rounded once, without the double pipe (2 lanes
 // a clock and SM, where the 8 conversions and 8 sums of a value took 0.94 ms in a
-// regrid of 26 M cells; now 0.21 ms, bound by memory): the sum as hi + lo of error-free additions (Knuth's TwoSum).  With no
-// error left over, hi + lo is the exact sum, the sum in double is exact as well, and
-// the one rounding is the same.  False where an error is left (values more than some
-// 20 binary digits apart), the result is near or beyond the range's ends, or not
+// regrid of 26 M cells; now 0.21 ms, bound by memory): the sum as hi + lo of error-free
+// additions (Knuth's TwoSum).  With no error left over, hi + lo is the exact sum.  The
+// double sums are exact too where the largest and the smallest nonzero value are at most
+// 26 binary digits apart: all sums of up to 8 are then multiples of the smallest one's
+// last digit below 2^53 of it.  The one rounding is then the same.  False where an error
+// is left, the values are further apart (in double the smaller ones may be rounded away
+// before the larger ones cancel), the result is near or beyond the range's ends, or not
 // finite: the double sum decides.
 __device__ __forceinline__ bool mean_exact(const float2* pr, int nrow, float inv, float& mean) {
   float hi = 0.f, lo = 0.f, left = 0.f;
+  unsigned big = 0u, small = 0xffffffffu;  // bits of the magnitudes; zeros left out of small
 #pragma unroll
   for (int r = 0; r < 4; r++) {
     if (r >= nrow) continue;
 #pragma unroll
     for (int x = 0; x < 2; x++) {
-      const ff2 a = two_sum(hi, x ? pr[r].y : pr[r].x);
+      const float val = x ? pr[r].y : pr[r].x;
+      const ff2 a = two_sum(hi, val);
       const ff2 b = two_sum(lo, a.lo);
       hi = a.hi;
       lo = b.hi;
       left = __fadd_rn(left, fabsf(b.lo));
+      const unsigned bits = (unsigned)__float_as_int(val) & 0x7fffffffu;
+      big = max(big, bits);
+      small = min(small, bits - 1u);
     }
   }
   const float s = __fadd_rn(hi, lo);
   mean = __fmul_rn(s, inv);
-  return left == 0.f && (s == 0.f || (fabsf(s) > 1e-30f && fabsf(s) < 1e38f));
+  // (zeros only: big is 0 and small + 1 wraps to 0)
+  const bool close = (big >> 23) - ((small + 1u) >> 23) <= 26u;
+  return left == 0.f && close && (s == 0.f || (fabsf(s) > 1e-30f && fabsf(s) < 1e38f));
 }
 __device__ __forceinline__ bool mean_exact(const double2*, int, double, double&) { return false; }
 
