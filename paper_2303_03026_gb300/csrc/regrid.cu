@@ -306,12 +306,15 @@ constexpr int EST_SLOTS = 2 * 152;
 
 // the quantities of a conserved cell as hi + lo (lo of the velocities and the
 // pressure only, the others are exact): v = m/rho with its remainder; the pressure
-// over gamma - 1 with kinetic and magnetic energies as sums of exact products and
+// over gamma - 1 with kinetic (m v) and magnetic energies as sums of exact products and
 // the subtraction compensated, within 1e-12 of e + ke + me; NaN where that exceeds
-// 1e-8 of it, and for a velocity that underflows (a zero means an exact one)
-__device__ __forceinline__ void sq_add(float x, float& hi, float& lo) {
-  const float h = __fmul_rn(x, x);
-  lo = __fadd_rn(lo, __fmaf_rn(x, x, -h));
+// 1e-8 of it, and for a velocity that underflows (a zero means an exact one).
+// Remainders are exact to the smallest float, 1.4e-45: energies below 1e-22 and
+// momenta below 1e-32 in a velocity are NaN too.  (Products of the size of the
+// energies, not m^2: that underflows where densities are small in the caller's units.)
+__device__ __forceinline__ void product_add(float a, float b, float& hi, float& lo) {
+  const float h = __fmul_rn(a, b);
+  lo = __fadd_rn(lo, __fmaf_rn(a, b, -h));
   const ff2 t = two_sum(hi, h);
   hi = t.hi;
   lo = __fadd_rn(lo, t.lo);
@@ -320,28 +323,23 @@ __device__ __forceinline__ void sq_add(float x, float& hi, float& lo) {
 __device__ __forceinline__ void est_float(const float* u, float* q, float* lo, float& ratio) {
   const float nan = __int_as_float(0x7fc00000);
   const float ir = __frcp_rn(u[0]);
+  float kh = 0.f, kl = 0.f, bh = 0.f, bl = 0.f;
   q[0] = u[0];
 #pragma unroll
   for (int c = 1; c < 4; c++) {
     const float h = __fmul_rn(u[c], ir);
     lo[c] = __fmul_rn(__fmaf_rn(-h, u[0], u[c]), ir);
-    q[c] = u[c] != 0.f && !(fabsf(h) > 1e-30f) ? nan : h;
+    q[c] = u[c] != 0.f && !(fabsf(h) > 1e-30f && fabsf(u[c]) > 1e-32f) ? nan : h;
+    product_add(u[c], h, kh, kl);
+    kl = __fmaf_rn(u[c], lo[c], kl);
+    product_add(u[4 + c], u[4 + c], bh, bl);
   }
-  float mh = 0.f, ml = 0.f, bh = 0.f, bl = 0.f;
-#pragma unroll
-  for (int c = 1; c < 4; c++) {
-    sq_add(u[c], mh, ml);
-    sq_add(u[4 + c], bh, bl);
-  }
-  // m^2 / rho as k1 + k2
-  const float k1 = __fmul_rn(mh, ir);
-  const float k2 = __fmul_rn(__fadd_rn(__fmaf_rn(-k1, u[0], mh), ml), ir);
-  const ff2 a = two_sum(u[4], -0.5f * k1);
+  const ff2 a = two_sum(u[4], -0.5f * kh);
   const ff2 b = two_sum(a.hi, -0.5f * bh);
   const ff2 p =
-      two_sum(b.hi, __fadd_rn(__fadd_rn(a.lo, b.lo), -0.5f * __fadd_rn(k2, bl)));
-  const float scale = fabsf(u[4]) + 0.5f * (fabsf(k1) + bh);
-  const bool kept = 1e-4f * scale < fabsf(p.hi);
+      two_sum(b.hi, __fadd_rn(__fadd_rn(a.lo, b.lo), -0.5f * __fadd_rn(kl, bl)));
+  const float scale = fabsf(u[4]) + 0.5f * (fabsf(kh) + bh);
+  const bool kept = scale > 1e-22f && 1e-4f * scale < fabsf(p.hi);
   q[4] = kept ? p.hi : nan;
   ratio = kept ? 1.0001f * __fdividef(scale, fabsf(p.hi)) : 0.f;
   lo[4] = p.lo;
