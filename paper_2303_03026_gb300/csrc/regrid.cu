@@ -41,6 +41,7 @@ int grid_for(int nblocks) { return nblocks < 152 * 8 ? nblocks : 152 * 8; }
 struct EstWeights {
   double w[NV];  // weight of each primitive variable (rho, v, p, B, psi)
   int prim;      // 1 when a variable other than rho is weighted
+  float wf[NV];  // the weights over the largest one, for the float screening
 };
 
 // the weighted quantities of block-local cell (i, j, k) with at most one
@@ -290,8 +291,8 @@ __global__ void __launch_bounds__(EST_TILED_THREADS, 1)
 // quotient does not see; s > 1e4 makes the cell a candidate, see est_float).  So the
 // second difference is within 3.2 u a + 1e-12 s f, and with the roundings of d, the
 // squares, sums and roots (23 u e, e <= |a|/|d| in norms) a quantity's e is within
-// 27 u |a|/|d| + 2e-10 s: tol = sum of |w| (2e-6 |a|/|d| + 4e-10 s), and never above
-// 8e-6 of the sum of |w|.  The first term is what lets a block of rounding noise
+// 27 u |a|/|d| + 2e-10 s: tol = sum of w (2e-6 |a|/|d| + 4e-10 s), and never above
+// 8e-6 of the sum of w (the weights over the largest one, whatever its magnitude).  The first term is what lets a block of rounding noise
 // (|a|/|d| of 1e-5) be told apart; with 6e-6 throughout each of its cells was a
 // candidate.  Values that are not finite and denominators below 1e-30 make a cell a
 // candidate.
@@ -570,9 +571,9 @@ __global__ void __launch_bounds__(EST_SCREEN_THREADS, 2)
             den += (dd[d] * id) * (dd[d] * id);
           }
           const float r = sqrtf(num / den);
-          if (as > 0.f) rel += (float)ew.w[v] * (as * id);  // not below the quotient of the norms
-          e += (float)ew.w[v] * (!nan && dm == 0.f ? 0.f  // every value is exactly 0
-                                            : dm >= 1e-30f && !nan ? r : __int_as_float(0x7fc00000));
+          if (as > 0.f) rel += ew.wf[v] * (as * id);  // not below the quotient of the norms
+          e += ew.wf[v] * (!nan && dm == 0.f ? 0.f  // every value is exactly 0
+                                             : dm >= 1e-30f && !nan ? r : __int_as_float(0x7fc00000));
         }
         if (!(fabsf(e) < 1e30f)) e = 3e38f;
         // NaN (a quantity of zeros only) gives the larger bound
@@ -702,8 +703,10 @@ int launch_estimate(amrvac_state* s, const T* U, const EstWeights& ew, double th
     }
     if (chain >= EST_SCREEN_CELLS && smem <= SMEM_MAX &&
         cells + sizeof(double) * np <= SMEM_MAX) {
-      double wsum = 0.0;
-      for (int v = 0; v < (ew.prim ? NV : 1); v++) wsum += fabs(ew.w[v]);
+      EstWeights sw = ew;
+      double wmax = 0.0, wsum = 0.0;
+      for (int v = 0; v < (ew.prim ? NV : 1); v++) wmax = fmax(wmax, ew.w[v]);
+      for (int v = 0; v < (ew.prim ? NV : 1); v++) wsum += sw.wf[v] = (float)(ew.w[v] / wmax);
       int dev = 0, nsm = 0, per = 0;
       if (cudaFuncSetAttribute(k_regrid_estimate_screen,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
@@ -715,7 +718,7 @@ int launch_estimate(amrvac_state* s, const T* U, const EstWeights& ew, double th
         return -1;
       const int g = s->nblocks < nsm * per * 2 ? s->nblocks : nsm * per * 2;
       k_regrid_estimate_screen<<<g, EST_SCREEN_THREADS, smem, s->stream>>>(
-          M, U, ew, EST_TOL * (float)wsum, thr, dthr, maxlev, s->d_est, s->d_eflags);
+          M, U, sw, EST_TOL * (float)wsum, thr, dthr, maxlev, s->d_est, s->d_eflags);
       if (cudaPeekAtLastError() != cudaSuccess) return -1;
       todo_only = true;
       launched = 1;

@@ -10,8 +10,8 @@ it, four terms and weights that add up to 3.6: below 2e-12; 1e-11.  A cell misse
 the screening would cost up to 1e-5.
 
 Units: scaling a state by powers of two (densities, momenta and energies by s, fields
-by sqrt(s)) scales every operation of the double estimate exactly, so the estimates are
-the same bits.
+by sqrt(s)) or all weights by one scales every operation of the double estimate
+exactly, so the estimates are the same bits.
 """
 import numpy as np
 import pytest
@@ -126,3 +126,17 @@ def test_other_units(amr, nd, bnx, weights, k):
     U[:5] *= 4.0 ** k
     U[5:] *= 2.0 ** k
     assert np.array_equal(_estimates(amr, cfg, inst, meta, U, WEIGHTS[weights]), E)
+
+
+@pytest.mark.parametrize("nd,bnx", [(1, 2048), (2, 64), (3, 16)])
+@pytest.mark.parametrize("weights", ["rho_p", "all"])
+@pytest.mark.parametrize("k", [-1020, -148, -140, -128, 100, 130, 1000])
+def test_other_weights(amr, nd, bnx, weights, k):
+    cfg, inst, meta = _uniform(nd, bnx, 24)
+    U = _contents(meta, bnx ** nd, 13, KINDS, 2.0 ** -21)
+    w = np.array(WEIGHTS[weights])
+    E = _estimates(amr, cfg, inst, meta, U, w)
+    got = _estimates(amr, cfg, inst, meta, U, w * 2.0 ** k)
+    # at 2^-1020 products of weights and sums are subnormal: 9 of each, and the scaled
+    # E, are rounded by half of 2^-1074
+    assert np.abs(got - E * 2.0 ** k).max() <= (9.5 * 2.0 ** -1074 if k == -1020 else 0.0)
