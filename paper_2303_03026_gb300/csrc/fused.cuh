@@ -227,15 +227,28 @@ template <class T, int G> struct HelperLine {
 // The shared-slope x and y fluxes of a plane: prim[v][y][x] its primitives with
 // G ghost layers, fx and fy the face arrays (which first carry the states
 // handed over).  keep(face, idx, f) sees every block-boundary flux.  Contains
-// one barrier; the caller's next barrier makes the fluxes visible.
+// one barrier, between the slopes and the fluxes, that owners and helpers reach
+// together; the caller's next barrier makes the fluxes visible.
 template <class T, int LIM, int FLUX, int G, int PW, class Keep>
 __device__ __forceinline__ void shared_slope_xy(const T (*prim)[PW][PW], T (*fx)[FB][FXW],
                                                 T (*fy)[FB + 1][FXW], int x, int y, bool owner,
                                                 int runtime_lim, int glm, const FaceConst<T>& fc,
                                                 Keep keep) {
   const int lim = LIM >= 0 ? LIM : runtime_lim;
+  const int r = threadIdx.x & 15;
+  auto line = [&]() {
+    HelperLine<T, G> h;
+    h.ydir = (threadIdx.x & 16) != 0;
+    h.row = h.ydir ? &prim[0][0][r + G] : &prim[0][r + G][0];
+    h.fr = h.ydir ? &fy[0][0][r] : &fx[0][r][0];
+    h.st = h.ydir ? PW : 1;
+    h.cv = PW * PW;
+    h.fs = h.ydir ? FXW : 1;
+    h.fv = h.ydir ? (FB + 1) * FXW : FB * FXW;
+    return h;
+  };
+  T lox[NV], loy[NV];  // of the own cell; a helper's are of its line, in lox
   if (owner) {
-    T lox[NV], loy[NV];
 #pragma unroll
     for (int v = 0; v < NV; v++) {
       const T c = prim[v][y + G][x + G];
@@ -245,7 +258,11 @@ __device__ __forceinline__ void shared_slope_xy(const T (*prim)[PW][PW], T (*fx)
       cell_faces(lim, prim[v][y + G - 1][x + G], c, prim[v][y + G + 1][x + G], loy[v], hi);
       fy[v][y + 1][x] = hi;
     }
-    __syncthreads();
+  } else {
+    line().slopes(lim, lox);
+  }
+  __syncthreads();
+  if (owner) {
     T wl[NV], f[NV];
 #pragma unroll
     for (int v = 0; v < NV; v++) wl[v] = fx[v][y][x];
@@ -264,19 +281,9 @@ __device__ __forceinline__ void shared_slope_xy(const T (*prim)[PW][PW], T (*fx)
     for (int v = 0; v < NV; v++) fy[v][y][x] = f[v];
     if (y == 0) keep(2, x, f);
   } else {
-    const int r = threadIdx.x & 15;
-    HelperLine<T, G> h;
-    h.ydir = (threadIdx.x & 16) != 0;
-    h.row = h.ydir ? &prim[0][0][r + G] : &prim[0][r + G][0];
-    h.fr = h.ydir ? &fy[0][0][r] : &fx[0][r][0];
-    h.st = h.ydir ? PW : 1;
-    h.cv = PW * PW;
-    h.fs = h.ydir ? FXW : 1;
-    h.fv = h.ydir ? (FB + 1) * FXW : FB * FXW;
-    T lo[NV], out[NV];
-    h.slopes(lim, lo);
-    __syncthreads();
-    h.template flux<FLUX>(lo, glm, fc, out);
+    const HelperLine<T, G> h = line();
+    T out[NV];
+    h.template flux<FLUX>(lox, glm, fc, out);
     keep(h.ydir ? 3 : 1, r, out);
   }
 }
