@@ -67,6 +67,18 @@ __device__ __forceinline__ void est_cell(const DevMesh& M, const T* U, size_t vs
   }
 }
 
+// a direction's terms of the quotient: squares of the second difference and of the
+// denominator
+__device__ __forceinline__ void est_terms(double rp, double r0, double rm, double& num,
+                                          double& den) {
+  const double s2 = __dadd_rn(__dsub_rn(rp, 2.0 * r0), rm);
+  num = __dadd_rn(num, __dmul_rn(s2, s2));
+  const double a = __dadd_rn(fabs(__dsub_rn(rp, r0)), fabs(__dsub_rn(r0, rm)));
+  const double f = __dadd_rn(__dadd_rn(fabs(rp), 2.0 * fabs(r0)), fabs(rm));
+  const double dd = __dadd_rn(a, __dmul_rn(LOEHNER_EPS, f));
+  den = __dadd_rn(den, __dmul_rn(dd, dd));
+}
+
 // estimate of cell ci of block b in double: sum over the weighted quantities of
 // w sqrt(num/den)
 template <class T>
@@ -85,13 +97,7 @@ __device__ double est_double(const DevMesh& M, const T* U, size_t vs, int b, con
     est_cell(M, U, vs, b, m[0], m[1], m[2], ew, g, qm);
     for (int v = 0; v < nq; v++) {
       if (ew.w[v] == 0.0) continue;
-      const double rp = qp[v], r0 = q0[v], rm = qm[v];
-      const double s2 = __dadd_rn(__dsub_rn(rp, 2.0 * r0), rm);
-      num[v] = __dadd_rn(num[v], __dmul_rn(s2, s2));
-      const double a = __dadd_rn(fabs(__dsub_rn(rp, r0)), fabs(__dsub_rn(r0, rm)));
-      const double f = __dadd_rn(__dadd_rn(fabs(rp), 2.0 * fabs(r0)), fabs(rm));
-      const double dd = __dadd_rn(a, __dmul_rn(LOEHNER_EPS, f));
-      den[v] = __dadd_rn(den[v], __dmul_rn(dd, dd));
+      est_terms(qp[v], q0[v], qm[v], num[v], den[v]);
     }
   }
   double e = 0.0;
@@ -301,6 +307,8 @@ constexpr float EST_TOL = 8e-6f;
 // The estimate of 26 M cells on three levels: 6.8 ms all in double, below 2.0 ms so (256
 // threads of 128 registers 2.2 ms); the double pipe is then busy for a quarter of it.
 constexpr int EST_SCREEN_THREADS = 512;
+// candidates that eight lanes share, two rounds of them
+constexpr int EST_SCREEN_FEW = EST_SCREEN_THREADS / 4;
 // worth it from this many cells (see launch_estimate)
 constexpr size_t EST_SCREEN_CELLS = 2048;
 constexpr int EST_SLOTS = 2 * 152;
@@ -354,6 +362,18 @@ static __device__ __noinline__ void est_cell_call(const DevMesh& M, const float*
                                                   const EstWeights& ew, double g, double* q) {
   est_cell(M, U, vs, b, i, j, k, ew, g, q);
 }
+// the same of one variable that is not a conserved one (v = 1 .. 4)
+static __device__ __noinline__ double est_value_call(const DevMesh& M, const float* U, size_t vs,
+                                                     int b, int i, int j, int k, int v,
+                                                     double g) {
+  float u[NV];
+  double ud[NV], w[NV];
+  block_cell_value(M, U, vs, b, i, j, k, u);
+#pragma unroll
+  for (int c = 0; c < NV; c++) ud[c] = (double)u[c];
+  cons2prim(g, ud, w);
+  return v == 1 ? w[1] : v == 2 ? w[2] : v == 3 ? w[3] : w[4];
+}
 static __device__ __noinline__ void halo_cell_call(const DevMesh& M, const float* U, size_t vs,
                                                    int b, int i, int j, int k, float* u) {
   block_cell_value(M, U, vs, b, i, j, k, u);
@@ -363,7 +383,7 @@ __global__ void __launch_bounds__(EST_SCREEN_THREADS, 2)
     k_regrid_estimate_screen(DevMesh M, const float* __restrict__ U, EstWeights ew, float tol,
                              double thr, double dthr, int maxlev, double* est,
                              signed char* flags) {
-  // [quantity][padded cell], then [cell] estimates, then the list of candidates
+  // [quantity][padded cell], [cell] estimates, a byte a padded cell
   extern __shared__ float ftile[];
   __shared__ double red[EST_SCREEN_THREADS / 32];
   __shared__ float fred[EST_SCREEN_THREADS / 32];
@@ -396,10 +416,14 @@ __global__ void __launch_bounds__(EST_SCREEN_THREADS, 2)
   unsigned dep = mask | (mask & 0xeu ? 1u : 0u) | (mask & 0x10u ? 0xffu : 0u);
   const int ntile = __popc(mask) + __popc(mask & 0x1eu);  // a second one for the low parts
   float* ecell = ftile + (size_t)ntile * np;
-  int* list = (int*)(ecell + M.ncell);
-  const int most = M.ncell / 16;  // candidates taken here, seven cells' work each
-  // padded cells that hold the first cell's values, bit for bit
-  unsigned char* as_first = (unsigned char*)(list + most);
+  // padded cells that hold the first cell's values, bit for bit; once the estimates are
+  // there, the list of candidates
+  unsigned char* as_first = (unsigned char*)(ecell + M.ncell);
+  unsigned short* list = (unsigned short*)as_first;
+  // candidates taken here: a velocity or pressure costs a candidate the primitives of
+  // 2 nd + 1 cells, where the tiled kernel recovers a cell's once
+  const int ntwo = ntile - __popc(mask);
+  const int most = M.ncell / (ntwo > 1 ? 2 * ntwo : 2);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int b = blockIdx.x; b < M.nblocks; b += gridDim.x) {
     const double g = M.gamma[M.blk[b * 5]];
@@ -599,7 +623,7 @@ __global__ void __launch_bounds__(EST_SCREEN_THREADS, 2)
     for (int c = threadIdx.x; c < M.ncell; c += blockDim.x)
       if (ecell[c] >= fmx) {
         const int n = atomicAdd(&ncand, 1);
-        if (n < most) list[n] = c;
+        if (n < most) list[n] = (unsigned short)c;
       }
     __syncthreads();
     const int nc = ncand;
@@ -610,11 +634,40 @@ __global__ void __launch_bounds__(EST_SCREEN_THREADS, 2)
       __syncthreads();
       continue;  // uniform across the CTA
     }
-    // the candidates in double: eight lanes each, a stencil cell a lane (the cell
-    // itself, then +d, -d); the maximum does not depend on the list's order
+    // the candidates in double; the maximum does not depend on the list's order.  Few
+    // of them: eight lanes each, a stencil cell a lane (the cell itself, then +d, -d).
+    // Many (cells that tie): a lane each, an eighth of the quotients and roots.
     double emax = 0.0;
     const int sc = lane & 7, d0 = (sc - 1) >> 1;
-    for (int n0c = warp * 4; n0c < nc; n0c += EST_SCREEN_THREADS / 8) {
+    if (nc > EST_SCREEN_FEW) {
+#pragma unroll 1
+      for (int n = threadIdx.x; n < nc; n += EST_SCREEN_THREADS) {
+        const int c = list[n], i = c % n0, j = (c / n0) % n1, k = c / (n0 * n1);
+        const float* q = ftile + ((k + h2) * P1 + (j + h1)) * P0 + i + 1;
+        double e = 0.0;
+#pragma unroll 1
+        for (unsigned m = mask; m; m &= m - 1, q += np) {
+          const int v = __ffs(m) - 1;
+          const bool two = v >= 1 && v <= 4;
+          const double r0 = two ? est_value_call(M, U, vs, b, i, j, k, v, g) : (double)q[0];
+          double num = 0.0, den = 0.0;
+#pragma unroll 1
+          for (int d = 0; d < nd; d++) {
+            const int x = d == 0, y = d == 1, z = d == 2, st = x ? 1 : y ? P0 : PL;
+            const double rp =
+                two ? est_value_call(M, U, vs, b, i + x, j + y, k + z, v, g) : (double)q[st];
+            const double rm =
+                two ? est_value_call(M, U, vs, b, i - x, j - y, k - z, v, g) : (double)q[-st];
+            est_terms(rp, r0, rm, num, den);
+          }
+          const double r = den > 0.0 ? num / den : 0.0;
+          e = __dadd_rn(e, __dmul_rn(ew.w[v], sqrt(r)));
+          if (two) q += np;
+        }
+        emax = e > emax ? e : emax;
+      }
+    }
+    for (int n0c = warp * 4; nc <= EST_SCREEN_FEW && n0c < nc; n0c += EST_SCREEN_THREADS / 8) {
       const int n = n0c + (lane >> 3);
       const int c = list[n < nc ? n : n0c];
       int ci[3] = {c % n0, (c / n0) % n1, c / (n0 * n1)};
@@ -635,12 +688,7 @@ __global__ void __launch_bounds__(EST_SCREEN_THREADS, 2)
           if (d >= nd) continue;
           const double rp = __shfl_sync(0xffffffffu, q[v], base + 1 + 2 * d);
           const double rm = __shfl_sync(0xffffffffu, q[v], base + 2 + 2 * d);
-          const double s2 = __dadd_rn(__dsub_rn(rp, 2.0 * r0), rm);
-          num = __dadd_rn(num, __dmul_rn(s2, s2));
-          const double a = __dadd_rn(fabs(__dsub_rn(rp, r0)), fabs(__dsub_rn(r0, rm)));
-          const double f = __dadd_rn(__dadd_rn(fabs(rp), 2.0 * fabs(r0)), fabs(rm));
-          const double dd = __dadd_rn(a, __dmul_rn(LOEHNER_EPS, f));
-          den = __dadd_rn(den, __dmul_rn(dd, dd));
+          est_terms(rp, r0, rm, num, den);
         }
         const double r = den > 0.0 ? num / den : 0.0;
         e = __dadd_rn(e, __dmul_rn(ew.w[v], sqrt(r)));
@@ -680,19 +728,20 @@ int launch_estimate(amrvac_state* s, const T* U, const EstWeights& ew, double th
     // float screening: two CTAs an SM where the tile allows
     int nt = nw;
     for (int v = 1; v < 5; v++) nt += ew.prim && ew.w[v] != 0.0;
-    const size_t smem = sizeof(float) * (np * (size_t)nt + (size_t)M.ncell) +
-                        sizeof(int) * (size_t)(M.ncell / 16) + np;
+    const size_t smem = sizeof(float) * (np * (size_t)nt + (size_t)M.ncell) + np;
     // It saves double arithmetic, which is in proportion to the cells that one CTA
     // works off, and costs a second launch and a longer chain of latencies where levels
     // meet.  For density and pressure, both ways in us: 2D 16^2, 1024 blocks 150 and 110,
     // 16384 blocks 1633 and 849; 3D 8^3, 1024 blocks 275 and 129; 16^3, 16 blocks 248
     // and 89, 1024 blocks 1493 and 266; but 288 blocks of 8^3 on three levels 89 and
     // 141, 43 blocks of 8^2 64 and 80, 1024 blocks of 128 cells in 1D 102 and 105.
-    // Blocks that differ by less than the bounds tell apart are worked twice: 3106 such
-    // blocks among 6448 of 16^3 (the blast after 60 steps) 11.3 and 11.8 ms; with the
-    // tiled kernel's flat quantities left out 7.2.  Noise of an ulp is told apart (1024
-    // blocks of 16^3 1647 and 487) unless many cells tie (2D, 64 blocks of 64^2, 235
-    // and 355).
+    // Blocks with more candidates than the screening takes are worked twice: where half
+    // the cells and more tie (an exact checkerboard: 64 blocks of 64^2 210 and 251, 1024
+    // of 16^3 1564 and 1825) or the values differ by less than the bounds tell apart
+    // (the blast after 60 steps, 3106 such blocks among 6448 of 16^3: 11.2 and, with the
+    // tiled kernel's flat quantities left out, 7.1 ms).  Noise of an ulp is told apart:
+    // 1024 blocks of 16^3 1649 and 517; 2D, 64 blocks of 64^2, where one cell in 16 ties
+    // for the maximum, 235 and 113 (328 with eight lanes a candidate for all of them).
     // 1128 blocks of 8^3 on three levels 177 and 198, 64 blocks of 16^3 on three 289 and
     // 111: across levels the block itself has to be large enough.
     size_t chain = (size_t)M.ncell;

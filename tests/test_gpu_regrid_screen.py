@@ -78,6 +78,16 @@ def _mesh(name, bc):
     return cfg, wl.Instance(base_blocks=base), leaves
 
 
+KINDS = np.repeat([1, 2, 3], 8)  # runs of a kind, so that a block's maximum may lie inside
+
+
+def _uniform(nd, bnx, blocks):
+    base = (blocks, 1, 1)
+    cfg = wl.Config(ndim=nd, block_nx=tuple(bnx if d < nd else 1 for d in range(3)),
+                    precision="fp32")
+    return cfg, wl.Instance(base_blocks=base), wl.uniform_meta(base)
+
+
 @pytest.mark.parametrize("name", ["1d", "2d46", "2d64", "3d"])
 @pytest.mark.parametrize("bc", [(P, P, P), (O, O, O), (O, Y, O), (Y, O, Y)],
                          ids=["periodic", "outflow", "oyo", "yoy"])
@@ -98,22 +108,33 @@ def test_levels_and_boundaries(amr, orc, name, bc):
     S.close()
 
 
+@pytest.mark.parametrize("nd,bnx", [(1, 2048), (2, 46), (2, 64), (3, 14), (3, 16)])
+@pytest.mark.parametrize("period", [2, 4])
+def test_ties(amr, orc, nd, bnx, period):
+    # random contents that repeat with the period: 60 to 1024 cells tie for the maximum
+    # (46 and 14 are no multiples of 4: the seams add others), so that few candidates,
+    # many and more than the screening takes occur
+    cfg, inst, meta = _uniform(nd, bnx, 20)
+    at = np.indices(tuple(bnx if d < nd else 1 for d in (2, 1, 0))).reshape(3, -1) % period
+    pat = _contents(meta, period ** 3, 14, np.full(len(meta), 3))
+    pat[:, 1::2] = pat[:, :1]  # every other block the first one's
+    U = pat[:, :, (at[0] * period + at[1]) * period + at[2]]
+    W = wl.Workload("ties", cfg, [inst], meta, U)
+    S = amr.State.from_workload(W, kernel="plain")
+    S.set_conserved(U.astype(np.float32))
+    for weights in WEIGHTS.values():
+        Eo = rg.estimator(orc.mesh_for(W), U, cfg, weights=weights)
+        E, _ = S.regrid_estimate(0.1, 0.5, max_level=3, weights=weights)
+        assert np.abs(E - Eo).max() <= 1e-11, np.abs(E - Eo).max()
+    S.close()
+
+
 def _estimates(amr, cfg, inst, meta, U, weights):
     S = amr.State(cfg, [inst], meta, kernel="plain")
     S.set_conserved(U.astype(np.float32))
     E, _ = S.regrid_estimate(0.1, 0.5, max_level=3, weights=weights)
     S.close()
     return E
-
-
-KINDS = np.repeat([1, 2, 3], 8)  # runs of a kind, so that a block's maximum may lie inside
-
-
-def _uniform(nd, bnx, blocks):
-    base = (blocks, 1, 1)
-    cfg = wl.Config(ndim=nd, block_nx=tuple(bnx if d < nd else 1 for d in range(3)),
-                    precision="fp32")
-    return cfg, wl.Instance(base_blocks=base), wl.uniform_meta(base)
 
 
 @pytest.mark.parametrize("nd,bnx", [(1, 2048), (2, 64), (3, 16)])
