@@ -181,8 +181,10 @@ __global__ void __launch_bounds__(EST_TILED_THREADS, 1)
     if (ew.w[v] != 0.0) vars[nw++] = v;
   const int stride[3] = {1, P0, P0 * P1};
   for (int b = blockIdx.x; b < M.nblocks; b += gridDim.x) {
-    if (todo_only && est[b] != EST_TODO) continue;
-    __syncthreads();  // est[b] is written below
+    if (todo_only) {
+      if (est[b] != EST_TODO) continue;
+      __syncthreads();  // est[b] is written below
+    }
     const double g = M.gamma[M.blk[b * 5]];
     // uniform block: every stencil cell equal to the first cell, bit for bit
     T ref[NV];
@@ -235,24 +237,19 @@ __global__ void __launch_bounds__(EST_TILED_THREADS, 1)
         for (int cc = 0; cc < cn; cc++) {
           const double* q = tile + (size_t)cc * np;
           const double r0 = q[t0];
+          // equal values add nothing (their second differences are 0, or the quotient's
+          // guard makes it 0), and the work is left out.  Told from the bits on the integer
+          // pipe: a test of num holds up the denominator's operations (2D, 16384 blocks of
+          // 16^2 in double, density alone: 1.20 ms so, 1.12 with the bits, 1.10 with no
+          // test).  The evolved blast, 26 M cells, density and pressure, 3106 blocks of
+          // uniform density: 11.2 -> 6.4 ms
+          bool flat = true;
+          for (int d = 0; d < M.ndim; d++)
+            flat = flat && same_bits(q[t0 + stride[d]], r0) && same_bits(q[t0 - stride[d]], r0);
+          if (flat) continue;
           double num = 0.0, den = 0.0;
-          for (int d = 0; d < M.ndim; d++) {
-            const double rp = q[t0 + stride[d]], rm = q[t0 - stride[d]];
-            const double s2 = __dadd_rn(__dsub_rn(rp, 2.0 * r0), rm);
-            num = __dadd_rn(num, __dmul_rn(s2, s2));
-          }
-          // a flat quantity adds nothing: the quotient is 0 whatever the denominator, and
-          // the larger part of the work (50 of 62 operations) is left out.  The evolved
-          // blast, 26 M cells, density and pressure: 9.6 -> 5.0 ms for its 3106 blocks
-          // of uniform density
-          if (num == 0.0) continue;
-          for (int d = 0; d < M.ndim; d++) {
-            const double rp = q[t0 + stride[d]], rm = q[t0 - stride[d]];
-            const double a = __dadd_rn(fabs(__dsub_rn(rp, r0)), fabs(__dsub_rn(r0, rm)));
-            const double f = __dadd_rn(__dadd_rn(fabs(rp), 2.0 * fabs(r0)), fabs(rm));
-            const double dd = __dadd_rn(a, __dmul_rn(LOEHNER_EPS, f));
-            den = __dadd_rn(den, __dmul_rn(dd, dd));
-          }
+          for (int d = 0; d < M.ndim; d++)
+            est_terms(q[t0 + stride[d]], r0, q[t0 - stride[d]], num, den);
           const double r = den > 0.0 ? num / den : 0.0;
           e = __dadd_rn(e, __dmul_rn(ew.w[vars[c0 + cc]], sqrt(r)));
         }
@@ -739,7 +736,7 @@ int launch_estimate(amrvac_state* s, const T* U, const EstWeights& ew, double th
     // the cells and more tie (an exact checkerboard: 64 blocks of 64^2 210 and 251, 1024
     // of 16^3 1564 and 1825) or the values differ by less than the bounds tell apart
     // (the blast after 60 steps, 3106 such blocks among 6448 of 16^3: 11.2 and, with the
-    // tiled kernel's flat quantities left out, 7.1 ms).  Noise of an ulp is told apart:
+    // tiled kernel's flat quantities left out, 6.4 ms).  Noise of an ulp is told apart:
     // 1024 blocks of 16^3 1649 and 517; 2D, 64 blocks of 64^2, where one cell in 16 ties
     // for the maximum, 235 and 113 (328 with eight lanes a candidate for all of them).
     // 1128 blocks of 8^3 on three levels 177 and 198, 64 blocks of 16^3 on three 289 and
