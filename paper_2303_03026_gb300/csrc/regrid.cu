@@ -308,7 +308,6 @@ constexpr int EST_SCREEN_THREADS = 512;
 constexpr int EST_SCREEN_FEW = EST_SCREEN_THREADS / 4;
 // worth it from this many cells (see launch_estimate)
 constexpr size_t EST_SCREEN_CELLS = 2048;
-constexpr int EST_SLOTS = 2 * 152;
 
 // the quantities of a conserved cell as hi + lo (lo of the velocities and the
 // pressure only, the others are exact): v = m/rho with its remainder; the pressure
@@ -741,27 +740,28 @@ int launch_estimate(amrvac_state* s, const T* U, const EstWeights& ew, double th
     // for the maximum, 235 and 113 (328 with eight lanes a candidate for all of them).
     // 1128 blocks of 8^3 on three levels 177 and 198, 64 blocks of 16^3 on three 289 and
     // 111: across levels the block itself has to be large enough.
+    const bool fits = smem <= SMEM_MAX && cells + sizeof(double) * np <= SMEM_MAX;
+    int dev = 0, nsm = 0, per = 0;
+    if (fits &&
+        (cudaFuncSetAttribute(k_regrid_estimate_screen, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)smem) != cudaSuccess ||
+         cudaGetDevice(&dev) != cudaSuccess ||
+         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_regrid_estimate_screen,
+                                                       EST_SCREEN_THREADS, smem) != cudaSuccess ||
+         per < 1))
+      return -1;
     size_t chain = (size_t)M.ncell;
-    if (chain < EST_SCREEN_CELLS) {
+    if (fits && chain < EST_SCREEN_CELLS) {
       bool one = true;
       for (int b = 1; b < s->nblocks && one; b++) one = s->meta[5 * b + 1] == s->meta[1];
-      if (one) chain *= (size_t)((s->nblocks + EST_SLOTS - 1) / EST_SLOTS);
+      if (one) chain *= (size_t)((s->nblocks + nsm * per - 1) / (nsm * per));
     }
-    if (chain >= EST_SCREEN_CELLS && smem <= SMEM_MAX &&
-        cells + sizeof(double) * np <= SMEM_MAX) {
+    if (fits && chain >= EST_SCREEN_CELLS) {
       EstWeights sw = ew;
       double wmax = 0.0, wsum = 0.0;
       for (int v = 0; v < (ew.prim ? NV : 1); v++) wmax = fmax(wmax, ew.w[v]);
       for (int v = 0; v < (ew.prim ? NV : 1); v++) wsum += sw.wf[v] = (float)(ew.w[v] / wmax);
-      int dev = 0, nsm = 0, per = 0;
-      if (cudaFuncSetAttribute(k_regrid_estimate_screen,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-              cudaSuccess ||
-          cudaGetDevice(&dev) != cudaSuccess ||
-          cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_regrid_estimate_screen,
-                                                        EST_SCREEN_THREADS, smem) != cudaSuccess)
-        return -1;
       const int g = s->nblocks < nsm * per * 2 ? s->nblocks : nsm * per * 2;
       k_regrid_estimate_screen<<<g, EST_SCREEN_THREADS, smem, s->stream>>>(
           M, U, sw, EST_TOL * (float)wsum, thr, dthr, maxlev, s->d_est, s->d_eflags);
