@@ -21,7 +21,7 @@ size_t align_up(size_t x) { return (x + ALIGN - 1) / ALIGN * ALIGN; }
 
 struct Tables {
   std::vector<int> blk, nbr, gface, glist, gkind, rlist, lmap, lmap_off, lnb, istart, iblocks;
-  std::vector<double> gamma, dx;
+  std::vector<double> gamma, dx, idx;
   // device regrid plan: per instance the deepest level, and the offsets of the
   // dense new-leaf maps of levels 0 .. deepest + 1 ([ninst * MAXLEV + 1];
   // empty when a map that fine would be too large)
@@ -115,6 +115,7 @@ bool build_tables(const amrvac_config* c, int ninst, const amrvac_instance_desc*
   T.lmap_off.assign((size_t)ninst * MAXLEV, 0);
   T.lnb.assign((size_t)ninst * MAXLEV * 3, 1);
   T.dx.assign((size_t)ninst * MAXLEV * 3, 1.0);
+  T.idx.assign((size_t)ninst * MAXLEV * 3, 1.0);
   T.gamma.resize(ninst);
   size_t total = 0;
   for (int q = 0; q < ninst; q++) {
@@ -126,9 +127,11 @@ bool build_tables(const amrvac_config* c, int ninst, const amrvac_instance_desc*
         long n = d < c->ndim ? ((long)inst[q].base_blocks[d] << L) : 1;
         if (L <= maxlev[q] && n > (1 << 20)) return T.err = "mesh too fine", false;
         T.lnb[(q * MAXLEV + L) * 3 + d] = (int)std::min<long>(n, 1 << 30);
-        if (d < c->ndim)
-          T.dx[(q * MAXLEV + L) * 3 + d] =
-              (inst[q].xmax[d] - inst[q].xmin[d]) / ((double)n * c->block_nx[d]);
+        if (d < c->ndim) {
+          const double len = inst[q].xmax[d] - inst[q].xmin[d], cells = (double)n * c->block_nx[d];
+          T.dx[(q * MAXLEV + L) * 3 + d] = len / cells;
+          T.idx[(q * MAXLEV + L) * 3 + d] = cells / len;
+        }
         cnt *= (size_t)n;
       }
       T.lmap_off[q * MAXLEV + L] = (int)total;
@@ -155,10 +158,12 @@ bool build_tables(const amrvac_config* c, int ninst, const amrvac_instance_desc*
     if (!fits) T.pseg.clear();
   }
   // the wenozp5 lambda = dx^(2/3) of every (instance, level, dimension), kept
-  // after the cell sizes in the same table
+  // after the cell sizes in the same table, then the inverse cell sizes: rounded once,
+  // from the domain (1/dx of the rounded dx is rounded twice, for every cell alike)
   const size_t ndx = T.dx.size();
   T.dx.resize(2 * ndx);
   for (size_t i = 0; i < ndx; i++) T.dx[ndx + i] = std::pow(T.dx[i], 2.0 / 3.0);
+  T.dx.insert(T.dx.end(), T.idx.begin(), T.idx.end());
   T.lmap.assign(total, MAP_COARSER);
   auto pos = [&](int q, int L, long i, long j, long k) -> int& {
     const int* nb = &T.lnb[(q * MAXLEV + L) * 3];
@@ -523,6 +528,7 @@ amrvac_status amrvac_state_create(const amrvac_config* cfg, int32_t ninst,
   M.gamma = at<double>(s, L.gamma);
   M.dx = at<double>(s, L.dx);
   M.wzlam = M.dx + (size_t)ninst * MAXLEV * 3;
+  M.idx = M.wzlam + (size_t)ninst * MAXLEV * 3;
   M.inst_start = at<int>(s, L.istart);
   M.inst_blocks = at<int>(s, L.iblocks);
   M.rt = at<InstRT>(s, L.rt);

@@ -65,6 +65,7 @@ struct DevMesh {
   const double* gamma;    // [ninst]
   const double* dx;       // [ninst][MAXLEV][3] cell size
   const double* wzlam;    // [ninst][MAXLEV][3] dx^(2/3), the wenozp5 lambda
+  const double* idx;      // [ninst][MAXLEV][3] 1/dx, rounded once (cells over length)
   const int* inst_start;  // [ninst + 1] CSR of blocks per instance
   const int* inst_blocks; // [nblocks]
   InstRT* rt;             // [ninst]

@@ -40,11 +40,11 @@ double* g_partials_addr[kMaxDevices] = {nullptr};
 // per-block maxima of sum_d (|v_d| + c_f,d)/dx_d and of |v_d| + c_f,d
 template <class T>
 __global__ void __launch_bounds__(256) k_cfl_partials_static(DevMesh M, const T* __restrict__ U,
-                                                             double gamma, double dx0,
-                                                             double dx1, double dx2, int ff,
+                                                             double gamma, double idx0,
+                                                             double idx1, double idx2, int ff,
                                                              double* __restrict__ partials) {
   const size_t vs = (size_t)M.nblocks * M.ncell;
-  const T idx[3] = {(T)(1.0 / dx0), (T)(1.0 / dx1), (T)(1.0 / dx2)};
+  const T idx[3] = {(T)idx0, (T)idx1, (T)idx2};
   for (int b = blockIdx.x; b < M.nblocks; b += gridDim.x) {
     T smx = T(0), cmx = T(0);
     for (int c = threadIdx.x; c < M.ncell; c += blockDim.x) {
@@ -122,7 +122,7 @@ extern "C" amrvac_status amrvac_cfl_dt_noalloc(const amrvac_config* cfg,
   long long blocks = 1, cells = 1;  // 64-bit products: 4096^3 overflows an int
   DevMesh M{};
   M.ndim = cfg->ndim;
-  double dx[3] = {1.0, 1.0, 1.0};
+  double idx[3] = {1.0, 1.0, 1.0};
   for (int d = 0; d < 3; d++) {
     const bool act = d < cfg->ndim;
     M.nx[d] = act ? cfg->block_nx[d] : 1;
@@ -132,7 +132,7 @@ extern "C" amrvac_status amrvac_cfl_dt_noalloc(const amrvac_config* cfg,
       if (!(inst->xmax[d] > inst->xmin[d])) return AMRVAC_E_INVALID;
       blocks *= inst->base_blocks[d];
       cells *= cfg->block_nx[d];
-      dx[d] = (inst->xmax[d] - inst->xmin[d]) / ((double)inst->base_blocks[d] * cfg->block_nx[d]);
+      idx[d] = (double)inst->base_blocks[d] * cfg->block_nx[d] / (inst->xmax[d] - inst->xmin[d]);
     }
   }
   if (blocks != nblocks) return AMRVAC_E_INVALID;  // one uniform level-0 instance only
@@ -148,11 +148,11 @@ extern "C" amrvac_status amrvac_cfl_dt_noalloc(const amrvac_config* cfg,
   // float-float pressure recovery for FP32-bulk states configured with it
   const int ff = cfg->precision == AMRVAC_FP32_BULK && cfg->pressure == AMRVAC_PRESSURE_FF;
   if (cfg->precision == AMRVAC_FP64)
-    k_cfl_partials_static<double><<<grid, 256, 0, s>>>(M, (const double*)d_U, inst->gamma, dx[0],
-                                                       dx[1], dx[2], 0, partials);
+    k_cfl_partials_static<double><<<grid, 256, 0, s>>>(M, (const double*)d_U, inst->gamma, idx[0],
+                                                       idx[1], idx[2], 0, partials);
   else
-    k_cfl_partials_static<float><<<grid, 256, 0, s>>>(M, (const float*)d_U, inst->gamma, dx[0],
-                                                      dx[1], dx[2], ff, partials);
+    k_cfl_partials_static<float><<<grid, 256, 0, s>>>(M, (const float*)d_U, inst->gamma, idx[0],
+                                                      idx[1], idx[2], ff, partials);
   k_cfl_finish_static<<<1, 256, 0, s>>>(partials, nblocks, cfg->courant, t, inst->t_end, d_out);
   return cudaPeekAtLastError() == cudaSuccess ? AMRVAC_OK : AMRVAC_E_CUDA;
 }

@@ -214,8 +214,7 @@ __global__ void __launch_bounds__(256) k_update(DevMesh M, const T* U0,
 
 // CFL maxima of every block of U, a CTA per chunk of `chunk` cells of a block
 // (one chunk a block: stored; else merged into part, zeroed before).  Only the two
-// maxima are reduced, and 1/dx and the terms shared by the directions are formed
-// once.
+// maxima are reduced, and the terms shared by the directions are formed once.
 template <class T>
 __global__ void __launch_bounds__(256) k_cfl(DevMesh M, const T* __restrict__ U, int ff,
                                              int nchunk, int chunk) {
@@ -224,8 +223,8 @@ __global__ void __launch_bounds__(256) k_cfl(DevMesh M, const T* __restrict__ U,
   for (size_t item = blockIdx.x; item < nitem; item += gridDim.x) {
     const int b = (int)(item / nchunk), c0 = (int)(item - (size_t)b * nchunk) * chunk;
     const int q = M.blk[b * 5], L = M.blk[b * 5 + 1];
-    const double* dx = M.dx + (q * MAXLEV + L) * 3;
-    const T idx[3] = {(T)(1.0 / dx[0]), (T)(1.0 / dx[1]), (T)(1.0 / dx[2])};
+    const double* id = M.idx + (q * MAXLEV + L) * 3;
+    const T idx[3] = {(T)id[0], (T)id[1], (T)id[2]};
     const double gamma = M.gamma[q];
     T smx = T(0), cmx = T(0);
     const int c1 = c0 + chunk < M.ncell ? c0 + chunk : M.ncell;
@@ -466,7 +465,7 @@ __global__ void k_level_consts(DevMesh M, double glm_alpha, int glm, int k0, Sta
   for (int e = 0; e < 3; e++) {
     d[LC_DX + e] = dx[e];
     f[LC_DX + e] = (float)dx[e];
-    d[LC_IDX + e] = 1.0 / dx[e];
+    d[LC_IDX + e] = M.idx[(q * MAXLEV + L) * 3 + e];
     f[LC_IDX + e] = 1.0f / (float)dx[e];
   }
   d[LC_SKIP] = rt.dt == 0.0 ? 1.0 : 0.0;
