@@ -640,9 +640,12 @@ def main():
                 "traffic": tr * cells / 3.0 if tr is not None else None,
                 "traffic_unit": "DRAM bytes per stage launch (ncu, mean of the 3 stages)",
                 "peak_source": src,
-                "kernel": ("k_fused%s (one persistent launch per SSPRK stage, after the "
+                "kernel": ("k_fused%s%s (one persistent launch per SSPRK stage, after the "
                            "k_ghost_slabs pre-pass where the mesh has level-change faces; "
-                           "stage_ms covers both)" % ("" if W.cfg.ndim == 3 else "2d"))
+                           "stage_ms covers both)"
+                           % ("" if W.cfg.ndim == 3 else "2d",
+                              "" if W.cfg.limiter in ("mp5", "weno5", "wenoz5", "wenozp5")
+                              else "_f2"))
                 if fused else "plain per-block kernels (prim + flux x ndim + update) per stage",
                 "issue_ceiling": issue,
                 "stage_ms": [float(x) for x in stage_ms],
