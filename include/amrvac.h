@@ -67,7 +67,7 @@ typedef enum {
   AMRVAC_E_CUDA = 3,         /* a CUDA runtime call failed                    */
   AMRVAC_E_SMALL_VALUES = 4, /* density or pressure at or below its floor (Sect. 7.4:
                                 check_small_values stops and reports)         */
-  AMRVAC_E_TIMEOUT = 5,      /* reserved: a bounded device wait gave up       */
+  AMRVAC_E_TIMEOUT = 5,      /* a bounded wait of a stage kernel gave up      */
   AMRVAC_E_STATE = 6         /* call out of order, or a mesh lookup failed    */
 } amrvac_status;
 

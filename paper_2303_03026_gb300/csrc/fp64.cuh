@@ -25,7 +25,9 @@ __device__ __forceinline__ unsigned long long bits64(double x) {
 }
 
 // biased exponent 1 .. 2045: zero, subnormal, 2^1023 and above, infinities and
-// NaN (whose approximation is 0 or infinite) are left to the caller's fallback
+// NaN (whose approximation is 0 or infinite) are left to the caller's fallback.
+// (A reciprocal that would be subnormal, of 2^1022 and above, is 0, and that of a
+// subnormal number infinite.)
 __device__ __forceinline__ bool mid_range(double x) {
   const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
   return e - 1u < 2045u;

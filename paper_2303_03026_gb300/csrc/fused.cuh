@@ -2,9 +2,10 @@
 // fused2d.cuh) blocks: double, and FP32 with the five-point limiters (FP32 with
 // two ghost layers: fused_f2.cuh).
 //
-// One CTA of 272 threads owns one block at a time and loops over the work
-// list (grid = resident CTAs).  Thread (x, y) < 256 owns a column of the block;
-// 16 helper threads take the 32 faces on the +x/+y block boundary.
+// One CTA of 272 threads (double with two ghost layers: 288) owns one block at a
+// time and loops over the work list (grid = resident CTAs).  Thread (x, y) < 256
+// owns a column of the block; 16 helper threads (a warp of 32) take the 32 faces
+// on the +x/+y block boundary.
 //   3D: march over z with a ring of 2G primitive planes in shared memory,
 //       each with its G-cell x/y halo (G = 2 ghost layers: 4 planes of 20 x
 //       20, 128 halo cells a plane; G = 3 for the five-point limiters: 6
@@ -15,12 +16,13 @@
 //           level-change face (built before the launch by k_ghost_slabs);
 //           for stages k > 0 also U0 of the owner's cell of plane z;
 //         x- and y-face fluxes of plane z into shared memory (double-buffered
-//           by plane parity);
+//           by plane parity; double with two ghost layers: slopes, a barrier,
+//           fluxes, see shared_slope_xy);
 //         wait for the copies, conserved -> primitive in place of the own
 //           cells of plane z+G and (owners 256-64G .. 255, one cell each) of
 //           the halo of plane z+1 (float-float or fp64 pressure for FP32 bulk);
 //         the z-face z+1/2 flux of the thread's own column (registers);
-//         one barrier; update of cell (x, y, z): flux divergence with the
+//         barrier; update of cell (x, y, z): flux divergence with the
 //           z-face flux carried from the previous plane, psi damping, SSPRK
 //           combination; in the last stage the CFL terms of the new state
 //           (reduced per block for the time step).
@@ -38,12 +40,13 @@
 namespace amrvac {
 
 constexpr int FB = 16;          // block edge handled by the fused kernel
-// threads per CTA: 256 column owners (x- and y-face of their cell, z-face of
-// their column, their cell's update; with two ghost layers owners 0..127 also
-// copy in and owners 128..255 convert one of the 128 x/y halo cells of each
-// plane, with three owners 0..191 and 64..255 share the 192) and 16 helpers
-// (the 32 faces on the +x/+y block boundary).  The 2D kernel uses the same
-// roles with threads 0 .. 64G-1 copying and converting the halo.
+// threads per CTA where each face is evaluated from its own stencil: 256 column
+// owners (x- and y-face of their cell, z-face of their column, their cell's
+// update; with two ghost layers owners 0..127 also copy in and owners 128..255
+// convert one of the 128 x/y halo cells of each plane, with three owners 0..191
+// and 64..255 share the 192) and 16 helpers (the 32 faces on the +x/+y block
+// boundary).  The 2D kernel uses the same roles with threads 0 .. 64G-1 copying
+// and converting the halo.
 constexpr int FT = FB * FB + FB;
 // limiter template values: a limiter, or in double -2 = the five-point ones at run
 // time (-1, -3: see fused.cu); ghost layers of the tile
@@ -58,7 +61,7 @@ __host__ __device__ constexpr int tile_ghosts(int lim) { return five_tile(lim) ?
 // row r, lane 16 + r the y faces of column r, one flux evaluation for both.
 // With the refined approximations of fp64.cuh for division and square root: a
 // step of the 3D AMR blast in double (6.0 M cells) 85.6 -> 42.0 ms, of the 1024^2
-// vortex with koren 10.3 -> 5.3 ms. 
+// vortex with koren 10.3 -> 5.3 ms.
 template <class T, int LIM> constexpr bool share_slopes() {
   return sizeof(T) == 8 && tile_ghosts(LIM) == NG;
 }
@@ -66,7 +69,6 @@ template <class T, int LIM> constexpr int fused_threads() {
   return share_slopes<T, LIM>() ? FB * FB + 2 * FB : FT;
 }
 constexpr int FXW = 20;           // row stride of the face-flux arrays
-
 
 // Thread (x, y) of a warp: lanes 0-15 take row r, lanes 16-31 row r + 4, so the
 // two half-warps of a row-stride-20 array fall on disjoint banks (4*20 = 16 mod 32;
@@ -77,12 +79,12 @@ __device__ __forceinline__ int fused_row(int warp, int lane) {
 
 // G: ghost layers; a plane is (16 + 2G)^2 (row stride 20 or 22) and the ring
 // holds the 2G planes of a z stencil
-template <class T, int DIM, int G = NG> struct FusedSmem {
+template <class T, int G = NG> struct FusedSmem {
   static constexpr int PW = FB + 2 * G;
-  static constexpr int NSLOT = DIM == 3 ? 2 * G : 1;
+  static constexpr int NSLOT = 2 * G;
   T plane[NSLOT][NV][PW][PW];
   // face fluxes of the current plane, double-buffered by plane parity so that
-  // one barrier per plane separates writers and readers
+  // the barrier before the update separates writers and readers
   T fx[2][NV][FB][FXW];       // x faces: column i = face i - 1/2, i = 0..16
   T fy[2][NV][FB + 1][FXW];   // y faces: row j = face j - 1/2
   // float path: U0 of the owners' cells of the current plane, copied in ahead
@@ -399,18 +401,16 @@ __global__ void __launch_bounds__(256)
 // the lean instantiation runs otherwise)
 // Five-point limiters: three ghost layers (a 6-plane ring of 22 x 22 planes and
 // 192 halo cells a plane, one CTA per SM)
-template <class T, int DIM, int LIM, int FLUX, bool FULL>
+template <class T, int LIM, int FLUX, bool FULL>
 __global__ void __launch_bounds__(fused_threads<T, LIM>(), 1)
     k_fused(DevMesh M, const T* U0, const T* __restrict__ Uk, const T* U2, T* out, T* out2,
             const int* __restrict__ work, int nwork, const T* __restrict__ gslab,
             int* __restrict__ counter, StageParams sp) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  static_assert(DIM == 3, "16x16 blocks in 2D use k_fused2d");
   static_assert(sizeof(T) == 8 || five_tile(LIM), "FP32 with two ghost layers: k_fused_f2");
   constexpr int G = tile_ghosts(LIM);
-  using Smem = FusedSmem<T, DIM, G>;
+  using Smem = FusedSmem<T, G>;
   Smem& S = *reinterpret_cast<Smem*>(smraw);
-  constexpr int NZ = DIM == 3 ? FB : 1;
   constexpr int NSLOT = Smem::NSLOT;
   constexpr int PW = Smem::PW;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -418,8 +418,7 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), 1)
   const size_t vs = (size_t)M.nblocks * M.ncell;
   const int ncell = M.ncell;
   const bool ff = sp.pressure_ff != 0;
-  constexpr int NT2 = DIM == 3 ? FB : 1;          // second tangential extent of a face
-  constexpr int SLAB_FACE = NV * G * FB * NT2;    // one face: [v][layer][t2][t1]
+  constexpr int SLAB_FACE = NV * G * FB * FB;  // one face: [v][layer][t2][t1]
   constexpr bool SHARE = share_slopes<T, LIM>();
 
   const bool owner = tid < FB * FB;
@@ -472,7 +471,7 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), 1)
           out[at] = u[v];
           if (FULL && sp.has2) out2[at] = u[v];
         }
-        if (sp.epilogue) cfl_terms<T, DIM>(u, gammad, g, ff, gm1f, idd, smx, cmx);
+        if (sp.epilogue) cfl_terms<T, 3>(u, gammad, g, ff, gm1f, idd, smx, cmx);
       }
       if (sp.epilogue) cta_reduce_max2(S.red, smx, cmx, owner, M.part + (size_t)b * NPART);
       continue;
@@ -492,7 +491,7 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), 1)
     int wmask = 0;
 #pragma unroll
     for (int f = 0; f < 6; f++) {
-      nb[f] = f < 2 * DIM ? M.nbr[b * 6 + f] : NBR_OUTFLOW;
+      nb[f] = M.nbr[b * 6 + f];
       if (FULL && nb[f] == NBR_WALL) {  // before slab codes, which reach -5 too
         nb[f] = NBR_OUTFLOW;
         wmask |= 1 << f;
@@ -507,7 +506,7 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), 1)
       int f = -1, n = 0, t1 = 0, t2 = 0;
       if (i < 0 || i >= FB) { f = i < 0 ? 0 : 1; n = i; t1 = j; t2 = k; }
       else if (j < 0 || j >= FB) { f = j < 0 ? 2 : 3; n = j; t1 = i; t2 = k; }
-      else if (DIM == 3 && (k < 0 || k >= FB)) { f = k < 0 ? 4 : 5; n = k; t1 = i; t2 = j; }
+      else if (k < 0 || k >= FB) { f = k < 0 ? 4 : 5; n = k; t1 = i; t2 = j; }
       vstride = vs;
       if (f < 0) {
         ptr = Uk + (size_t)b * ncell + (k * FB + j) * FB + i;
@@ -516,8 +515,8 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), 1)
       const int code = nb[f];
       if (code <= -3) {
         const int layer = n < 0 ? n + G : n - FB;
-        ptr = gslab + (size_t)(-3 - code) * SLAB_FACE + (layer * NT2 + t2) * FB + t1;
-        vstride = G * NT2 * FB;
+        ptr = gslab + (size_t)(-3 - code) * SLAB_FACE + (layer * FB + t2) * FB + t1;
+        vstride = G * FB * FB;
         return;
       }
       int nn = code >= 0 ? (n < 0 ? n + FB : n - FB) : (n < 0 ? 0 : FB - 1);
@@ -555,7 +554,7 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), 1)
 #pragma unroll
         for (int v = 0; v < NV; v++)
           cp_async_elem(&S.plane[slot][v][y + G][x + G], ptr + v * st);
-        if (tid < NH && pz >= 0 && pz < NZ) {
+        if (tid < NH && pz >= 0 && pz < FB) {
           int hx, hy;
           halo_xy(tid, hx, hy);
           locate(hx, hy, pz, ptr, st);
@@ -570,7 +569,7 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), 1)
     // conversion of its own cell ...
     auto convert_plane = [&](int pz) {
       const int slot = ((pz % NSLOT) + NSLOT) % NSLOT;
-      const int flip = FULL && ((pz < 0 && (wmask & 16)) || (pz >= NZ && (wmask & 32))) ? 4 : 0;
+      const int flip = FULL && ((pz < 0 && (wmask & 16)) || (pz >= FB && (wmask & 32))) ? 4 : 0;
       if (owner) to_prim(&S.plane[slot][0][y + G][x + G], 0, flip);
     };
     // ... and, one barrier after their copies landed, the conversion of the
@@ -653,17 +652,18 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), 1)
     convert_halo(0);
     __syncthreads();  // plane 0 with its halo in primitives
 
-    // One barrier per plane.  Iteration z: issue the copies of U0 of plane z
-    // (stages k > 0) and of plane z+G into the slot of plane z-G (its last
-    // readers were the faces of plane z-G and this thread's own z face of
-    // iteration z-1); x/y faces of plane z into the flux buffer of parity z;
-    // wait for and convert the own cells of plane z+G, convert the halo of
-    // plane z+1 (owners 256-NH..255); load U_k of the own cell of plane z; z
-    // face z+1/2 (planes z+1-G .. z+G); barrier; update of plane z.  The buffer of parity z is rewritten at
-    // iteration z+2, after the barrier of iteration z+1, which every thread
-    // passes only after its update of plane z.
+    // Iteration z: issue the copies of U0 of plane z (float, stages k > 0) and
+    // of plane z+G into the slot of plane z-G (its last readers were the faces
+    // of plane z-G and this thread's own z face of iteration z-1); x/y faces of
+    // plane z into the flux buffer of parity z (SHARE: its slopes first, with a
+    // barrier between); wait for and convert the own cells of plane z+G, convert
+    // the halo of plane z+1 (owners 256-NH..255); float: load U_k of the own
+    // cell of plane z; z face z+1/2 (planes z+1-G .. z+G); barrier; update of
+    // plane z.  The buffer of parity z is rewritten at iteration z+2, after the
+    // last barrier of iteration z+1, which every thread passes only after its
+    // update of plane z.
 #pragma unroll 1
-    for (int z = 0; z < NZ; z++) {
+    for (int z = 0; z < FB; z++) {
       if (pre0) issue_u0(z);
       issue_plane(z + G);  // commits this thread's copies as one group
       const int sl = z % NSLOT, fb = z & 1;
@@ -703,7 +703,7 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), 1)
       // iteration)
       cp_async_wait_all();
       convert_plane(z + G);
-      if (z + 1 < NZ) convert_halo(z + 1);
+      if (z + 1 < FB) convert_halo(z + 1);
       // float path: the stage input of the own cell, loaded before the z face
       // and the barrier so that its L2 latency overlaps them (the double path
       // has no registers to spare and loads it in the update)
@@ -714,8 +714,8 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), 1)
         for (int v = 0; v < NV; v++) ukr[v] = Uk[(size_t)v * vs + (size_t)b * ncell + c];
       }
       T fz[NV];
-      if (DIM == 3 && owner) zflux(z + 1, fz);
-      if (FULL && sp.reflux && owner && z == NZ - 1 && nb[5] <= -3)
+      if (owner) zflux(z + 1, fz);
+      if (FULL && sp.reflux && owner && z == FB - 1 && nb[5] <= -3)
         keep_face_flux(M, nb[5], y * FB + x, fz);
       __syncthreads();
       if (!owner) continue;  // helpers: no cell of their own
@@ -725,7 +725,7 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), 1)
       for (int v = 0; v < NV; v++) {
         T acc = (S.fx[fb][v][y][x + 1] - S.fx[fb][v][y][x]) * idx0;
         acc += (S.fy[fb][v][y + 1][x] - S.fy[fb][v][y][x]) * idx1;
-        if (DIM == 3) acc += (fz[v] - fzp[v]) * idx2;
+        acc += (fz[v] - fzp[v]) * idx2;
         const size_t at = (size_t)v * vs + (size_t)b * ncell + c;
         const T uk = PRE0 ? ukr[PRE0 ? v : 0] : Uk[at];
         T ut = uk - dt * acc;
@@ -742,11 +742,9 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), 1)
         }
         out[at] = un[v];
       }
-      if (sp.epilogue) cfl_terms<T, DIM>(un, gammad, g, ff, gm1f, idd, smx, cmx);
-      if (DIM == 3) {
+      if (sp.epilogue) cfl_terms<T, 3>(un, gammad, g, ff, gm1f, idd, smx, cmx);
 #pragma unroll
-        for (int v = 0; v < NV; v++) fzp[v] = fz[v];
-      }
+      for (int v = 0; v < NV; v++) fzp[v] = fz[v];
     }
     if (sp.epilogue) cta_reduce_max2(S.red, smx, cmx, owner, M.part + (size_t)b * NPART);
   }
@@ -769,13 +767,13 @@ template <class T, int DIM, int LIM, int FLUX, bool FULL> struct FusedKernel {
   static constexpr auto kernel() {
     if constexpr (F2 && DIM == 3) return &k_fused_f2<LIM, FLUX, FULL>;
     else if constexpr (F2) return &k_fused2d_f2<LIM, FLUX, FULL>;
-    else if constexpr (DIM == 3) return &k_fused<T, 3, LIM, FLUX, FULL>;
+    else if constexpr (DIM == 3) return &k_fused<T, LIM, FLUX, FULL>;
     else return &k_fused2d<T, LIM, FLUX, FULL>;
   }
   static constexpr int smem() {
     if constexpr (F2 && DIM == 3) return (int)sizeof(FusedF2Smem);
     else if constexpr (F2) return (int)sizeof(Fused2dF2Smem);
-    else if constexpr (DIM == 3) return (int)sizeof(FusedSmem<T, 3, tile_ghosts(LIM)>);
+    else if constexpr (DIM == 3) return (int)sizeof(FusedSmem<T, tile_ghosts(LIM)>);
     else return (int)sizeof(Fused2dSmem<T, tile_ghosts(LIM)>);
   }
 };

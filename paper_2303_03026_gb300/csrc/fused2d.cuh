@@ -9,12 +9,14 @@
 //   wait for this thread's copies of the current block (slot s);
 //   conserved -> primitive: owners their cell, threads 0 .. 64G-1 one halo
 //   cell (G = 2, or 3 for the five-point limiters with a 22 x 22 tile);
-//   barrier; x and y faces (owners the low faces of their cell, the 16 helper
-//   threads the +x / +y block-boundary faces);
+//   barrier; x and y faces: owners the low faces of their cell, the helpers the
+//   +x / +y block-boundary faces (double with two ghost layers: slopes once a
+//   cell, a barrier, fluxes, the helpers a whole warp, see shared_slope_xy; the
+//   five-point limiters: each face from its stencil, 16 helpers);
 //   barrier; update of the owner's cell from the conserved values in slot s.
 // Each thread reads back only the slot entries it copied itself, so a slot can
 // be refilled without a barrier once the thread has used it.  Arithmetic is
-// that of the 3D kernel (stencil_flux, cfl_terms, cons2prim).
+// that of the 3D kernel.
 #pragma once
 
 namespace amrvac {
@@ -116,7 +118,7 @@ __global__ void __launch_bounds__(fused_threads<T, LIM>(), sizeof(T) == 4 ? 2 : 
   };
 
   // work items: static (i, i + grid, ...) or drawn from the counter; the
-  // item after next is fetched by thread 0 between the two barriers of a block
+  // item after next is fetched by thread 0 between two barriers of a block
   int wi, wn;
   if (counter) {
     if (tid == 0) {

@@ -27,19 +27,18 @@
 //
 // 3D: one CTA of 256 threads (a column each) per block, two CTAs an SM, marching
 // over z with a ring of four primitive planes with their two-cell x/y halo.
-// Iteration z, with planes z and z+1 converted, plane z+2 copied and the x and y
-// slopes of plane z done:
+// Iteration z, with planes z and z+1 converted and the copies of plane z+2 issued:
+//   x and y slopes of plane z, states handed over;
 //   arrive 1; convert plane z+2 (own cell; threads 0 .. 127 one halo cell) in
 //   place; issue the copies of U0 of plane z and of plane z+3; wait 1;
 //   x and y fluxes of plane z into the flux arrays;
-//   arrive 2; z slopes of cell z+1, flux of face z+1/2 (own column); x and y
-//   slopes of plane z+1, states handed over; wait 2;
+//   arrive 2; z slopes of cell z+1, flux of face z+1/2 (own column); wait 2;
 //   update of plane z.
 // The two barriers are split (mbarriers, one arrival per warp), so that a warp
 // works on its own column while the others catch up: the warps of the block
 // boundary have up to 250 instructions more in a plane.  The flux arrays are
 // double-buffered by plane parity: the states of plane z+1 are handed over after
-// wait 1 of plane z, i.e. once every warp has updated plane z-1.  After wait 2
+// both waits of plane z, i.e. once every warp has updated plane z-1.  After wait 2
 // every warp is done with the neighbours in plane z, whose ring slot is refilled
 // in the next iteration.
 #pragma once

@@ -23,8 +23,8 @@ static inline int grid_for(size_t work, int threads) {
 }
 
 // Threads per CTA of the passes over cells and faces: one SM evaluates 2 double
-// lanes a clock, so a small mesh is spread over the SMs in CTAs of one to four
-// warps (a 512-cell shock tube's face pass: 33 us in 3 CTAs of 256, the work of a
+// lanes a clock, so a small mesh is spread over the SMs in CTAs of one warp up to
+// eight (a 512-cell shock tube's face pass: 33 us in 3 CTAs of 256, the work of a
 // face being some 400 double operations), a large one takes 256.
 static inline int threads_for(size_t work) {
   int t = 32;

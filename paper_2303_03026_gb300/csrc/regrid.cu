@@ -725,21 +725,20 @@ int launch_estimate(amrvac_state* s, const T* U, const EstWeights& ew, double th
     int nt = nw;
     for (int v = 1; v < 5; v++) nt += ew.prim && ew.w[v] != 0.0;
     const size_t smem = sizeof(float) * (np * (size_t)nt + (size_t)M.ncell) + np;
-    // It saves double arithmetic, which is in proportion to the cells that one CTA
-    // works off, and costs a second launch and a longer chain of latencies where levels
-    // meet.  For density and pressure, both ways in us: 2D 16^2, 1024 blocks 150 and 110,
-    // 16384 blocks 1633 and 849; 3D 8^3, 1024 blocks 275 and 129; 16^3, 16 blocks 248
-    // and 89, 1024 blocks 1493 and 266; but 288 blocks of 8^3 on three levels 89 and
-    // 141, 43 blocks of 8^2 64 and 80, 1024 blocks of 128 cells in 1D 102 and 105.
-    // Blocks with more candidates than the screening takes are worked twice: where half
-    // the cells and more tie (an exact checkerboard: 64 blocks of 64^2 210 and 251, 1024
-    // of 16^3 1564 and 1825) or the values differ by less than the bounds tell apart
-    // (the blast after 60 steps, 3106 such blocks among 6448 of 16^3: 11.2 and, with the
-    // tiled kernel's flat quantities left out, 6.4 ms).  Noise of an ulp is told apart:
-    // 1024 blocks of 16^3 1649 and 517; 2D, 64 blocks of 64^2, where one cell in 16 ties
-    // for the maximum, 235 and 113 (328 with eight lanes a candidate for all of them).
-    // 1128 blocks of 8^3 on three levels 177 and 198, 64 blocks of 16^3 on three 289 and
-    // 111: across levels the block itself has to be large enough.
+    // It saves double arithmetic, which is in proportion to the cells that one CTA works
+    // off, and costs a second launch and a longer chain of latencies where levels meet:
+    // taken from 2048 cells of a block, and where all blocks are of one level from 2048
+    // cells a CTA slot.  In double and screened, us, density and pressure:
+    //   one level   16^3  16 blocks 248, 89; 1024 1493, 290     8^3  4096 952, 364
+    //               16^2  16384 blocks 1633, 981     64^2  64 blocks 201, 87
+    //   three       16^3  64 blocks 289, 111     8^3  288 blocks 89, 141; 1128 177, 198
+    //   below       8^2  43 blocks 64, 80     128 cells  1024 blocks 102, 105
+    // Blocks with more candidates than the screening takes are worked twice: half the
+    // cells and more tie (an exact checkerboard: 64 blocks of 64^2 210, 251) or differ by
+    // less than the bounds tell apart (the blast after 60 steps, 3106 such blocks among
+    // 6448: 11.2, 6.4 ms with the tiled kernel's flat quantities left out).  Noise of an
+    // ulp is told apart (1024 blocks of 16^3 1649, 517), also where one cell in 16 ties
+    // (64 blocks of 64^2 235, 113).
     const bool fits = smem <= SMEM_MAX && cells + sizeof(double) * np <= SMEM_MAX;
     int dev = 0, nsm = 0, per = 0;
     if (fits &&
