@@ -734,7 +734,7 @@ int launch_estimate(amrvac_state* s, const T* U, const EstWeights& ew, double th
     //   three       16^3  64 blocks 289, 111     8^3  288 blocks 89, 141; 1128 177, 198
     //   below       8^2  43 blocks 64, 80     128 cells  1024 blocks 102, 105
     // Blocks with more candidates than the screening takes are worked twice: half the
-    // cells and more tie (an exact checkerboard: 64 blocks of 64^2 210, 251) or differ by
+    // cells and more tie (two values in exact turn: 64 blocks of 64^2 210, 251) or differ by
     // less than the bounds tell apart (the blast after 60 steps, 3106 such blocks among
     // 6448: 11.2, 6.4 ms with the tiled kernel's flat quantities left out).  Noise of an
     // ulp is told apart (1024 blocks of 16^3 1649, 517), also where one cell in 16 ties
